@@ -46,6 +46,7 @@ struct BInst {
 };
 
 struct BGroup {
+  bool pair;  // CTA pairs (units with pair_rows) run this group
   std::vector<int> members;
   std::vector<std::vector<xe::XUnit>> units;  // per member
   xe::StageLayout L;
@@ -130,6 +131,7 @@ float time_cover(const std::vector<xe::XUnit> &units, int n_in, int C, int T, in
   p.pk_stages = L.pk_stages;
   p.z_stage_bytes = L.z_stage_bytes;
   p.pk_stage_bytes = L.pk_stage_bytes;
+  p.sum_rows = L.sum_rows;
   for (int rep = 0; rep < 6; ++rep) {
     if (cudaEventRecord(e0, st) != cudaSuccess ||
         xe::launch_cmac(maps, p, grid, L.smem_bytes, st) != cudaSuccess ||
@@ -261,7 +263,13 @@ int upload_group(corr_batch *b, BGroup &g) {
   }
   std::vector<xe::XItem> items;
   std::vector<int> first;
-  g.grid = xe::build_items(work, b->n_sm, items, first);
+  g.pair = g.units[0][0].pair_rows != 0;
+  int workers = b->n_sm;
+  if (g.pair) {
+    workers = std::min(b->n_sm / 2, xe::cmac_pair_clusters_batch(g.L.smem_bytes));
+    if (workers < 1) return CORR_ECUDA;
+  }
+  g.grid = xe::build_items(work, workers, items, first);
   int rc;
   if ((rc = cuda_err(cudaMalloc(&g.d_units, all.size() * sizeof(xe::XUnit)))) != CORR_OK ||
       (rc = cuda_err(cudaMalloc(&g.d_probs, g.members.size() * sizeof(xe::XProb)))) != CORR_OK ||
@@ -383,13 +391,16 @@ int corr_batch_create(int n_inst, const int *n_ant, const int *n_pol, const int 
   std::vector<std::vector<xe::XUnit>> units(n_inst);
   std::map<std::pair<uint32_t, uint32_t>, std::vector<int>> by_layout;
   for (int k = 0; k < n_inst; ++k) {
-    units[k] = xe::build_schedule(b->inst[k].n_in, b->inst[k].cover);
+    // above 256 inputs the pairs cover runs in its CTA-pair form
+    units[k] = xe::build_schedule(b->inst[k].n_in,
+                                  b->inst[k].n_in > 256 ? xe::kCoverQuads : b->inst[k].cover);
     xe::StageLayout L;
     if (units[k].empty() || !xe::stage_layout({&units[k]}, optin, xe::kMaxZStages, &L)) {
       free_batch(b);
       return CORR_EINVAL;
     }
-    by_layout[{L.z_stage_bytes, L.pk_stage_bytes}].push_back(k);
+    const uint32_t pair_bit = units[k][0].pair_rows ? 1u : 0u;  // stage sizes are multiples of 1024
+    by_layout[{L.z_stage_bytes | pair_bit, L.pk_stage_bytes}].push_back(k);
   }
   for (auto &kv : by_layout) {
     const std::vector<int> &ks = kv.second;
@@ -492,8 +503,11 @@ int corr_batch_push(corr_batch *b, const uint8_t *const *d_blocks, void *stream)
     p.pk_stages = g.L.pk_stages;
     p.z_stage_bytes = g.L.z_stage_bytes;
     p.pk_stage_bytes = g.L.pk_stage_bytes;
+    p.sum_rows = g.L.sum_rows;
     if (g.grid > 0) {
-      if ((rc = cuda_err(xe::launch_cmac_batch(maps, p, g.grid, g.L.smem_bytes, st))) != CORR_OK)
+      if ((rc = cuda_err(g.pair ? xe::launch_cmac_batch_pair(maps, p, g.grid, g.L.smem_bytes, st)
+                                : xe::launch_cmac_batch(maps, p, g.grid, g.L.smem_bytes, st))) !=
+          CORR_OK)
         return rc;
       b->launches++;
     }

@@ -41,6 +41,7 @@ struct corr_ctx {
   ItemPlan plans[xe::kMaxBlocksPerLaunch + 1];
   int smem_bytes, z_stages, pk_stages;
   uint32_t z_stage_bytes, pk_stage_bytes;
+  int sum_rows;
   int tm;  // 1: the TMEM-operand kernel (xengine_tm.cu) runs this context's launches
   int pair;  // 1: CTA pairs (the quad cover, M = 256 MMAs) run this context's launches
   int ch_rows;  // inputs per channel in the TMA box (64, or 16 / 32 for multi-channel tiles)
@@ -117,15 +118,15 @@ bool use_tm_kernel(int n_in) {
   return e && std::strcmp(e, "tm") == 0;
 }
 
-// Whether CTA pairs run a context of n_in inputs (more than 256 only).  The
-// pair's shared B operand halves the inputs each SM unpacks per MMA, but on
-// this part the pair kernel measured 5 % slower per issued MAC than one-CTA
-// units at 512 to 2048 inputs, and its cover issues more padding on the
-// diagonal: it runs only when CORR_CMAC_KERNEL=pair asks for it.
+// Whether CTA pairs run a context of n_in inputs: above 256 inputs, unless
+// CORR_CMAC_KERNEL=smem asks for one-CTA units.  The pair's shared B operand
+// halves the inputs each SM unpacks per MMA: 2048 inputs, 32 channels, 4
+// blocks of 4096 samples 4.70 ms against 4.97 ms on one-CTA units; up to 256
+// inputs one window unit per channel is the smaller cover.
 bool use_pair_kernel(int n_in) {
   if (n_in <= 256) return false;
   const char *e = std::getenv("CORR_CMAC_KERNEL");
-  return e && std::strcmp(e, "pair") == 0;
+  return !e || std::strcmp(e, "smem") != 0;
 }
 
 // Shared-memory stages of the TMEM-operand kernel for n_in inputs: operand
@@ -242,6 +243,7 @@ int corr_create(int n_ant, int n_pol, int n_chan, int block_len, corr_ctx **out)
   ctx->pk_stages = L.pk_stages;
   ctx->z_stage_bytes = L.z_stage_bytes;
   ctx->pk_stage_bytes = L.pk_stage_bytes;
+  ctx->sum_rows = L.sum_rows;
   ctx->smem_bytes = L.smem_bytes;
   // the TMEM-operand kernel where it is the faster one (up to three row
   // tiles); the item split then models its one window unit
@@ -365,6 +367,7 @@ int launch_staged(corr_ctx *ctx, const uint8_t *const *staged, int nb, cudaStrea
   p.pk_stages = ctx->pk_stages;
   p.z_stage_bytes = ctx->z_stage_bytes;
   p.pk_stage_bytes = ctx->pk_stage_bytes;
+  p.sum_rows = ctx->sum_rows;
   xe::XMaps maps;
   std::memset(&maps, 0, sizeof(maps));
   int rc;

@@ -22,6 +22,7 @@
 
 #include "corr.h"
 #include "xe_internal.h"
+#include "xe_sched.h"
 
 namespace {
 
@@ -141,12 +142,14 @@ int plan_single_window(int N, xe::XUnit *units) {
     r.pk_off = 0;
     u.n_reg = 1;
     u.z_rows = 2 * r.n_in;
+    u.n_sum = r.n_in;
     u.pk_bytes = r.n_in * xe::kPackedRowBytes;
     for (int t = n_rt - 1; t >= 0; --t) {
       if (bin_of[t] != b) continue;
       xe::XSeg &s = u.seg[u.n_seg];
       s.a_zrow = 128 * t;
       s.b_zrow = 0;
+      s.a_sum = xe::kTileInputs * t;
       s.b_sbo = 2048;
       s.n = std::min(xe::kTileInputs * (t + 1), n16);
       s.tmem_col = u.work;
@@ -187,16 +190,18 @@ extern "C" int corr_xcorr_static(const uint8_t *d_block, int n_ant, int n_pol, i
   const int n_tpl = plan_single_window((int)N, units);
   if (n_tpl > kMaxStaticUnits || n_tpl > kMaxCallUnits) return CORR_EINVAL;
   plan.n_units = n_tpl;
-  int max_z = 0, max_pk = 0;
+  int max_z = 0, max_pk = 0, max_sum = 0;
   for (int k = 0; k < n_tpl; ++k) {
     max_z = std::max(max_z, units[k].z_rows);
     max_pk = std::max(max_pk, units[k].pk_bytes);
+    max_sum = std::max(max_sum, units[k].n_sum);
   }
   // shared-memory stages, sized as for a context
   const int optin = g_smem_optin[dev];
   const int z_bytes = (max_z * 128 + 1023) / 1024 * 1024;
   const int pk_bytes = (max_pk + 1023) / 1024 * 1024;
-  const int fixed = 1024 + xe::kBarrierBytes;
+  const int fixed = 1024 + xe::kBarrierBytes + xe::kEpiWarps * xe::kEpiBufBytes +
+                    max_sum * xe::kSumBytesPerInput;
   int pk_stages = 3, z_stages = 0;
   for (int ps = 3; ps >= 2 && z_stages < 2; --ps) {
     pk_stages = ps;
@@ -247,18 +252,21 @@ extern "C" int corr_xcorr_static(const uint8_t *d_block, int n_ant, int n_pol, i
   xe::XParams p;
   std::memset(&p, 0, sizeof(p));
   p.probs = d_prob;
-  p.items = nullptr;  // whole units, dealt round-robin over the CTAs
+  p.items = nullptr;  // units (or their fold windows), dealt round-robin over the CTAs
   p.cta_first = nullptr;
   p.implicit_n_tpl = n_tpl;
   p.implicit_n_chan = n_chan;
   p.implicit_npk = prob.pk_per_block;
+  // as many items per unit as keep every fp32 partial exact
+  p.implicit_nseg = (prob.pk_per_block + xe::kMaxFoldStages - 1) / xe::kMaxFoldStages;
   p.status = d_status;
   p.timeout_ns = g_timeout_ns;
   p.z_stages = z_stages;
   p.pk_stages = pk_stages;
   p.z_stage_bytes = (uint32_t)z_bytes;
   p.pk_stage_bytes = (uint32_t)pk_bytes;
-  const long long n_work = (long long)n_tpl * n_chan;
+  p.sum_rows = max_sum;
+  const long long n_work = (long long)n_tpl * n_chan * p.implicit_nseg;
   const int grid = (int)std::min<long long>(n_work, g_n_sm[dev]);
   return rc_of(xe::launch_cmac(maps, p, grid, smem, st));
 }

@@ -234,6 +234,16 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar, uint32_t rank)
       : "memory");
 }
 
+// Two words to the same shared-memory offset in cluster CTA `rank`.
+__device__ __forceinline__ void st_cluster_v2(uint32_t addr, uint32_t rank, uint32_t x,
+                                              uint32_t y) {
+  asm volatile(
+      "{\n.reg .b32 ra;\n"
+      "mapa.shared::cluster.u32 ra, %0, %1;\n"
+      "st.shared::cluster.v2.b32 [ra], {%2, %3};\n}" ::"r"(addr), "r"(rank), "r"(x), "r"(y)
+      : "memory");
+}
+
 // As mbar_try_wait_sleep, acquiring at cluster scope (for arrivals from the
 // peer CTA).
 __device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity,
@@ -314,6 +324,18 @@ __device__ __forceinline__ void tmem_ld_32x32b_x16(uint32_t taddr, uint32_t (&v)
       : "memory");
 }
 
+// 16 lanes x 256 bits, repeated twice along the columns (16 columns): thread i
+// reads lane (i / 4) into v[4k], v[4k + 1] and lane (i / 4) + 8 into
+// v[4k + 2], v[4k + 3], at columns 8k + 2 (i % 4) + {0, 1} (k = 0, 1).
+__device__ __forceinline__ void tmem_ld_16x256b_x2(uint32_t taddr, uint32_t (&v)[8]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
+        "=r"(v[7])
+      : "r"(taddr)
+      : "memory");
+}
+
 __device__ __forceinline__ void tmem_ld_wait() {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
@@ -351,6 +373,14 @@ __host__ __device__ constexpr uint32_t idesc_f16_f32(int M, int N) {
 __host__ __device__ constexpr uint32_t idesc_e5m2_f32(int M, int N) {
   return (1u << 4)                              // D format: f32
          | (1u << 7) | (1u << 10)               // A, B format: E5M2
+         | ((uint32_t)(N >> 3) << 17)           // N / 8
+         | ((uint32_t)(M >> 4) << 24);          // M / 16
+}
+
+// Instruction descriptor, kind::f8f6f4: E4M3 A and B (K-major), fp32 D.
+__host__ __device__ constexpr uint32_t idesc_e4m3_f32(int M, int N) {
+  return (1u << 4)                              // D format: f32
+         | (0u << 7) | (0u << 10)               // A, B format: E4M3
          | ((uint32_t)(N >> 3) << 17)           // N / 8
          | ((uint32_t)(M >> 4) << 24);          // M / 16
 }

@@ -39,6 +39,11 @@ constexpr int kMaxRegionInputs = 2 * 8 * kUnpackWarps;
 constexpr int kMaxPkStages = 8;
 constexpr int kMaxZStages = 6;
 constexpr int kBarrierBytes = 512;
+// One epilogue warp's buffer: 8 rows of 16 (re, im) int32 pairs.
+constexpr int kEpiBufBytes = 8 * 16 * 8;
+// Two tables of operand sums (the item being folded and the next), an entry
+// of two words per staged input.
+constexpr int kSumBytesPerInput = 2 * 8;
 // Blocks integrated by one launch before the fold into int64.
 constexpr int kMaxBlocksPerLaunch = 8;
 
@@ -56,6 +61,7 @@ struct XRegion {
   int interleaved;
   int z_row;        // first row in the Z stage buffer (multiple of 8)
   int pk_off;       // byte offset in the packed stage buffer
+  int sum_row;      // first entry in the CTA's table of operand sums (one per input)
   int chan_off;     // channel: the item's first channel + chan_off
 };
 
@@ -66,6 +72,8 @@ struct XSeg {
   int b_sbo;     // byte stride between 8-row groups of B (2048 interleaved, 1024 plain)
   int n;         // B rows = output columns (multiple of 16, <= 256)
   int tmem_col;  // first TMEM column of the accumulator
+  int a_sum;     // entries of the table of operand sums: the tile's first row,
+  int b_sum;     // and the first column (a pair: of each CTA's half of the columns)
   int row_in0;   // input index of the tile's first row
   int row_in1;   // the same on the odd CTA of a pair (unused otherwise)
   // input index of the first column of each 64-column block of the
@@ -90,6 +98,7 @@ struct XUnit {
   // N / 2 B rows followed by the odd one's
   int pair_rows;
   int z_rows;    // rows staged per chunk (sum over regions)
+  int n_sum;     // inputs staged per chunk (sum over regions)
   int pk_bytes;  // packed bytes per chunk (sum over regions)
   int work;      // relative MMA work (sum of n), for ordering
   XRegion reg[2];
@@ -151,16 +160,18 @@ __device__ __forceinline__ void acc_add(int64_t *base, long long elems, int *sta
 struct XParams {
   const XProb *probs;
   // Explicit items: CTA b runs items [cta_first[b], cta_first[b + 1]).
-  // With items == nullptr the launch holds problem 0 alone and CTA b runs the
-  // whole units b, b + grid, ... of its n_tpl x n_chan units (unit w is
-  // template w / n_chan on channel w % n_chan) over all npk stages.
+  // With items == nullptr the launch holds problem 0 alone and CTA b runs
+  // items b, b + grid, ... of its n_tpl x n_chan units (unit w is template
+  // w / n_chan on channel w % n_chan), all npk stages of each.
   const XItem *items;
   const int *cta_first;
-  int implicit_n_tpl, implicit_n_chan, implicit_npk;
+  // Each unit is cut into implicit_nseg items of equal length.
+  int implicit_n_tpl, implicit_n_chan, implicit_npk, implicit_nseg;
   int *status;           // device status word (kStatusTimeout | kStatusBounds)
   unsigned long long timeout_ns;
   int z_stages, pk_stages;
   uint32_t z_stage_bytes, pk_stage_bytes;
+  int sum_rows;    // entries of a table of operand sums (largest n_sum of the launch)
   int selftest_never;  // failure-detection self-test (see corr_selftest_timeout)
   // 1: the blocks are in F-engine order, uint8 [time][channel][input], and
   // their maps are 3-D (input, channel, time) with 64-input x 128-sample
@@ -245,6 +256,9 @@ cudaError_t launch_cmac_pair(const XMaps &maps, const XParams &p, int clusters, 
 // Clusters of two CTAs of the pair instance that can be resident at once
 // (0 if the query fails).
 int cmac_pair_clusters(int smem_bytes);
+cudaError_t launch_cmac_batch_pair(const XBatchMaps &maps, const XParams &p, int clusters,
+                                   int smem_bytes, cudaStream_t stream);
+int cmac_pair_clusters_batch(int smem_bytes);
 cudaError_t launch_cmac_tm(const XMaps &maps, const XParams &p, int grid, int smem_bytes,
                            cudaStream_t stream);
 cudaError_t cmac_tm_set_smem(int smem_bytes);

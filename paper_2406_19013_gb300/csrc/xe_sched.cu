@@ -38,9 +38,22 @@ void add_reg(XUnit &u, int in_lo, int n_in, int interleaved) {
   r.interleaved = interleaved;
   r.z_row = u.z_rows;
   r.pk_off = u.pk_bytes;
+  r.sum_row = u.n_sum;
   u.z_rows += interleaved ? 2 * n_in : n_in;
+  u.n_sum += n_in;
   u.pk_bytes += n_in * kPackedRowBytes;
   u.n_reg++;
+}
+
+// Entry of the table of operand sums that belongs to Z row z of unit u (the
+// row of an 8-row group of A rows).
+int sum_entry(const XUnit &u, int z) {
+  for (int r = 0; r < u.n_reg; ++r) {
+    const XRegion &g = u.reg[r];
+    const int step = g.interleaved ? 2 : 1;
+    if (z >= g.z_row && z < g.z_row + step * g.n_in) return g.sum_row + (z - g.z_row) / step;
+  }
+  return 0;
 }
 
 XUnit empty_unit() {
@@ -174,22 +187,25 @@ std::vector<XUnit> build_schedule(int N, int cover) {
       }
     }
   } else {
-    // pairs of row tiles (2m, 2m+1) against 256-column pieces of their strip
+    // pairs of row tiles (2m, 2m+1) against W-column pieces of their strip;
+    // above 256 inputs, where a piece's columns are staged beside 128 rows,
+    // 192 columns (256 would leave no shared memory for the operand sums)
+    const int W = N > 256 ? 192 : 256;
     for (int m = 0; 2 * m < n_rt; ++m) {
       const int t0 = 2 * m;
       const bool two = t0 + 1 < n_rt;
       const int row_lo = kTileInputs * t0;
-      const int kd = row_lo / 256;  // piece holding the diagonal
+      const int kd = row_lo / W;  // piece holding the diagonal
       for (int k = 0; k <= kd; ++k) {
         XUnit u = empty_unit();
         if (k < kd) {
           add_reg(u, row_lo, two ? 128 : 64, 1);
-          add_reg(u, 256 * k, 256, 0);
+          add_reg(u, W * k, W, 0);
           const int bz = u.reg[1].z_row;
-          add_seg(u, 0, bz, 1024, 256, row_lo, 256 * k);
-          if (two) add_seg(u, 128, bz, 1024, 256, row_lo + 64, 256 * k);
+          add_seg(u, 0, bz, 1024, W, row_lo, W * k);
+          if (two) add_seg(u, 128, bz, 1024, W, row_lo + 64, W * k);
         } else {
-          const int lo = 256 * k;
+          const int lo = W * k;
           const int hi = row_lo + (two ? 128 : 64);
           // inputs lo .. row_lo - 1 are only columns here: no Q rows
           if (row_lo > lo) add_reg(u, lo, row_lo - lo, 2);
@@ -204,6 +220,11 @@ std::vector<XUnit> build_schedule(int N, int cover) {
   }
   std::stable_sort(units.begin(), units.end(),
                    [](const XUnit &a, const XUnit &b) { return a.work > b.work; });
+  for (XUnit &u : units)
+    for (int s = 0; s < u.n_seg; ++s) {
+      u.seg[s].a_sum = sum_entry(u, u.seg[s].a_zrow);
+      u.seg[s].b_sum = sum_entry(u, u.seg[s].b_zrow);
+    }
   // the unpack handles regions of at most kMaxRegionInputs inputs (every
   // cover above satisfies this; an empty schedule reports a violation)
   for (const XUnit &u : units)
@@ -221,17 +242,21 @@ int tile_ch_rows(const std::vector<XUnit> &units) {
 
 bool stage_layout(const std::vector<const std::vector<XUnit> *> &unit_sets, int smem_optin,
                   int max_z, StageLayout *out) {
-  int max_zr = 0, max_pk = 0;
+  int max_zr = 0, max_pk = 0, max_sum = 0;
   for (const auto *set : unit_sets)
     for (const XUnit &u : *set) {
       max_zr = std::max(max_zr, u.z_rows);
       max_pk = std::max(max_pk, u.pk_bytes);
+      max_sum = std::max(max_sum, (u.pair_rows ? 2 : 1) * u.n_sum);
     }
   StageLayout L;
+  L.sum_rows = max_sum;
   L.z_stage_bytes = (uint32_t)round_up(max_zr * 128, 1024);
   L.pk_stage_bytes = (uint32_t)round_up(max_pk, 1024);  // swizzled TMA destination
-  const int fixed = 1024 /* alignment slack */ + kBarrierBytes;
-  static_assert(8 * (2 * kMaxPkStages + 2 * kMaxZStages + 2 + kMmaWarps + 1) + 16 <= kBarrierBytes,
+  const int fixed = 1024 /* alignment slack */ + kBarrierBytes + kEpiWarps * kEpiBufBytes +
+                    max_sum * kSumBytesPerInput;
+  static_assert(8 * (2 * kMaxPkStages + 2 * kMaxZStages + 2 + kMmaWarps + 1 + 6) + 16 <=
+                    kBarrierBytes,
                 "barrier area");
   const int avail = smem_optin - fixed;
   const int zb = (int)L.z_stage_bytes, pb = (int)L.pk_stage_bytes;

@@ -33,6 +33,7 @@ std::vector<XUnit> build_schedule(int n_in, int cover = kCoverWindow);
 struct StageLayout {
   int z_stages, pk_stages;
   uint32_t z_stage_bytes, pk_stage_bytes;
+  int sum_rows;  // entries of a table of operand sums
   int smem_bytes;
 };
 // Largest z_stages (<= max_z, >= 2) and pk_stages (3 if it leaves >= 2
@@ -49,10 +50,12 @@ struct ProbWork {
   int n_blocks;  // blocks in the launch
 };
 
-// Packed stages one item may integrate before its fold: 1023 stages are at
-// most 130944 samples, so every fp32 partial stays an integer below 2^24
-// (128 per sample at most).
-constexpr int kMaxFoldStages = 131071 / kPkSamples;
+// Packed stages one item may integrate before its fold: 32768 samples.  The
+// biased operands are integers u in [0, 15], so a sample adds at most
+// 2 x 15^2 = 450 to an accumulator (in units of 2^-18) and 32768 of them stay
+// below 2^24: every fp32 partial is exact.
+constexpr int kMaxFoldStages = 32768 / kPkSamples;
+static_assert(2LL * 15 * 15 * kMaxFoldStages * kPkSamples < (1LL << 24), "exact fp32 partials");
 
 // Cuts every unit (problem, template, channel) into items and deals
 // contiguous runs of them to at most `grid` CTAs.  Each CTA receives about

@@ -57,6 +57,24 @@ __device__ __forceinline__ void decode_word_a(uint32_t w, uint2 &a) {
   a = make_uint2(__byte_perm(re02, im02, 0x7531), __byte_perm(re13, im13, 0x7531));
 }
 
+// The biased E4M3 form of the same samples (xengine.cu's operand rows).  E4M3
+// is linear over its subnormals and first binade: the byte c, 0 <= c <= 15,
+// is c 2^-9, and 0x80 | c is -c 2^-9.  So the nibble n of a two's complement
+// value v, with its sign bit flipped, is already the operand of u = v + 8
+// (in units of 2^-9): one logic operation makes four operand bytes, where the
+// exact E5M2 form above takes two half-precision operations, two logic
+// operations and a byte permute.  The products then carry the bias of 8 on
+// both sides, which the epilogue takes out with the rows' sums of u.
+// re, im: u of the four samples; nre: -u of the real parts.  A row piece:
+// (re, im); Q row piece: (im, nre).
+__device__ __forceinline__ void decode_biased(uint32_t w, uint32_t &re, uint32_t &im,
+                                              uint32_t &nre) {
+  const uint32_t hi = w >> 4;
+  im = (w & 0x0F0F0F0Fu) ^ 0x08080808u;
+  re = (hi & 0x0F0F0F0Fu) ^ 0x08080808u;
+  nre = (hi & 0x0F0F0F0Fu) ^ 0x88888888u;
+}
+
 // 16-byte shared-memory load and store on a 32-bit shared address.  The
 // operand buffers are carved from the dynamic shared memory by integer
 // alignment, so plain pointers into them would be generic pointers; these
@@ -75,6 +93,16 @@ __device__ __forceinline__ uint32_t lds32(uint32_t a) {
   uint32_t v;
   asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(a));
   return v;
+}
+__device__ __forceinline__ void lds64(uint32_t a, uint32_t &x, uint32_t &y) {
+  asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(x), "=r"(y) : "r"(a));
+}
+__device__ __forceinline__ void sts64(uint32_t a, uint32_t x, uint32_t y) {
+  asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y));
+}
+// Atomic add into shared memory.
+__device__ __forceinline__ void reds32(uint32_t a, int v) {
+  asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 // As sts128, 1024 bytes (eight 128-byte operand rows) further on.
 __device__ __forceinline__ void sts128_q(uint32_t a, uint32_t x, uint32_t y, uint32_t z,

@@ -8,15 +8,21 @@
 // product D = Arows * Brows^T, where every input contributes an "A row"
 // [a, b] (used on both sides) and a "Q row" [b, -a] (row side only).  That is
 // a dense rank-2T update, so it runs on the tensor cores: 8-bit float operands
-// (E5M2: every integer in [-8, 8] is exact) and fp32 accumulators in TMEM.
-// Each product is an integer of magnitude <= 64 and an item never spans more
-// than 131071 samples, so its partial sums stay below 128 * 131071 < 2^24 and
-// every fp32 accumulation is exact; each item's partials are folded into the
-// int64 integration buffer when it ends.
+// and fp32 accumulators in TMEM.  The operands are E4M3 bytes of the biased
+// values u = v + 8, 0 <= u <= 15 (E4M3 is linear there: byte u is u 2^-9), so
+// a nibble becomes an operand byte by one logic operation; 15 operations for
+// four samples' A and Q rows became 4 (192 inputs, 1024 channels, 8 blocks of
+// 8192 samples with the dump: 5.85 -> 4.88 ms).  The epilogue takes the bias
+// out exactly with the rows' sums of u, which the unpack warps accumulate:
+//   sum (u_i - 8)(u_j - 8) = sum u_i u_j - 8 sum u_i - 8 sum u_j + 64 T.
+// A sample adds at most 2 x 225 units of 2^-18 to an accumulator and an item
+// spans at most 32768 samples, so every fp32 partial is an integer below 2^24
+// (times 2^-18) and exact; each item's sums are folded into the int64
+// integration buffer when it ends.
 //
 // Kernel structure (persistent, one CTA per SM, 25 warps):
 //   warp 20     TMA producer: packed bytes [channel][input][time] -> smem ring
-//   warps 0-15  unpack: 4-bit nibbles -> E5M2 A/Q rows in the 128B-swizzled
+//   warps 0-15  unpack: 4-bit nibbles -> E4M3 A/Q rows in the 128B-swizzled
 //               K-major layout the MMA reads (the paper's CPU "fluff" step,
 //               Sec. 2.3, moved on chip)
 //   warps 21-24 MMA issuers: tcgen05.mma M=128 (64 inputs' A rows + Q rows),
@@ -24,10 +30,11 @@
 //               one issuing thread per accumulator, because a single thread
 //               issues an MMA only every ~110-126 cycles in a loop with
 //               waits and commits, too slow for the N = 64 strips alone
-//   warps 16-19 epilogue: tcgen05.ld of the fp32 accumulators, exchange of
-//               re/im between lanes, int64 red.add into the lower triangle
+//   warps 16-19 epilogue: tcgen05.ld of the fp32 accumulators, bias out,
+//               rows regrouped through a small buffer, int64 red.add into the
+//               lower triangle (256 contiguous bytes an instruction)
 // A launch integrates up to kMaxBlocksPerLaunch blocks; the host cuts its
-// items at fold windows of at most 131071 samples.
+// items at fold windows of at most 32768 samples.
 // A work unit is (problem, template, channel); a template names the inputs
 // staged per chunk and the MMAs (row tile x column range) that cover its part
 // of the triangle.  The host cuts the units into items (a unit over a range
@@ -48,6 +55,7 @@
 
 #include "ptx.cuh"
 #include "xe_internal.h"
+#include "xe_sched.h"
 #include "xe_unpack.cuh"
 
 namespace xe {
@@ -56,6 +64,9 @@ namespace {
 
 struct Bars {
   uint32_t pk_full, pk_empty, z_full, z_empty, acc_full, acc_empty, drain, never;
+  // the two tables of operand sums: written by the unpack warps, read by the
+  // epilogue, and (F-engine order) read by all of it and not yet cleared
+  uint32_t sum_full, sum_empty, sum_read;
 };
 
 }  // namespace
@@ -65,10 +76,11 @@ __device__ __forceinline__ XItem item_at(const XParams &p, int it) {
   if (p.items) return p.items[it];
   XItem r;
   r.prob = 0;
-  r.tpl = it / p.implicit_n_chan;
-  r.chan = it - r.tpl * p.implicit_n_chan;
-  r.pk0 = 0;
-  r.npk = p.implicit_npk;
+  const int unit = it / p.implicit_nseg, seg = it - unit * p.implicit_nseg;
+  r.tpl = unit / p.implicit_n_chan;
+  r.chan = unit - r.tpl * p.implicit_n_chan;
+  r.pk0 = (int)((long long)p.implicit_npk * seg / p.implicit_nseg);
+  r.npk = (int)((long long)p.implicit_npk * (seg + 1) / p.implicit_nseg) - r.pk0;
   return r;
 }
 
@@ -96,9 +108,14 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint8_t *pk_buf = z_buf + (size_t)p.z_stages * p.z_stage_bytes;
   uint64_t *bar_mem = reinterpret_cast<uint64_t *>(pk_buf + (size_t)p.pk_stages * p.pk_stage_bytes);
   // [pk_full x S][pk_empty x S][z_full x Z][z_empty x Z][acc_full][acc_empty][drain x kMmaWarps]
-  // [never]: the last is only waited on by the failure-detection self-test
+  // [never]: only waited on by the failure-detection self-test
+  // [sum_full x 2][sum_empty x 2][sum_read x 2]
   uint32_t *misc = reinterpret_cast<uint32_t *>(bar_mem + 2 * p.pk_stages + 2 * p.z_stages + 2 +
-                                                kMmaWarps + 1);
+                                                kMmaWarps + 1 + 6);
+  // behind the barrier area: the epilogue warps' buffers, then the two tables
+  // of operand sums (p.sum_rows entries of 8 bytes each)
+  uint8_t *epi_mem = reinterpret_cast<uint8_t *>(bar_mem) + kBarrierBytes;
+  uint8_t *sum_mem = epi_mem + kEpiWarps * kEpiBufBytes;
   volatile int *abort_flag = reinterpret_cast<volatile int *>(misc + 1);
   const uint32_t bar0 = smem_u32(bar_mem);
   Bars b;
@@ -110,6 +127,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   b.acc_empty = b.acc_full + 8;
   b.drain = b.acc_empty + 8;
   b.never = b.drain + 8 * kMmaWarps;
+  b.sum_full = b.never + 8;
+  b.sum_empty = b.sum_full + 16;
+  b.sum_read = b.sum_empty + 16;
+  const uint32_t sum_s0 = smem_u32(sum_mem), sum_tab = (uint32_t)p.sum_rows * 8u;
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -127,9 +148,17 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_init(b.acc_empty, PAIR ? 2 * kEpiWarps : kEpiWarps);
     for (int m = 0; m < kMmaWarps; ++m) mbar_init(b.drain + 8 * m, 1);
     mbar_init(b.never, 1);  // nothing ever arrives here
+    for (int k = 0; k < 2; ++k) {
+      mbar_init(b.sum_full + 8 * k, (PAIR ? 2 : 1) * kUnpackWarps);
+      mbar_init(b.sum_empty + 8 * k, (PAIR ? 2 : 1) * kEpiWarps);
+      mbar_init(b.sum_read + 8 * k, kEpiWarps);
+    }
     *abort_flag = 0;
     fence_mbar_init();
   }
+  if (TCN)  // the transposing unpack adds to the tables, starting from zero
+    for (int k = threadIdx.x; k < 4 * p.sum_rows; k += kThreads)
+      reinterpret_cast<uint32_t *>(sum_mem)[k] = 0u;
   if (warp == kWarpMma0) {
     if (PAIR) {
       tmem_alloc_pair(smem_u32(misc), kTmemCols);
@@ -242,7 +271,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (int j = 0; j < 2; ++j) {
           const XSeg &sgm = u->seg[j < n_mine ? m + kMmaWarps * j : 0];
           d_col[j] = tmem + (uint32_t)sgm.tmem_col;
-          idesc[j] = idesc_e5m2_f32(PAIR ? 256 : 128, sgm.n);
+          idesc[j] = idesc_e4m3_f32(PAIR ? 256 : 128, sgm.n);
           a_lo[j] = sdesc_sw128_lo(z0 + (uint32_t)sgm.a_zrow * 128u);
           b_lo[j] = sdesc_sw128_lo(z0 + (uint32_t)sgm.b_zrow * 128u);
           b_hi[j] = sdesc_sw128_hi((uint32_t)sgm.b_sbo);
@@ -342,11 +371,20 @@ __global__ void __launch_bounds__(kThreads, 1)
     int s = 0, zs = 0;
     uint32_t ph = 0, zph = 0;
     bool ok = true;
-    for (int it = it0; it < it1 && ok && !*abort_flag; it += it_step) {
+    long long nu = 0;
+    for (int it = it0; it < it1 && ok && !*abort_flag; it += it_step, ++nu) {
       const XItem item = item_at(p, it);
       const XProb pb = p.probs[item.prob];
       const XUnit *u = pb.units + item.tpl;
       const int n_reg = u->n_reg;
+      // This thread's share of the operand sums: for each of its rows, the
+      // sums of u over the item's real and imaginary parts.  (F-engine order:
+      // for each of its four inputs of a region, both in one word's halves:
+      // at most 512 chunks x 8 samples x 15 < 2^16.)
+      uint32_t sum_re[2][2] = {{0u, 0u}, {0u, 0u}}, sum_im[2][2] = {{0u, 0u}, {0u, 0u}};
+      uint32_t sum_tcn[2][4] = {{0u, 0u, 0u, 0u}, {0u, 0u, 0u, 0u}};
+      static_assert(!TCN || kMaxFoldStages * kChunksPerPk * 8 * 15 < 65536, "16-bit sums");
+      int n_chunks = 0;
       // per-region constants of this thread (at most two regions).  When
       // both regions together have at most R rows (a two-channel unit),
       // region 1's rows follow region 0's in the thread mapping, so every
@@ -368,6 +406,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       for (int k = item.pk0; k < item.pk0 + item.npk && ok; ++k) {
         const int nch = chunks_in_pk(pb, k % pb.pk_per_block);
+        n_chunks += nch;
         if (!mbar_wait(b.pk_full + 8 * s, ph, abort_flag, to)) { ok = false; break; }
         const uint32_t pk_s = pk_s0 + (uint32_t)s * p.pk_stage_bytes;
 #pragma unroll
@@ -404,15 +443,17 @@ __global__ void __launch_bounds__(kThreads, 1)
                 transpose4(w[4], w[5], w[6], w[7], hi[0], hi[1], hi[2], hi[3]);
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                  uint2 al, ql, ah, qh;
-                  decode_word(lo[e], al, ql);
-                  decode_word(hi[e], ah, qh);
+                  uint32_t re_l, im_l, nre_l, re_h, im_h, nre_h;
+                  decode_biased(lo[e], re_l, im_l, nre_l);
+                  decode_biased(hi[e], re_h, im_h, nre_h);
+                  sum_tcn[r][e] = __dp4a(re_l + re_h, 0x01010101u, sum_tcn[r][e]) +
+                                  (__dp4a(im_l + im_h, 0x01010101u, 0u) << 16);
                   const int i_rel = kTileInputs * box + 4 * qd + e, grp = i_rel >> 3;
                   const int pos = ((i_rel & 7) + (grp & 3)) & 7;
                   const int zrow = rg.z_row + (rg.interleaved ? 16 * grp : 8 * grp) + pos;
                   const uint32_t d = z_s + (uint32_t)zrow * 128u + (uint32_t)((j ^ pos) << 4);
-                  sts128(d, al.x, al.y, ah.x, ah.y);
-                  if (rg.interleaved == 1) sts128_q(d, ql.x, ql.y, qh.x, qh.y);
+                  sts128(d, re_l, im_l, re_h, im_h);
+                  if (rg.interleaved == 1) sts128_q(d, im_l, nre_l, im_h, nre_h);
                 }
               }
             }
@@ -432,26 +473,19 @@ __global__ void __launch_bounds__(kThreads, 1)
               const uint4 in = kr == 0 ? in0 : in1;
               const uint32_t d0 = dst + (kr ? dst_step[r] : 0u) + off0;
               const uint32_t d1 = dst + (kr ? dst_step[r] : 0u) + off1;
-              if (il[r]) {
-                uint2 a0, q0, a1, q1, a2, q2, a3, q3;
-                decode_word(in.x, a0, q0);
-                decode_word(in.y, a1, q1);
-                decode_word(in.z, a2, q2);
-                decode_word(in.w, a3, q3);
-                sts128(d0, a0.x, a0.y, a1.x, a1.y);
-                sts128(d1, a2.x, a2.y, a3.x, a3.y);
-                // the Q rows follow 8 rows (1024 bytes) after the A rows
-                sts128_q(d0, q0.x, q0.y, q1.x, q1.y);
-                sts128_q(d1, q2.x, q2.y, q3.x, q3.y);
-              } else {
-                uint2 a0, a1, a2, a3;
-                decode_word_a(in.x, a0);
-                decode_word_a(in.y, a1);
-                decode_word_a(in.z, a2);
-                decode_word_a(in.w, a3);
-                sts128(d0, a0.x, a0.y, a1.x, a1.y);
-                sts128(d1, a2.x, a2.y, a3.x, a3.y);
+              uint32_t re0, im0, nre0, re1, im1, nre1, re2, im2, nre2, re3, im3, nre3;
+              decode_biased(in.x, re0, im0, nre0);
+              decode_biased(in.y, re1, im1, nre1);
+              decode_biased(in.z, re2, im2, nre2);
+              decode_biased(in.w, re3, im3, nre3);
+              sts128(d0, re0, im0, re1, im1);
+              sts128(d1, re2, im2, re3, im3);
+              if (il[r]) {  // the Q rows follow 8 rows (1024 bytes) after the A rows
+                sts128_q(d0, im0, nre0, im1, nre1);
+                sts128_q(d1, im2, nre2, im3, nre3);
               }
+              sum_re[r][kr] = __dp4a(re0 + re1 + re2 + re3, 0x01010101u, sum_re[r][kr]);
+              sum_im[r][kr] = __dp4a(im0 + im1 + im2 + im3, 0x01010101u, sum_im[r][kr]);
             }
           }
           }
@@ -465,12 +499,86 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         if (++s == p.pk_stages) { s = 0; ph ^= 1u; }
       }
+      // ---- the item's operand sums, for the epilogue: entry = (8 (Ua + Ub) -
+      // 64 T, 8 (Ub - Ua)) with Ua, Ub the sums of u over the input's T real
+      // and imaginary parts (zero-filled samples are u = 8, so they cancel)
+      if (!ok) break;
+      const int sb = (int)(nu & 1);
+      if (!(PAIR ? mbar_wait_cluster(b.sum_empty + 8 * sb, (uint32_t)((nu >> 1) & 1) ^ 1u,
+                                     abort_flag, to)
+                 : mbar_wait(b.sum_empty + 8 * sb, (uint32_t)((nu >> 1) & 1) ^ 1u, abort_flag, to)))
+        break;
+      const uint32_t tab = sum_s0 + (uint32_t)sb * sum_tab;
+      if (TCN) {
+        // the two half-warps hold 16 of a chunk's 64 samples of the same
+        // inputs; four warps hold the 64, and add to the cleared table
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          if (r >= n_reg) break;
+          const XRegion rg = u->reg[r];
+          const bool mine = tid < (rg.n_in / kTileInputs) * 128;  // whole warps
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            int ua = (int)(sum_tcn[r][e] & 0xFFFFu), ub = (int)(sum_tcn[r][e] >> 16);
+            ua += __shfl_xor_sync(0xffffffffu, ua, 16);
+            ub += __shfl_xor_sync(0xffffffffu, ub, 16);
+            if (mine && lane < 16) {
+              const int i_rel = kTileInputs * (tid >> 7) + 4 * (tid & 15) + e, grp = i_rel >> 3;
+              const int at = rg.sum_row + 8 * grp + (((i_rel & 7) + (grp & 3)) & 7);
+              reds32(tab + 8u * (uint32_t)at, 8 * (ua + ub) - 64 * 16 * n_chunks);
+              reds32(tab + 8u * (uint32_t)at + 4u, 8 * (ub - ua));
+            }
+          }
+        }
+      } else {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          const XRegion rg = u->reg[r < n_reg ? r : 0];
+#pragma unroll
+          for (int kr = 0; kr < 2; ++kr) {
+            if (kr >= n_k[r]) break;  // uniform in the warp: its 8 rows lie in one region
+            int ua = (int)sum_re[r][kr], ub = (int)sum_im[r][kr];
+            ua += __shfl_xor_sync(0xffffffffu, ua, 8);
+            ub += __shfl_xor_sync(0xffffffffu, ub, 8);
+            ua += __shfl_xor_sync(0xffffffffu, ua, 16);
+            ub += __shfl_xor_sync(0xffffffffu, ub, 16);
+            if (lane < 8) {
+              const int rr = (r == 1 ? row0 - pack : row0) + R * kr;
+              const uint32_t at =
+                  tab + 8u * (uint32_t)((int)rank * (p.sum_rows >> 1) + rg.sum_row + rr);
+              const uint32_t vx = (uint32_t)(8 * (ua + ub) - 64 * kChunkSamples * n_chunks);
+              const uint32_t vy = (uint32_t)(8 * (ub - ua));
+              sts64(at, vx, vy);
+              if (PAIR) st_cluster_v2(at, rank ^ 1u, vx, vy);
+            }
+          }
+        }
+      }
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(b.sum_full + 8 * sb);
+        if (PAIR) mbar_arrive_cluster(b.sum_full + 8 * sb, rank ^ 1u);
+      }
     }
   } else if (warp < kWarpTma) {
     // ------------------------------------------------------------ epilogue
-    const int q = warp & 3;  // TMEM lane quarter this warp may access
-    const int rho = 32 * q + lane;
-    const int g = rho >> 4, is_im = (rho >> 3) & 1, l = rho & 7;
+    // The warp's TMEM lane quarter holds 16 inputs, each a real row and, 8
+    // lanes on, an imaginary one.  Two 16-lane loads bring 16 columns of 8
+    // inputs each, a thread getting both parts of two columns of one input:
+    // the bias comes off there, and the 8 x 16 complex values go through a
+    // 1 KB buffer so that each atomic instruction adds 256 contiguous bytes
+    // of one row of the integration buffer.  (Lane-per-row adds, 32 rows an
+    // instruction, made four times the memory requests: the fold of a
+    // 192-input channel took 31 us.)
+    const int q = warp & 3;
+    const uint32_t ebuf = smem_u32(epi_mem) + (uint32_t)(warp - kWarpEpi0) * kEpiBufBytes;
+    const int er = lane >> 2, ec = lane & 3;  // the thread's row and column pair as loaded
+    // 16-byte chunk (4 k + ec) of buffer row er, swizzled by the row's parity
+    const uint32_t est0 = ebuf + (uint32_t)(er * 128 + ((ec ^ ((er & 1) << 2)) << 4));
+    const uint32_t est1 = ebuf + (uint32_t)(er * 128 + (((4 + ec) ^ ((er & 1) << 2)) << 4));
+    // word `lane` of an even and of an odd row
+    const uint32_t eld0 = ebuf + (uint32_t)(lane * 4);
+    const uint32_t eld1 = ebuf + (uint32_t)((((lane >> 2) ^ 4) << 4) + (lane & 3) * 4);
     long long nu = 0;
     // failure-detection self-test: wait for a barrier that nothing completes;
     // the bounded wait gives up, raises the abort flag and every role winds
@@ -485,67 +593,73 @@ __global__ void __launch_bounds__(kThreads, 1)
       // integration is void and is reported as such
       if (*abort_flag) break;
       tc_fence_after();
+      const int sb = (int)(nu & 1);
+      if (!(PAIR ? mbar_wait_cluster(b.sum_full + 8 * sb, (uint32_t)((nu >> 1) & 1), abort_flag, to)
+                 : mbar_wait(b.sum_full + 8 * sb, (uint32_t)((nu >> 1) & 1), abort_flag, to)))
+        break;
+      const uint32_t tab = sum_s0 + (uint32_t)sb * sum_tab;
+      const uint32_t rank_off = PAIR ? (uint32_t)(p.sum_rows >> 1) * 8u : 0u;
+      const long long acc_elems = (long long)pb.n_chan * pb.n_pairs * 2;
       const int n_seg = u->n_seg;
-      // in F-engine-order launches, lane 16 g + l holds the input at group
-      // position (l - g) % 8 of its 8-input group, and column 8 G + e the one
-      // at (e - G) % 8 (the groups of a row tile or column range start at
-      // multiples of 64 inputs, so only g % 4 and G % 4 matter)
-      const int l_in = TCN ? ((l - (g & 3)) & 7) : l;
       for (int sg = 0; sg < n_seg; ++sg) {
         const XSeg sgm = u->seg[sg];
-        // a tile of several channels: this lane's row belongs to channel
-        // block ci (the same for every lane of the warp, whose 16 rows lie in
-        // one block of at least 16)
         const int rpc = sgm.ch_rows;
-        const int il = (rank ? sgm.row_in1 : sgm.row_in0) + 8 * g + l_in;
-        const int ci = rpc ? il / rpc : 0;
-        const int c = item.chan + sgm.chan_off + ci;
-        if (c >= pb.n_chan) continue;  // a multi-channel unit's missing last channels
-        const int i = il - ci * rpc;
-        const bool row_ok = i < pb.n_in;
-        int64_t *arow = pb.acc + ((long long)c * pb.n_pairs + (long long)i * (i + 1) / 2) * 2;
-        const long long acc_elems = (long long)pb.n_chan * pb.n_pairs * 2;
-        for (int cb = 0; cb < sgm.n; cb += 16) {
-          uint32_t v[16];
-          __syncwarp();
-          tmem_ld_32x32b_x16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(sgm.tmem_col + cb), v);
-          tmem_ld_wait();
-          int re[8], im[8];
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const uint32_t send = is_im ? v[e] : v[8 + e];
-            const uint32_t got = __shfl_xor_sync(0xffffffffu, send, 8);
-            const int mine = __float2int_rn(__uint_as_float(is_im ? v[8 + e] : v[e]));
-            const int other = __float2int_rn(__uint_as_float(got));
-            re[e] = is_im ? other : mine;
-            im[e] = is_im ? mine : other;
-          }
-          const int cc = cb + (is_im ? 8 : 0);  // the 8 columns of this lane
-          int j0 = sgm.col_blk[cc >> 6] + (cc & 63);
-          bool blk_ok = true;  // the 8 columns lie in this row's channel block
-          if (rpc) {
-            blk_ok = j0 / rpc == ci;
-            j0 -= (j0 / rpc) * rpc;
-          }
-          if (TCN) {
-            const int rot = ((cb + (is_im ? 8 : 0)) >> 3) & 3;
-#pragma unroll
-            for (int e = 0; e < 8; ++e) {
-              const int jj = j0 + ((e - rot) & 7);
-              if (row_ok && blk_ok && jj <= i) {
-                acc_add(pb.acc, acc_elems, p.status, arow + 2 * (long long)jj, re[e]);
-                acc_add(pb.acc, acc_elems, p.status, arow + 2 * (long long)jj + 1, im[e]);
-              }
+#pragma unroll 1
+        for (int h = 0; h < 2; ++h) {
+          // 8 inputs: group g of the tile.  In F-engine-order launches group
+          // position l holds input (l - g) % 8 of the group, and column 8 G +
+          // e the one at (e - G) % 8 (a row tile or column range starts at a
+          // multiple of 64 inputs, so only g % 4 and G % 4 matter).
+          const int g = 2 * q + h;
+          const int i_tile = (rank ? sgm.row_in1 : sgm.row_in0) + 8 * g;
+          // a tile of several channels: the 8 rows belong to channel block ci
+          const int ci = rpc ? i_tile / rpc : 0;
+          const int c = item.chan + sgm.chan_off + ci;
+          if (c >= pb.n_chan) continue;  // a multi-channel unit's missing last channels
+          const int i0 = i_tile - ci * rpc;
+          if (i0 >= pb.n_in) continue;
+          int64_t *cacc = pb.acc + (long long)c * pb.n_pairs * 2;
+          // the row's sums: the thread's row as loaded
+          uint32_t p_i, m_i;
+          lds64(tab + (rank ? rank_off : 0u) + 8u * (uint32_t)(sgm.a_sum + 8 * g + er), p_i, m_i);
+          for (int cb = 0; cb < sgm.n; cb += 16) {
+            // input of the first column, the block's columns being 16 inputs
+            // of one channel block
+            int j0 = sgm.col_blk[cb >> 6] + (cb & 63);
+            if (rpc) {
+              if (j0 / rpc != ci) continue;
+              j0 -= ci * rpc;
             }
-          } else {
-            const int nvalid = row_ok && blk_ok ? min(8, i - j0 + 1) : 0;
-            int64_t *ptr = arow + 2 * (long long)j0;
+            if (j0 > i0 + 7) continue;  // above the diagonal (uniform)
+            uint32_t v[8];
+            __syncwarp();
+            tmem_ld_16x256b_x2(tmem + ((uint32_t)(32 * q + 16 * h) << 16) +
+                                   (uint32_t)(sgm.tmem_col + cb), v);
+            // the two column pairs' sums: of a pair's columns, the first half
+            // is the even CTA's rows, the second the odd one's
+            const int hc = PAIR && cb >= (sgm.n >> 1) ? 1 : 0;
+            const uint32_t cs = tab + (hc ? rank_off : 0u) +
+                                8u * (uint32_t)(sgm.b_sum + cb - hc * (sgm.n >> 1) + 2 * ec);
+            const uint4 s0 = lds128(cs), s1 = lds128(cs + 64u);
+            tmem_ld_wait();
+            // back to whole numbers: accumulators are in units of 2^-18
+            auto whole = [](uint32_t x) { return (uint32_t)__float2int_rn(__uint_as_float(x) * 262144.0f); };
+            sts128(est0, whole(v[0]) - p_i - s0.x, whole(v[2]) - m_i + s0.y,
+                   whole(v[1]) - p_i - s0.z, whole(v[3]) - m_i + s0.w);
+            sts128(est1, whole(v[4]) - p_i - s1.x, whole(v[6]) - m_i + s1.y,
+                   whole(v[5]) - p_i - s1.z, whole(v[7]) - m_i + s1.w);
+            __syncwarp();
+            // lane w adds word w of each row: column w / 2, part w % 2
+            const int jc = lane >> 1;
+            const int j = TCN ? j0 + (jc & 8) + (((jc & 7) - (((cb + jc) >> 3) & 3)) & 7) : j0 + jc;
 #pragma unroll
-            for (int e = 0; e < 8; ++e)
-              if (e < nvalid) {
-                acc_add(pb.acc, acc_elems, p.status, ptr + 2 * e, re[e]);
-                acc_add(pb.acc, acc_elems, p.status, ptr + 2 * e + 1, im[e]);
-              }
+            for (int r = 0; r < 8; ++r) {
+              const int x = (int)lds32((r & 1 ? eld1 : eld0) + (uint32_t)(r * 128));
+              const int i = i0 + (TCN ? ((r - (g & 3)) & 7) : r);
+              if (i < pb.n_in && j <= i)
+                acc_add(pb.acc, acc_elems, p.status,
+                        cacc + (long long)i * (i + 1) + 2 * j + (lane & 1), x);
+            }
           }
         }
       }
@@ -556,6 +670,16 @@ __global__ void __launch_bounds__(kThreads, 1)
           mbar_arrive_cluster(b.acc_empty, 0);
         else
           mbar_arrive(b.acc_empty);
+        mbar_arrive(TCN ? b.sum_read + 8 * sb : b.sum_empty + 8 * sb);
+        if (PAIR) mbar_arrive_cluster(b.sum_empty + 8 * sb, rank ^ 1u);
+      }
+      if (TCN) {
+        // every epilogue warp has read the table: clear it for the item after
+        // the next
+        if (!mbar_wait(b.sum_read + 8 * sb, (uint32_t)((nu >> 1) & 1), abort_flag, to)) break;
+        for (int k = q * 32 + lane; k < p.sum_rows; k += 32 * kEpiWarps) sts64(tab + 8u * k, 0u, 0u);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(b.sum_empty + 8 * sb);
       }
     }
   }
@@ -577,17 +701,18 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 cudaError_t cmac_set_smem(int smem_bytes) {
-  cudaError_t e = cudaFuncSetAttribute(xengine_cmac_kernel<kMaxMaps, false, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(xengine_cmac_kernel<kMaxMaps, true, false>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(xengine_cmac_kernel<kMaxMaps, false, true>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(xengine_cmac_kernel<kMaxBatchMaps, false, false>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+  const void *kernels[] = {
+      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxMaps, false, false>),
+      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxMaps, true, false>),
+      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxMaps, false, true>),
+      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxBatchMaps, false, false>),
+      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxBatchMaps, false, true>)};
+  for (const void *k : kernels) {
+    cudaError_t e =
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 cudaError_t launch_cmac(const XMaps &maps, const XParams &p, int grid, int smem_bytes,
@@ -626,13 +751,28 @@ cudaError_t launch_cmac_pair(const XMaps &maps, const XParams &p, int clusters, 
   return cudaLaunchKernelEx(&c.cfg, xengine_cmac_kernel<kMaxMaps, false, true>, maps, p);
 }
 
+cudaError_t launch_cmac_batch_pair(const XBatchMaps &maps, const XParams &p, int clusters,
+                                   int smem_bytes, cudaStream_t stream) {
+  PairConfig c(clusters, smem_bytes, stream);
+  return cudaLaunchKernelEx(&c.cfg, xengine_cmac_kernel<kMaxBatchMaps, false, true>, maps, p);
+}
+
 int cmac_pair_clusters(int smem_bytes) {
   PairConfig c(1, smem_bytes, nullptr);
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, xengine_cmac_kernel<kMaxMaps, false, true>, &c.cfg) !=
-      cudaSuccess)
-    return 0;
-  return n;
+  return cudaOccupancyMaxActiveClusters(&n, xengine_cmac_kernel<kMaxMaps, false, true>, &c.cfg) ==
+                 cudaSuccess
+             ? n
+             : 0;
+}
+
+int cmac_pair_clusters_batch(int smem_bytes) {
+  PairConfig c(1, smem_bytes, nullptr);
+  int n = 0;
+  return cudaOccupancyMaxActiveClusters(&n, xengine_cmac_kernel<kMaxBatchMaps, false, true>,
+                                        &c.cfg) == cudaSuccess
+             ? n
+             : 0;
 }
 
 cudaError_t launch_cmac_batch(const XBatchMaps &maps, const XParams &p, int grid, int smem_bytes,

@@ -234,13 +234,13 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar, uint32_t rank)
       : "memory");
 }
 
-// Two words to the same shared-memory offset in cluster CTA `rank`.
-__device__ __forceinline__ void st_cluster_v2(uint32_t addr, uint32_t rank, uint32_t x,
-                                              uint32_t y) {
+// Atomic add to the word at the same shared-memory offset in cluster CTA
+// `rank`.
+__device__ __forceinline__ void red_cluster(uint32_t addr, uint32_t rank, int v) {
   asm volatile(
       "{\n.reg .b32 ra;\n"
       "mapa.shared::cluster.u32 ra, %0, %1;\n"
-      "st.shared::cluster.v2.b32 [ra], {%2, %3};\n}" ::"r"(addr), "r"(rank), "r"(x), "r"(y)
+      "red.relaxed.cluster.shared::cluster.add.u32 [ra], %2;\n}" ::"r"(addr), "r"(rank), "r"(v)
       : "memory");
 }
 

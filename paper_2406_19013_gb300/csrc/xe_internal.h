@@ -24,15 +24,17 @@ constexpr int kChunksPerPk = kPkSamples / kChunkSamples;
 // Warp roles (see xengine.cu): unpack, epilogue (one per TMEM lane quarter),
 // TMA producer, MMA issuers (one issue stream per accumulator).
 constexpr int kUnpackWarps = 16;
+constexpr int kUnpackGroup = kUnpackWarps / 2;  // warps that decode one chunk
 constexpr int kEpiWarps = 4;
 constexpr int kMmaWarps = 4;
 constexpr int kWarpEpi0 = kUnpackWarps;
 constexpr int kWarpTma = kWarpEpi0 + kEpiWarps;
 constexpr int kWarpMma0 = kWarpTma + 1;
 constexpr int kThreads = 32 * (kWarpMma0 + kMmaWarps);
-// Largest region the unpack stages: each thread takes at most two rows of a
-// region per chunk (rows row0 and row0 + 8 kUnpackWarps).
-constexpr int kMaxRegionInputs = 2 * 8 * kUnpackWarps;
+// Largest region the unpack stages: each of a group's warps takes at most
+// four 8-row groups of a region per chunk.
+constexpr int kMaxRegionInputs = 4 * 8 * kUnpackGroup;
+static_assert(8 * kUnpackGroup == kTileInputs, "every warp has the same rows of a tile");
 // Pipeline depth limits and the shared-memory area for the barriers (full and
 // empty barrier per stage, accumulator full/empty, one drain barrier per MMA
 // issuer) and the TMEM address / abort flag behind them.

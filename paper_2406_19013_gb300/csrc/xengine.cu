@@ -89,6 +89,81 @@ __device__ __forceinline__ int chunks_in_pk(const XProb &pb, int kc) {
   return min(kChunksPerPk, pb.chunks_per_block - kChunksPerPk * kc);
 }
 
+// Decodes this warp's rows of one chunk of a staged region: n_k groups of 8
+// rows, 64 rows apart.  `src` and `dst` are the lane's addresses in the first
+// group; Q: Q rows are stored 1024 bytes (eight operand rows) after the A
+// rows.  The sums of u go to the halves of sum[k].
+template <bool Q>
+__device__ __forceinline__ void unpack_rows(uint32_t src, uint32_t dst, uint32_t dst_step, int n_k,
+                                            uint32_t (&sum)[4]) {
+  constexpr uint32_t kStep = kTileInputs * kPackedRowBytes;
+  uint4 in[2];
+  in[0] = lds128(src);
+  if (n_k > 1) in[1] = lds128(src + kStep);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    if (k >= n_k) break;
+    const uint4 x = in[k & 1];
+    if (k + 2 < n_k) in[k & 1] = lds128(src + (uint32_t)(k + 2) * kStep);
+    const uint32_t d0 = dst + (Q ? (uint32_t)k * 16384u : (uint32_t)k * dst_step), d1 = d0 ^ 16u;
+    uint32_t re0, im0, nre0, re1, im1, nre1, re2, im2, nre2, re3, im3, nre3;
+    decode_biased(x.x, re0, im0, nre0);
+    decode_biased(x.y, re1, im1, nre1);
+    decode_biased(x.z, re2, im2, nre2);
+    decode_biased(x.w, re3, im3, nre3);
+    sts128(d0, re0, im0, re1, im1);
+    sts128(d1, re2, im2, re3, im3);
+    if (Q) {
+      sts128_q(d0, im0, nre0, im1, nre1);
+      sts128_q(d1, im2, nre2, im3, nre3);
+    }
+    sum[k] = __dp4a(re0 + re1 + re2 + re3, 0x01010101u, sum[k]) +
+             (__dp4a(im0 + im1 + im2 + im3, 0x01010101u, 0u) << 16);
+  }
+}
+
+// The same for a region in F-engine order: each 64-input box is [128
+// samples][64 inputs].  Item (qd, j) of a box: inputs 4 qd .. 4 qd + 3,
+// samples 8 j .. 8 j + 7 of the chunk; eight 4-byte loads (one sample of four
+// inputs each), two 4 x 4 byte transposes, and per input two decoded words:
+// 16 bytes of its A row (and Q row) at K bytes 16 j .. 16 j + 15.  The
+// half-warp of odd j loads its samples rotated by one (the same rotation for
+// every input, so a fixed permutation of K), which puts the two half-warps'
+// rows on different bank halves.  Within every 8-input group of a region the
+// operand row of group position pos is (pos + group) % 8: the eight threads
+// of a store phase then hit eight bank groups.  Thread t of the group takes
+// item t % 128 of boxes t / 128 and t / 128 + 2.
+__device__ __forceinline__ void unpack_turned(uint32_t src, uint32_t dst, int kind, int n_box,
+                                              int t, int sub, uint32_t (&sum)[8]) {
+  const int v = t & 127, qd = v & 15, j = v >> 4, jj = j & 1;
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int box = 2 * k + (t >> 7);
+    if (box >= n_box) break;
+    const uint32_t at =
+        src + (uint32_t)box * 8192u + (uint32_t)(64 * (kChunkSamples * sub + 8 * j)) + 4u * qd;
+    uint32_t w[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) w[i] = lds32(at + 64u * (uint32_t)((i + jj) & 7));
+    uint32_t lo[4], hi[4];
+    transpose4(w[0], w[1], w[2], w[3], lo[0], lo[1], lo[2], lo[3]);
+    transpose4(w[4], w[5], w[6], w[7], hi[0], hi[1], hi[2], hi[3]);
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      uint32_t re_l, im_l, nre_l, re_h, im_h, nre_h;
+      decode_biased(lo[e], re_l, im_l, nre_l);
+      decode_biased(hi[e], re_h, im_h, nre_h);
+      sum[4 * k + e] = __dp4a(re_l + re_h, 0x01010101u, sum[4 * k + e]) +
+                       (__dp4a(im_l + im_h, 0x01010101u, 0u) << 16);
+      const int i_rel = kTileInputs * box + 4 * qd + e, gp = i_rel >> 3;
+      const int pos = ((i_rel & 7) + (gp & 3)) & 7;
+      const uint32_t d = dst + (uint32_t)((kind ? 16 : 8) * gp + pos) * 128u +
+                         (uint32_t)((j ^ pos) << 4);
+      sts128(d, re_l, im_l, re_h, im_h);
+      if (kind == 1) sts128_q(d, im_l, nre_l, im_h, nre_h);
+    }
+  }
+}
 // kThreads = 32 * 25: warps 0-15 unpack, 16-19 epilogue, 20 TMA, 21-24 MMA.
 // Every role walks the same item list, [cta_first[b], cta_first[b + 1]).
 // TCN: the blocks are in F-engine order (XParams::tcn), staged and unpacked
@@ -141,7 +216,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
     for (int s = 0; s < p.z_stages; ++s) {
       // a pair's even CTA also counts the odd CTA's forwarded arrive
-      mbar_init(b.z_full + 8 * s, (PAIR && cluster_ctarank() == 0) ? kUnpackWarps + 1 : kUnpackWarps);
+      mbar_init(b.z_full + 8 * s, (PAIR && cluster_ctarank() == 0) ? kUnpackGroup + 1 : kUnpackGroup);
       mbar_init(b.z_empty + 8 * s, PAIR ? kPairIssuers : kMmaWarps);
     }
     mbar_init(b.acc_full, PAIR ? kPairIssuers : kMmaWarps);
@@ -156,9 +231,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     *abort_flag = 0;
     fence_mbar_init();
   }
-  if (TCN)  // the transposing unpack adds to the tables, starting from zero
-    for (int k = threadIdx.x; k < 4 * p.sum_rows; k += kThreads)
-      reinterpret_cast<uint32_t *>(sum_mem)[k] = 0u;
+  // the unpack warps add to the tables of operand sums, starting from zero
+  for (int k = threadIdx.x; k < 4 * p.sum_rows; k += kThreads)
+    reinterpret_cast<uint32_t *>(sum_mem)[k] = 0u;
   if (warp == kWarpMma0) {
     if (PAIR) {
       tmem_alloc_pair(smem_u32(misc), kTmemCols);
@@ -353,20 +428,25 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp < kUnpackWarps) {
     // ------------------------------------------------------------ unpack
-    // Thread tid owns rows row0 + R k of every staged region (R = 8 *
-    // kUnpackWarps rows per pass) and the 16-sample group g of each chunk;
-    // the 8 lanes of a quarter-warp share g and take 8 consecutive rows, so
-    // their swizzled 16-byte accesses fall on 8 different bank groups.
-    constexpr int R = 8 * kUnpackWarps;
-    // a staged region holds at most 2 R rows, so a thread has at most two
-    // items per chunk: both loads go out before either decode
-    static_assert(2 * R >= kMaxRegionInputs, "two items per thread cover a region");
-    const int tid = threadIdx.x;
-    const int g = (tid >> 3) & 3, row0 = (tid & 7) | ((tid >> 5) << 3), sw = row0 & 7;
+    // The warps form two groups of kUnpackGroup.  A packed stage holds two
+    // operand chunks; group 0 decodes the first and group 1 the second, so a
+    // warp waits, fences and arrives once per stage and has all its loads of
+    // a chunk in flight together.  (All warps on every chunk spent half of
+    // their instructions on that hand-off: 3200 warp instructions per chunk
+    // of 192 inputs.)  A region's inputs are a multiple of kTileInputs, so
+    // every warp has the same number of 8-row groups: rows 8 w + 64 k + 0..7
+    // of the region, a lane one 16-sample group (lane / 8) of one row (lane %
+    // 8); the 8 lanes of a quarter-warp take 8 consecutive rows, so their
+    // swizzled 16-byte accesses fall on 8 different bank groups.
+    const int grp = warp / kUnpackGroup, w8 = warp % kUnpackGroup;
+    const int g = lane >> 3, sw = lane & 7;
+    const int t_grp = 32 * w8 + lane;  // thread of the group
     // packed rows arrive 128B-swizzled: 16-byte chunk c of row r sits at
-    // c ^ (r & 7); operand chunk `sub` of a stage is chunks 4 sub + g
-    const uint32_t src_sub0 = (uint32_t)((g ^ sw) << 4), src_sub1 = (uint32_t)(((4 + g) ^ sw) << 4);
-    const uint32_t off0 = (uint32_t)(((2 * g) ^ sw) << 4), off1 = (uint32_t)(((2 * g + 1) ^ sw) << 4);
+    // c ^ (r & 7); this group's operand chunk is chunks 4 grp + g
+    const uint32_t src_lane =
+        (uint32_t)((8 * w8 + sw) * kPackedRowBytes + (((4 * grp + g) ^ sw) << 4));
+    // the lane's 32 operand bytes are 16-byte chunks 2 g and 2 g + 1
+    const uint32_t dst_lane = (uint32_t)(sw * 128 + (((2 * g) ^ sw) << 4));
     const uint32_t pk_s0 = smem_u32(pk_buf), z_s0 = smem_u32(z_buf);
     int s = 0, zs = 0;
     uint32_t ph = 0, zph = 0;
@@ -377,179 +457,103 @@ __global__ void __launch_bounds__(kThreads, 1)
       const XProb pb = p.probs[item.prob];
       const XUnit *u = pb.units + item.tpl;
       const int n_reg = u->n_reg;
-      // This thread's share of the operand sums: for each of its rows, the
-      // sums of u over the item's real and imaginary parts.  (F-engine order:
-      // for each of its four inputs of a region, both in one word's halves:
-      // at most 512 chunks x 8 samples x 15 < 2^16.)
-      uint32_t sum_re[2][2] = {{0u, 0u}, {0u, 0u}}, sum_im[2][2] = {{0u, 0u}, {0u, 0u}};
-      uint32_t sum_tcn[2][4] = {{0u, 0u, 0u, 0u}, {0u, 0u, 0u, 0u}};
-      static_assert(!TCN || kMaxFoldStages * kChunksPerPk * 8 * 15 < 65536, "16-bit sums");
-      int n_chunks = 0;
-      // per-region constants of this thread (at most two regions).  When
-      // both regions together have at most R rows (a two-channel unit),
-      // region 1's rows follow region 0's in the thread mapping, so every
-      // unpack warp gets work; otherwise both start at row0.
-      const int pack =
-          n_reg == 2 && u->reg[0].n_in + u->reg[1].n_in <= R ? u->reg[0].n_in : 0;
+      // This thread's share of the operand sums: for each of its rows (F-
+      // engine order: for each of its four inputs of a box), the sums of u
+      // over the real parts (low half) and the imaginary parts (high half).
+      uint32_t sums[2][TCN ? 8 : 4];
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int k = 0; k < (TCN ? 8 : 4); ++k) sums[r][k] = 0u;
+      static_assert(kMaxFoldStages * 16 * 15 < 65536, "16-bit sums");
+      int n_mine = 0;  // chunks this warp decoded
+      // per-region constants (at most two regions of at most 256 inputs)
       uint32_t src_off[2], dst_off[2], dst_step[2];
-      int n_k[2], il[2];
+      int n_k[2], kind[2];
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
         const XRegion rg = u->reg[r < n_reg ? r : 0];
-        const int rr = r == 1 ? row0 - pack : row0;  // this thread's row of the region
-        il[r] = rg.interleaved == 1;  // Q rows are decoded and stored
-        const int rho0 = rg.interleaved ? (((rr >> 3) << 4) | sw) : rr;
-        src_off[r] = (uint32_t)(rg.pk_off + rr * kPackedRowBytes);
-        dst_off[r] = (uint32_t)(rg.z_row + rho0) * 128u;
-        dst_step[r] = (uint32_t)((rg.interleaved ? 2 * R : R) * 128);  // R rows further on
-        n_k[r] = r < n_reg && rr >= 0 && rr < rg.n_in ? (rg.n_in - rr + R - 1) / R : 0;
+        kind[r] = rg.interleaved;
+        n_k[r] = r < n_reg ? rg.n_in / kTileInputs : 0;
+        src_off[r] = (uint32_t)rg.pk_off + (TCN ? 0u : src_lane);
+        dst_step[r] = kind[r] ? 16384u : 8192u;  // 64 rows further on
+        dst_off[r] = (uint32_t)rg.z_row * 128u +
+                     (TCN ? 0u : (uint32_t)w8 * (dst_step[r] / kUnpackGroup) + dst_lane);
       }
-      for (int k = item.pk0; k < item.pk0 + item.npk && ok; ++k) {
+      for (int k = item.pk0; k < item.pk0 + item.npk; ++k) {
         const int nch = chunks_in_pk(pb, k % pb.pk_per_block);
-        n_chunks += nch;
         if (!mbar_wait(b.pk_full + 8 * s, ph, abort_flag, to)) { ok = false; break; }
-        const uint32_t pk_s = pk_s0 + (uint32_t)s * p.pk_stage_bytes;
-#pragma unroll
-        for (int sub = 0; sub < kChunksPerPk; ++sub) {
-          if (sub >= nch) break;
-          if (!mbar_wait(b.z_empty + 8 * zs, zph ^ 1u, abort_flag, to)) { ok = false; break; }
-          const uint32_t z_s = z_s0 + (uint32_t)zs * p.z_stage_bytes;
-          if (TCN) {
-            // F-engine order: each 64-input box is [128 samples][64 inputs].
-            // Item (q, j) of a box: inputs 4 q .. 4 q + 3, samples 8 j ..
-            // 8 j + 7 of the chunk; eight 4-byte loads (one sample of four
-            // inputs each), two 4 x 4 byte transposes, and per input two
-            // decoded words: 16 bytes of its A row (and Q row) at K bytes
-            // 16 j .. 16 j + 15.  The half-warp of odd j loads its samples
-            // rotated by one (the same rotation for every input, so a fixed
-            // permutation of K), which puts the two half-warps' rows on
-            // different bank halves.  Within every 8-input group of a region
-            // the operand row of group position pos is (pos + group) % 8: the
-            // eight threads of a store phase then hit eight bank groups.
-#pragma unroll
-            for (int r = 0; r < 2; ++r) {
-              if (r >= n_reg) break;
-              const XRegion rg = u->reg[r];
-              const int u_it = tid;
-              if (u_it < (rg.n_in / kTileInputs) * 128) {
-                const int box = u_it >> 7, v = u_it & 127, qd = v & 15, j = v >> 4, jj = j & 1;
-                const uint32_t src = pk_s + (uint32_t)rg.pk_off + (uint32_t)box * 8192u +
-                                     (uint32_t)(64 * (kChunkSamples * sub + 8 * j)) + 4u * qd;
-                uint32_t w[8];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) w[k] = lds32(src + 64u * (uint32_t)((k + jj) & 7));
-                uint32_t lo[4], hi[4];
-                transpose4(w[0], w[1], w[2], w[3], lo[0], lo[1], lo[2], lo[3]);
-                transpose4(w[4], w[5], w[6], w[7], hi[0], hi[1], hi[2], hi[3]);
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                  uint32_t re_l, im_l, nre_l, re_h, im_h, nre_h;
-                  decode_biased(lo[e], re_l, im_l, nre_l);
-                  decode_biased(hi[e], re_h, im_h, nre_h);
-                  sum_tcn[r][e] = __dp4a(re_l + re_h, 0x01010101u, sum_tcn[r][e]) +
-                                  (__dp4a(im_l + im_h, 0x01010101u, 0u) << 16);
-                  const int i_rel = kTileInputs * box + 4 * qd + e, grp = i_rel >> 3;
-                  const int pos = ((i_rel & 7) + (grp & 3)) & 7;
-                  const int zrow = rg.z_row + (rg.interleaved ? 16 * grp : 8 * grp) + pos;
-                  const uint32_t d = z_s + (uint32_t)zrow * 128u + (uint32_t)((j ^ pos) << 4);
-                  sts128(d, re_l, im_l, re_h, im_h);
-                  if (rg.interleaved == 1) sts128_q(d, im_l, nre_l, im_h, nre_h);
-                }
-              }
-            }
-          } else {
-          // operand chunk `sub` of the packed stage (64 of its 128 samples)
+        if (grp < nch) {
+          ++n_mine;
+          const int zm = zs + grp, zi = zm >= p.z_stages ? zm - p.z_stages : zm;
+          const uint32_t zp = zm >= p.z_stages ? zph ^ 1u : zph;
+          if (!mbar_wait(b.z_empty + 8 * zi, zp ^ 1u, abort_flag, to)) { ok = false; break; }
+          const uint32_t pk_s = pk_s0 + (uint32_t)s * p.pk_stage_bytes;
+          const uint32_t z_s = z_s0 + (uint32_t)zi * p.z_stage_bytes;
 #pragma unroll
           for (int r = 0; r < 2; ++r) {
-            if (r >= n_reg) break;
-            const uint32_t src = pk_s + src_off[r] + (sub ? src_sub1 : src_sub0);
-            const uint32_t dst = z_s + dst_off[r];
-            uint4 in0 = make_uint4(0u, 0u, 0u, 0u), in1 = in0;
-            if (n_k[r] > 0) in0 = lds128(src);
-            if (n_k[r] > 1) in1 = lds128(src + R * kPackedRowBytes);
-#pragma unroll
-            for (int kr = 0; kr < 2; ++kr) {
-              if (kr >= n_k[r]) break;
-              const uint4 in = kr == 0 ? in0 : in1;
-              const uint32_t d0 = dst + (kr ? dst_step[r] : 0u) + off0;
-              const uint32_t d1 = dst + (kr ? dst_step[r] : 0u) + off1;
-              uint32_t re0, im0, nre0, re1, im1, nre1, re2, im2, nre2, re3, im3, nre3;
-              decode_biased(in.x, re0, im0, nre0);
-              decode_biased(in.y, re1, im1, nre1);
-              decode_biased(in.z, re2, im2, nre2);
-              decode_biased(in.w, re3, im3, nre3);
-              sts128(d0, re0, im0, re1, im1);
-              sts128(d1, re2, im2, re3, im3);
-              if (il[r]) {  // the Q rows follow 8 rows (1024 bytes) after the A rows
-                sts128_q(d0, im0, nre0, im1, nre1);
-                sts128_q(d1, im2, nre2, im3, nre3);
-              }
-              sum_re[r][kr] = __dp4a(re0 + re1 + re2 + re3, 0x01010101u, sum_re[r][kr]);
-              sum_im[r][kr] = __dp4a(im0 + im1 + im2 + im3, 0x01010101u, sum_im[r][kr]);
-            }
-          }
+            if (n_k[r] == 0) break;
+            if constexpr (TCN)
+              unpack_turned(pk_s + src_off[r], z_s + dst_off[r], kind[r], n_k[r], t_grp, grp,
+                            sums[r]);
+            else if (kind[r] == 1)
+              unpack_rows<true>(pk_s + src_off[r], z_s + dst_off[r], 16384u, n_k[r], sums[r]);
+            else
+              unpack_rows<false>(pk_s + src_off[r], z_s + dst_off[r], dst_step[r], n_k[r], sums[r]);
           }
           fence_proxy_async_smem();
           __syncwarp();
-          if (lane == 0) {
-            mbar_arrive(b.z_full + 8 * zs);
-            if (sub == nch - 1) mbar_arrive(b.pk_empty + 8 * s);
-          }
-          if (++zs == p.z_stages) { zs = 0; zph ^= 1u; }
+          if (lane == 0) mbar_arrive(b.z_full + 8 * zi);
         }
+        if (lane == 0) mbar_arrive(b.pk_empty + 8 * s);
+        if ((zs += nch) >= p.z_stages) { zs -= p.z_stages; zph ^= 1u; }
         if (++s == p.pk_stages) { s = 0; ph ^= 1u; }
       }
-      // ---- the item's operand sums, for the epilogue: entry = (8 (Ua + Ub) -
-      // 64 T, 8 (Ub - Ua)) with Ua, Ub the sums of u over the input's T real
-      // and imaginary parts (zero-filled samples are u = 8, so they cancel)
       if (!ok) break;
+      // ---- the item's operand sums, for the epilogue, added up in a table
+      // that it has cleared: entry = (8 (Ua + Ub) - 64 T, 8 (Ub - Ua)) with
+      // Ua, Ub the sums of u over the input's T real and imaginary parts
+      // (zero-filled samples are u = 8, so they cancel)
       const int sb = (int)(nu & 1);
-      if (!(PAIR ? mbar_wait_cluster(b.sum_empty + 8 * sb, (uint32_t)((nu >> 1) & 1) ^ 1u,
-                                     abort_flag, to)
-                 : mbar_wait(b.sum_empty + 8 * sb, (uint32_t)((nu >> 1) & 1) ^ 1u, abort_flag, to)))
+      const uint32_t sum_ph = (uint32_t)((nu >> 1) & 1) ^ 1u;
+      if (!(PAIR ? mbar_wait_cluster(b.sum_empty + 8 * sb, sum_ph, abort_flag, to)
+                 : mbar_wait(b.sum_empty + 8 * sb, sum_ph, abort_flag, to)))
         break;
       const uint32_t tab = sum_s0 + (uint32_t)sb * sum_tab;
-      if (TCN) {
-        // the two half-warps hold 16 of a chunk's 64 samples of the same
-        // inputs; four warps hold the 64, and add to the cleared table
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          if (r >= n_reg) break;
-          const XRegion rg = u->reg[r];
-          const bool mine = tid < (rg.n_in / kTileInputs) * 128;  // whole warps
+      for (int r = 0; r < 2; ++r) {
+        const int sum_row = u->reg[r < n_reg ? r : 0].sum_row;
 #pragma unroll
-          for (int e = 0; e < 4; ++e) {
-            int ua = (int)(sum_tcn[r][e] & 0xFFFFu), ub = (int)(sum_tcn[r][e] >> 16);
-            ua += __shfl_xor_sync(0xffffffffu, ua, 16);
-            ub += __shfl_xor_sync(0xffffffffu, ub, 16);
-            if (mine && lane < 16) {
-              const int i_rel = kTileInputs * (tid >> 7) + 4 * (tid & 15) + e, grp = i_rel >> 3;
-              const int at = rg.sum_row + 8 * grp + (((i_rel & 7) + (grp & 3)) & 7);
-              reds32(tab + 8u * (uint32_t)at, 8 * (ua + ub) - 64 * 16 * n_chunks);
-              reds32(tab + 8u * (uint32_t)at + 4u, 8 * (ub - ua));
-            }
-          }
-        }
-      } else {
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          const XRegion rg = u->reg[r < n_reg ? r : 0];
-#pragma unroll
-          for (int kr = 0; kr < 2; ++kr) {
-            if (kr >= n_k[r]) break;  // uniform in the warp: its 8 rows lie in one region
-            int ua = (int)sum_re[r][kr], ub = (int)sum_im[r][kr];
+        for (int k = 0; k < (TCN ? 8 : 4); ++k) {
+          // whole warps: an 8-row group, or a quarter of a box, is in or out
+          const int box = TCN ? 2 * (k >> 2) + (t_grp >> 7) : k;
+          if (box >= n_k[r]) continue;
+          int ua = (int)(sums[r][k] & 0xFFFFu), ub = (int)(sums[r][k] >> 16);
+          if (!TCN) {
             ua += __shfl_xor_sync(0xffffffffu, ua, 8);
             ub += __shfl_xor_sync(0xffffffffu, ub, 8);
-            ua += __shfl_xor_sync(0xffffffffu, ua, 16);
-            ub += __shfl_xor_sync(0xffffffffu, ub, 16);
-            if (lane < 8) {
-              const int rr = (r == 1 ? row0 - pack : row0) + R * kr;
-              const uint32_t at =
-                  tab + 8u * (uint32_t)((int)rank * (p.sum_rows >> 1) + rg.sum_row + rr);
-              const uint32_t vx = (uint32_t)(8 * (ua + ub) - 64 * kChunkSamples * n_chunks);
-              const uint32_t vy = (uint32_t)(8 * (ub - ua));
-              sts64(at, vx, vy);
-              if (PAIR) st_cluster_v2(at, rank ^ 1u, vx, vy);
+          }
+          ua += __shfl_xor_sync(0xffffffffu, ua, 16);
+          ub += __shfl_xor_sync(0xffffffffu, ub, 16);
+          // normal order: the warp held all 64 samples of a chunk of 8 rows;
+          // F-engine order: 16 of them (8 a half-warp) of 64 inputs
+          if (lane < (TCN ? 16 : 8)) {
+            int at;
+            if (TCN) {
+              const int i_rel = kTileInputs * box + 4 * (t_grp & 15) + (k & 3), gp = i_rel >> 3;
+              at = 8 * gp + (((i_rel & 7) + (gp & 3)) & 7);  // by operand-row position
+            } else {
+              at = kTileInputs * k + 8 * w8 + sw;
+            }
+            const uint32_t addr =
+                tab + 8u * (uint32_t)((int)rank * (p.sum_rows >> 1) + sum_row + at);
+            const int vx = 8 * (ua + ub) - 64 * (TCN ? 16 : kChunkSamples) * n_mine;
+            const int vy = 8 * (ub - ua);
+            reds32(addr, vx);
+            reds32(addr + 4u, vy);
+            if (PAIR) {
+              red_cluster(addr, rank ^ 1u, vx);
+              red_cluster(addr + 4u, rank ^ 1u, vy);
             }
           }
         }
@@ -670,16 +674,16 @@ __global__ void __launch_bounds__(kThreads, 1)
           mbar_arrive_cluster(b.acc_empty, 0);
         else
           mbar_arrive(b.acc_empty);
-        mbar_arrive(TCN ? b.sum_read + 8 * sb : b.sum_empty + 8 * sb);
-        if (PAIR) mbar_arrive_cluster(b.sum_empty + 8 * sb, rank ^ 1u);
+        mbar_arrive(b.sum_read + 8 * sb);
       }
-      if (TCN) {
-        // every epilogue warp has read the table: clear it for the item after
-        // the next
-        if (!mbar_wait(b.sum_read + 8 * sb, (uint32_t)((nu >> 1) & 1), abort_flag, to)) break;
-        for (int k = q * 32 + lane; k < p.sum_rows; k += 32 * kEpiWarps) sts64(tab + 8u * k, 0u, 0u);
-        __syncwarp();
-        if (lane == 0) mbar_arrive(b.sum_empty + 8 * sb);
+      // once every epilogue warp has read the table it is cleared for the
+      // item after the next
+      if (!mbar_wait(b.sum_read + 8 * sb, (uint32_t)((nu >> 1) & 1), abort_flag, to)) break;
+      for (int k = q * 32 + lane; k < p.sum_rows; k += 32 * kEpiWarps) sts64(tab + 8u * k, 0u, 0u);
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(b.sum_empty + 8 * sb);
+        if (PAIR) mbar_arrive_cluster(b.sum_empty + 8 * sb, rank ^ 1u);
       }
     }
   }

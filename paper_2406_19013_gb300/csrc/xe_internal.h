@@ -13,7 +13,7 @@ constexpr int kChunkSamples = 64;
 // 64 inputs' imaginary-part rows (M = 128).
 constexpr int kTileInputs = 64;
 constexpr int kTmemCols = 512;
-constexpr int kMaxSegs = 8;
+constexpr int kMaxSegs = 6;
 constexpr int kMaxZRows = 512;
 // Samples per TMA box row (one byte per complex sample): a packed stage holds
 // kPkSamples samples of every staged input and feeds kPkSamples /
@@ -21,12 +21,12 @@ constexpr int kMaxZRows = 512;
 constexpr int kPkSamples = 128;
 constexpr int kPackedRowBytes = kPkSamples;
 constexpr int kChunksPerPk = kPkSamples / kChunkSamples;
-// Warp roles (see xengine.cu): unpack, epilogue (one per TMEM lane quarter),
+// Warp roles (see xengine.cu): unpack, epilogue (two per TMEM lane quarter),
 // TMA producer, MMA issuers (one issue stream per accumulator).
 constexpr int kUnpackWarps = 16;
 constexpr int kUnpackGroup = kUnpackWarps / 2;  // warps that decode one chunk
-constexpr int kEpiWarps = 4;
-constexpr int kMmaWarps = 4;
+constexpr int kEpiWarps = 8;
+constexpr int kMmaWarps = 3;
 constexpr int kWarpEpi0 = kUnpackWarps;
 constexpr int kWarpTma = kWarpEpi0 + kEpiWarps;
 constexpr int kWarpMma0 = kWarpTma + 1;
@@ -43,9 +43,8 @@ constexpr int kMaxZStages = 6;
 constexpr int kBarrierBytes = 512;
 // One epilogue warp's buffer: 8 rows of 16 (re, im) int32 pairs.
 constexpr int kEpiBufBytes = 8 * 16 * 8;
-// Two tables of operand sums (the item being folded and the next), an entry
-// of two words per staged input.
-constexpr int kSumBytesPerInput = 2 * 8;
+// The table of operand sums: an entry of two words per staged input.
+constexpr int kSumBytesPerInput = 8;
 // Blocks integrated by one launch before the fold into int64.
 constexpr int kMaxBlocksPerLaunch = 8;
 

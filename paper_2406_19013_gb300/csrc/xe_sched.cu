@@ -255,7 +255,7 @@ bool stage_layout(const std::vector<const std::vector<XUnit> *> &unit_sets, int 
   L.pk_stage_bytes = (uint32_t)round_up(max_pk, 1024);  // swizzled TMA destination
   const int fixed = 1024 /* alignment slack */ + kBarrierBytes + kEpiWarps * kEpiBufBytes +
                     max_sum * kSumBytesPerInput;
-  static_assert(8 * (2 * kMaxPkStages + 2 * kMaxZStages + 2 + kMmaWarps + 1 + 6) + 16 <=
+  static_assert(8 * (2 * kMaxPkStages + 2 * kMaxZStages + 2 + kMmaWarps + 1 + 3) + 16 <=
                     kBarrierBytes,
                 "barrier area");
   const int avail = smem_optin - fixed;
@@ -307,6 +307,7 @@ int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem>
   // operand row costs 1; the fold of a unit costs kFold per accumulator
   // column (its int64 atomic adds and the TMEM drain).
   constexpr long long kFold = 16;
+  constexpr int kChanBand = 8;  // a multiple of every unit's channels
   struct PW {
     int cpb, ppb, npk, nseg;  // nseg: fold-window segments of a unit's stages
   };
@@ -397,11 +398,18 @@ int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem>
   for (size_t p = 0; p < probs.size(); ++p) {
     const long long npk_total = pw[p].npk;
     const int nseg = pw[p].nseg;
-    for (int t = 0; t < (int)probs[p].units->size(); ++t)
-      for (int c = 0; c < probs[p].n_chan; c += std::max(1, (*probs[p].units)[t].n_chan))
-        // fold-window segment sg: stages [npk sg / nseg, npk (sg + 1) / nseg)
-        for (int sg = 0; sg < nseg; ++sg)
-          deal(p, t, c, (int)(npk_total * sg / nseg), (int)(npk_total * (sg + 1) / nseg));
+    // Bands of channels, one template after the other within a band: the
+    // CTAs running at one time then work on the same channels, whose inputs
+    // every template reads again (from L2 instead of HBM), and each template
+    // still runs over a band's channels in turn.
+    for (int c0 = 0; c0 < probs[p].n_chan; c0 += kChanBand)
+      for (int t = 0; t < (int)probs[p].units->size(); ++t) {
+        const int step = std::max(1, (*probs[p].units)[t].n_chan);
+        for (int c = c0; c < std::min(probs[p].n_chan, c0 + kChanBand); c += step)
+          // fold-window segment sg: stages [npk sg / nseg, npk (sg + 1) / nseg)
+          for (int sg = 0; sg < nseg; ++sg)
+            deal(p, t, c, (int)(npk_total * sg / nseg), (int)(npk_total * (sg + 1) / nseg));
+      }
   }
   if (load > 0 || (int)cta_first.size() == 1) close_cta();
   // drop trailing empty CTAs

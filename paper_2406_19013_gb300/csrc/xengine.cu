@@ -20,17 +20,17 @@
 // (times 2^-18) and exact; each item's sums are folded into the int64
 // integration buffer when it ends.
 //
-// Kernel structure (persistent, one CTA per SM, 25 warps):
-//   warp 20     TMA producer: packed bytes [channel][input][time] -> smem ring
+// Kernel structure (persistent, one CTA per SM, 28 warps):
+//   warp 24     TMA producer: packed bytes [channel][input][time] -> smem ring
 //   warps 0-15  unpack: 4-bit nibbles -> E4M3 A/Q rows in the 128B-swizzled
 //               K-major layout the MMA reads (the paper's CPU "fluff" step,
 //               Sec. 2.3, moved on chip)
-//   warps 21-24 MMA issuers: tcgen05.mma M=128 (64 inputs' A rows + Q rows),
+//   warps 25-27 MMA issuers: tcgen05.mma M=128 (64 inputs' A rows + Q rows),
 //               N = columns of the triangle strip, K = 32 per instruction;
 //               one issuing thread per accumulator, because a single thread
 //               issues an MMA only every ~110-126 cycles in a loop with
 //               waits and commits, too slow for the N = 64 strips alone
-//   warps 16-19 epilogue: tcgen05.ld of the fp32 accumulators, bias out,
+//   warps 16-23 epilogue: tcgen05.ld of the fp32 accumulators, bias out,
 //               rows regrouped through a small buffer, int64 red.add into the
 //               lower triangle (256 contiguous bytes an instruction)
 // A launch integrates up to kMaxBlocksPerLaunch blocks; the host cuts its
@@ -64,8 +64,8 @@ namespace {
 
 struct Bars {
   uint32_t pk_full, pk_empty, z_full, z_empty, acc_full, acc_empty, drain, never;
-  // the two tables of operand sums: written by the unpack warps, read by the
-  // epilogue, and (F-engine order) read by all of it and not yet cleared
+  // the table of operand sums: complete (unpack warps), cleared (epilogue),
+  // and read by every epilogue warp
   uint32_t sum_full, sum_empty, sum_read;
 };
 
@@ -84,10 +84,25 @@ __device__ __forceinline__ XItem item_at(const XParams &p, int it) {
   return r;
 }
 
-// Chunks (of kChunkSamples) in packed stage kc of a block.
-__device__ __forceinline__ int chunks_in_pk(const XProb &pb, int kc) {
-  return min(kChunksPerPk, pb.chunks_per_block - kChunksPerPk * kc);
-}
+// Walks the packed stages of an item through its blocks: stage kc of the
+// block (a division once per item instead of one per stage and role).
+struct StageWalk {
+  int kc, pk_per_block, last;  // last: chunks in a block's last stage
+  __device__ __forceinline__ StageWalk(const XProb &pb, int pk0)
+      : kc(pk0 % pb.pk_per_block),
+        pk_per_block(pb.pk_per_block),
+        last(pb.chunks_per_block - kChunksPerPk * (pb.pk_per_block - 1)) {}
+  // chunks (of kChunkSamples) in this stage
+  __device__ __forceinline__ int chunks() const {
+    return kc == pk_per_block - 1 ? last : kChunksPerPk;
+  }
+  // to the next stage; true if it is the first of the next block
+  __device__ __forceinline__ bool next() {
+    if (++kc < pk_per_block) return false;
+    kc = 0;
+    return true;
+  }
+};
 
 // Decodes this warp's rows of one chunk of a staged region: n_k groups of 8
 // rows, 64 rows apart.  `src` and `dst` are the lane's addresses in the first
@@ -164,7 +179,20 @@ __device__ __forceinline__ void unpack_turned(uint32_t src, uint32_t dst, int ki
     }
   }
 }
-// kThreads = 32 * 25: warps 0-15 unpack, 16-19 epilogue, 20 TMA, 21-24 MMA.
+// A folded value from an accumulator (in units of 2^-18) and the sum of its
+// operand-sum entries, given plus kMagicBits: acc 2^18 - 8 sum, returned plus
+// kMagicBits.  1.5 x 2^23 has a unit of 1, so adding a whole number below 2^22
+// to its bits or to its value is the same thing; the entries stay below 2^20,
+// folded values within 128 x 32768 = 2^22, and all steps are exact.  (Four
+// quick operations; the conversion instruction takes eight cycles a warp.)
+constexpr uint32_t kMagicBits = 0x4B400000u;  // 1.5 x 2^23
+__device__ __forceinline__ uint32_t unbias(uint32_t acc, uint32_t sum_magic) {
+  constexpr float kMagic = 12582912.0f;
+  const float bias = fmaf(__uint_as_float(sum_magic), -8.0f, 8.0f * kMagic);
+  return __float_as_uint(fmaf(__uint_as_float(acc), 262144.0f, bias) + kMagic);
+}
+
+// kThreads = 32 * 28: warps 0-15 unpack, 16-23 epilogue, 24 TMA, 25-27 MMA.
 // Every role walks the same item list, [cta_first[b], cta_first[b + 1]).
 // TCN: the blocks are in F-engine order (XParams::tcn), staged and unpacked
 // by the transposing path; a compile-time choice, so that the X-engine-order
@@ -184,11 +212,11 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint64_t *bar_mem = reinterpret_cast<uint64_t *>(pk_buf + (size_t)p.pk_stages * p.pk_stage_bytes);
   // [pk_full x S][pk_empty x S][z_full x Z][z_empty x Z][acc_full][acc_empty][drain x kMmaWarps]
   // [never]: only waited on by the failure-detection self-test
-  // [sum_full x 2][sum_empty x 2][sum_read x 2]
+  // [sum_full][sum_empty][sum_read]
   uint32_t *misc = reinterpret_cast<uint32_t *>(bar_mem + 2 * p.pk_stages + 2 * p.z_stages + 2 +
-                                                kMmaWarps + 1 + 6);
-  // behind the barrier area: the epilogue warps' buffers, then the two tables
-  // of operand sums (p.sum_rows entries of 8 bytes each)
+                                                kMmaWarps + 1 + 3);
+  // behind the barrier area: the epilogue warps' buffers, then the table of
+  // operand sums (p.sum_rows entries of 8 bytes)
   uint8_t *epi_mem = reinterpret_cast<uint8_t *>(bar_mem) + kBarrierBytes;
   uint8_t *sum_mem = epi_mem + kEpiWarps * kEpiBufBytes;
   volatile int *abort_flag = reinterpret_cast<volatile int *>(misc + 1);
@@ -203,9 +231,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   b.drain = b.acc_empty + 8;
   b.never = b.drain + 8 * kMmaWarps;
   b.sum_full = b.never + 8;
-  b.sum_empty = b.sum_full + 16;
-  b.sum_read = b.sum_empty + 16;
-  const uint32_t sum_s0 = smem_u32(sum_mem), sum_tab = (uint32_t)p.sum_rows * 8u;
+  b.sum_empty = b.sum_full + 8;
+  b.sum_read = b.sum_empty + 8;
+  const uint32_t tab = smem_u32(sum_mem);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
@@ -223,16 +251,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     mbar_init(b.acc_empty, PAIR ? 2 * kEpiWarps : kEpiWarps);
     for (int m = 0; m < kMmaWarps; ++m) mbar_init(b.drain + 8 * m, 1);
     mbar_init(b.never, 1);  // nothing ever arrives here
-    for (int k = 0; k < 2; ++k) {
-      mbar_init(b.sum_full + 8 * k, (PAIR ? 2 : 1) * kUnpackWarps);
-      mbar_init(b.sum_empty + 8 * k, (PAIR ? 2 : 1) * kEpiWarps);
-      mbar_init(b.sum_read + 8 * k, kEpiWarps);
-    }
+    mbar_init(b.sum_full, (PAIR ? 2 : 1) * kUnpackWarps);
+    mbar_init(b.sum_empty, (PAIR ? 2 : 1) * kEpiWarps);
+    mbar_init(b.sum_read, kEpiWarps);
     *abort_flag = 0;
     fence_mbar_init();
   }
-  // the unpack warps add to the tables of operand sums, starting from zero
-  for (int k = threadIdx.x; k < 4 * p.sum_rows; k += kThreads)
+  // the unpack warps add to the table of operand sums, starting from zero
+  for (int k = threadIdx.x; k < 2 * p.sum_rows; k += kThreads)
     reinterpret_cast<uint32_t *>(sum_mem)[k] = 0u;
   if (warp == kWarpMma0) {
     if (PAIR) {
@@ -282,9 +308,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         const XUnit *u = pb.units + item.tpl;
         const int n_reg = u->n_reg;
         const uint32_t bytes = (uint32_t)u->pk_bytes;
-        for (int k = item.pk0; k < item.pk0 + item.npk; ++k) {
-          const int blk = k / pb.pk_per_block, kc = k - blk * pb.pk_per_block;
-          const int mi = pb.map0 + blk;
+        StageWalk walk(pb, item.pk0);
+        int mi = pb.map0 + item.pk0 / pb.pk_per_block;
+        for (int k = 0; k < item.npk; ++k) {
+          const int kc = walk.kc;
           const void *tmap = &maps.m[mi][0];
           if (mi != last_map) { prefetch_tmap(tmap); last_map = mi; }
           if (!mbar_wait(b.pk_empty + 8 * s, ph ^ 1u, abort_flag, to)) { ok = false; break; }
@@ -306,6 +333,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                             in_lo + bx, ch);
             }
           }
+          if (walk.next()) ++mi;
           if (++s == p.pk_stages) { s = 0; ph ^= 1u; }
         }
       }
@@ -331,7 +359,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const XProb pb = p.probs[item.prob];
         const XUnit *u = pb.units + item.tpl;
         const int n_seg = u->n_seg;
-        static_assert(kMaxSegs / kMmaWarps == 2, "two segments per issuer at most");
+        static_assert(kMaxSegs == 2 * kMmaWarps, "two segments per issuer at most");
         // The (at most two) segments this issuer owns.  Their descriptors are
         // built once per item, for Z stage 0 and K slice 0, as 32-bit words:
         // a chunk in Z stage zs and K slice kk only adds (zs z_stage_bytes +
@@ -357,8 +385,9 @@ __global__ void __launch_bounds__(kThreads, 1)
           break;
         tc_fence_after();
         uint32_t acc0 = 0;  // the item's first MMA of each accumulator overwrites it
-        for (int k = item.pk0; k < item.pk0 + item.npk && ok; ++k) {
-          const int nch = chunks_in_pk(pb, k % pb.pk_per_block);
+        StageWalk walk(pb, item.pk0);
+        for (int k = 0; k < item.npk && ok; ++k, walk.next()) {
+          const int nch = walk.chunks();
           for (int sub = 0; sub < nch; ++sub) {
             if (!(PAIR ? mbar_wait_cluster(b.z_full + 8 * zs, zph, abort_flag, to)
                        : mbar_wait(b.z_full + 8 * zs, zph, abort_flag, to))) {
@@ -416,8 +445,9 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int it = it0; it < it1 && ok && !*abort_flag; it += it_step) {
         const XItem item = item_at(p, it);
         const XProb pb = p.probs[item.prob];
-        for (int k = item.pk0; k < item.pk0 + item.npk && ok; ++k) {
-          const int nch = chunks_in_pk(pb, k % pb.pk_per_block);
+        StageWalk walk(pb, item.pk0);
+        for (int k = 0; k < item.npk && ok; ++k, walk.next()) {
+          const int nch = walk.chunks();
           for (int sub = 0; sub < nch; ++sub) {
             if (!mbar_wait(b.z_full + 8 * zs, zph, abort_flag, to)) { ok = false; break; }
             mbar_arrive_cluster(b.z_full + 8 * zs, 0);
@@ -480,8 +510,9 @@ __global__ void __launch_bounds__(kThreads, 1)
         dst_off[r] = (uint32_t)rg.z_row * 128u +
                      (TCN ? 0u : (uint32_t)w8 * (dst_step[r] / kUnpackGroup) + dst_lane);
       }
-      for (int k = item.pk0; k < item.pk0 + item.npk; ++k) {
-        const int nch = chunks_in_pk(pb, k % pb.pk_per_block);
+      StageWalk walk(pb, item.pk0);
+      for (int k = 0; k < item.npk; ++k, walk.next()) {
+        const int nch = walk.chunks();
         if (!mbar_wait(b.pk_full + 8 * s, ph, abort_flag, to)) { ok = false; break; }
         if (grp < nch) {
           ++n_mine;
@@ -503,23 +534,25 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           fence_proxy_async_smem();
           __syncwarp();
-          if (lane == 0) mbar_arrive(b.z_full + 8 * zi);
+          if (lane == 0) {
+            mbar_arrive(b.z_full + 8 * zi);
+            mbar_arrive(b.pk_empty + 8 * s);
+          }
+        } else if (lane == 0) {
+          mbar_arrive(b.pk_empty + 8 * s);  // a block's odd last chunk
         }
-        if (lane == 0) mbar_arrive(b.pk_empty + 8 * s);
         if ((zs += nch) >= p.z_stages) { zs -= p.z_stages; zph ^= 1u; }
         if (++s == p.pk_stages) { s = 0; ph ^= 1u; }
       }
       if (!ok) break;
       // ---- the item's operand sums, for the epilogue, added up in a table
-      // that it has cleared: entry = (8 (Ua + Ub) - 64 T, 8 (Ub - Ua)) with
-      // Ua, Ub the sums of u over the input's T real and imaginary parts
-      // (zero-filled samples are u = 8, so they cancel)
-      const int sb = (int)(nu & 1);
-      const uint32_t sum_ph = (uint32_t)((nu >> 1) & 1) ^ 1u;
-      if (!(PAIR ? mbar_wait_cluster(b.sum_empty + 8 * sb, sum_ph, abort_flag, to)
-                 : mbar_wait(b.sum_empty + 8 * sb, sum_ph, abort_flag, to)))
+      // that it has cleared: entry = (Ua + Ub - 8 T, Ub - Ua) with Ua, Ub the
+      // sums of u over the input's T real and imaginary parts (zero-filled
+      // samples are u = 8, so they cancel)
+      const uint32_t sum_ph = (uint32_t)(nu & 1) ^ 1u;
+      if (!(PAIR ? mbar_wait_cluster(b.sum_empty, sum_ph, abort_flag, to)
+                 : mbar_wait(b.sum_empty, sum_ph, abort_flag, to)))
         break;
-      const uint32_t tab = sum_s0 + (uint32_t)sb * sum_tab;
 #pragma unroll
       for (int r = 0; r < 2; ++r) {
         const int sum_row = u->reg[r < n_reg ? r : 0].sum_row;
@@ -547,8 +580,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             const uint32_t addr =
                 tab + 8u * (uint32_t)((int)rank * (p.sum_rows >> 1) + sum_row + at);
-            const int vx = 8 * (ua + ub) - 64 * (TCN ? 16 : kChunkSamples) * n_mine;
-            const int vy = 8 * (ub - ua);
+            const int vx = ua + ub - 8 * (TCN ? 16 : kChunkSamples) * n_mine;
+            const int vy = ub - ua;
             reds32(addr, vx);
             reds32(addr + 4u, vy);
             if (PAIR) {
@@ -560,21 +593,21 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       __syncwarp();
       if (lane == 0) {
-        mbar_arrive(b.sum_full + 8 * sb);
-        if (PAIR) mbar_arrive_cluster(b.sum_full + 8 * sb, rank ^ 1u);
+        mbar_arrive(b.sum_full);
+        if (PAIR) mbar_arrive_cluster(b.sum_full, rank ^ 1u);
       }
     }
   } else if (warp < kWarpTma) {
     // ------------------------------------------------------------ epilogue
     // The warp's TMEM lane quarter holds 16 inputs, each a real row and, 8
-    // lanes on, an imaginary one.  Two 16-lane loads bring 16 columns of 8
-    // inputs each, a thread getting both parts of two columns of one input:
-    // the bias comes off there, and the 8 x 16 complex values go through a
-    // 1 KB buffer so that each atomic instruction adds 256 contiguous bytes
+    // lanes on, an imaginary one; each of the quarter's two warps folds 8 of
+    // them.  A 16-lane load brings 16 columns of the 8 inputs, a thread
+    // getting both parts of two column pairs of one input: the bias comes off
+    // there, and the 8 x 16 complex values go through a 1 KB buffer so that each atomic instruction adds 256 contiguous bytes
     // of one row of the integration buffer.  (Lane-per-row adds, 32 rows an
     // instruction, made four times the memory requests: the fold of a
     // 192-input channel took 31 us.)
-    const int q = warp & 3;
+    const int q = warp & 3, h = (warp - kWarpEpi0) >> 2;
     const uint32_t ebuf = smem_u32(epi_mem) + (uint32_t)(warp - kWarpEpi0) * kEpiBufBytes;
     const int er = lane >> 2, ec = lane & 3;  // the thread's row and column pair as loaded
     // 16-byte chunk (4 k + ec) of buffer row er, swizzled by the row's parity
@@ -597,73 +630,85 @@ __global__ void __launch_bounds__(kThreads, 1)
       // integration is void and is reported as such
       if (*abort_flag) break;
       tc_fence_after();
-      const int sb = (int)(nu & 1);
-      if (!(PAIR ? mbar_wait_cluster(b.sum_full + 8 * sb, (uint32_t)((nu >> 1) & 1), abort_flag, to)
-                 : mbar_wait(b.sum_full + 8 * sb, (uint32_t)((nu >> 1) & 1), abort_flag, to)))
+      if (!(PAIR ? mbar_wait_cluster(b.sum_full, (uint32_t)(nu & 1), abort_flag, to)
+                 : mbar_wait(b.sum_full, (uint32_t)(nu & 1), abort_flag, to)))
         break;
-      const uint32_t tab = sum_s0 + (uint32_t)sb * sum_tab;
       const uint32_t rank_off = PAIR ? (uint32_t)(p.sum_rows >> 1) * 8u : 0u;
       const long long acc_elems = (long long)pb.n_chan * pb.n_pairs * 2;
       const int n_seg = u->n_seg;
       for (int sg = 0; sg < n_seg; ++sg) {
         const XSeg sgm = u->seg[sg];
         const int rpc = sgm.ch_rows;
-#pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-          // 8 inputs: group g of the tile.  In F-engine-order launches group
-          // position l holds input (l - g) % 8 of the group, and column 8 G +
-          // e the one at (e - G) % 8 (a row tile or column range starts at a
-          // multiple of 64 inputs, so only g % 4 and G % 4 matter).
-          const int g = 2 * q + h;
-          const int i_tile = (rank ? sgm.row_in1 : sgm.row_in0) + 8 * g;
-          // a tile of several channels: the 8 rows belong to channel block ci
-          const int ci = rpc ? i_tile / rpc : 0;
-          const int c = item.chan + sgm.chan_off + ci;
-          if (c >= pb.n_chan) continue;  // a multi-channel unit's missing last channels
-          const int i0 = i_tile - ci * rpc;
-          if (i0 >= pb.n_in) continue;
-          int64_t *cacc = pb.acc + (long long)c * pb.n_pairs * 2;
-          // the row's sums: the thread's row as loaded
-          uint32_t p_i, m_i;
-          lds64(tab + (rank ? rank_off : 0u) + 8u * (uint32_t)(sgm.a_sum + 8 * g + er), p_i, m_i);
-          for (int cb = 0; cb < sgm.n; cb += 16) {
-            // input of the first column, the block's columns being 16 inputs
-            // of one channel block
-            int j0 = sgm.col_blk[cb >> 6] + (cb & 63);
-            if (rpc) {
-              if (j0 / rpc != ci) continue;
-              j0 -= ci * rpc;
-            }
-            if (j0 > i0 + 7) continue;  // above the diagonal (uniform)
-            uint32_t v[8];
-            __syncwarp();
-            tmem_ld_16x256b_x2(tmem + ((uint32_t)(32 * q + 16 * h) << 16) +
-                                   (uint32_t)(sgm.tmem_col + cb), v);
-            // the two column pairs' sums: of a pair's columns, the first half
-            // is the even CTA's rows, the second the odd one's
-            const int hc = PAIR && cb >= (sgm.n >> 1) ? 1 : 0;
-            const uint32_t cs = tab + (hc ? rank_off : 0u) +
-                                8u * (uint32_t)(sgm.b_sum + cb - hc * (sgm.n >> 1) + 2 * ec);
-            const uint4 s0 = lds128(cs), s1 = lds128(cs + 64u);
-            tmem_ld_wait();
-            // back to whole numbers: accumulators are in units of 2^-18
-            auto whole = [](uint32_t x) { return (uint32_t)__float2int_rn(__uint_as_float(x) * 262144.0f); };
-            sts128(est0, whole(v[0]) - p_i - s0.x, whole(v[2]) - m_i + s0.y,
-                   whole(v[1]) - p_i - s0.z, whole(v[3]) - m_i + s0.w);
-            sts128(est1, whole(v[4]) - p_i - s1.x, whole(v[6]) - m_i + s1.y,
-                   whole(v[5]) - p_i - s1.z, whole(v[7]) - m_i + s1.w);
-            __syncwarp();
-            // lane w adds word w of each row: column w / 2, part w % 2
-            const int jc = lane >> 1;
-            const int j = TCN ? j0 + (jc & 8) + (((jc & 7) - (((cb + jc) >> 3) & 3)) & 7) : j0 + jc;
+        // 8 inputs: group g of the tile.  In F-engine-order launches group
+        // position l holds input (l - g) % 8 of the group, and column 8 G +
+        // e the one at (e - G) % 8 (a row tile or column range starts at a
+        // multiple of 64 inputs, so only g % 4 and G % 4 matter).
+        const int g = 2 * q + h;
+        const int i_tile = (rank ? sgm.row_in1 : sgm.row_in0) + 8 * g;
+        // a tile of several channels: the 8 rows belong to channel block ci
+        const int ci = rpc ? i_tile / rpc : 0;
+        const int c = item.chan + sgm.chan_off + ci;
+        if (c >= pb.n_chan) continue;  // a multi-channel unit's missing last channels
+        const int i0 = i_tile - ci * rpc;
+        if (i0 >= pb.n_in) continue;
+        int64_t *cacc = pb.acc + (long long)c * pb.n_pairs * 2;
+        // the row's sums: the thread's row as loaded
+        uint32_t p_i, m_i;
+        lds64(tab + (rank ? rank_off : 0u) + 8u * (uint32_t)(sgm.a_sum + 8 * g + er), p_i, m_i);
+        p_i += kMagicBits;
+        m_i += kMagicBits;
+        // the columns to fold: up to the 16 that hold the 8 rows' diagonal,
+        // and of a multi-channel tile the rows' channel block only.  Column
+        // blocks of a pair's segment are not in input order: all of them.
+        const int cb0 = rpc ? ci * rpc : 0;
+        int cb1 = rpc ? cb0 + rpc : sgm.n;
+        if (!PAIR) cb1 = min(cb1, cb0 + ((i0 + 7 - (sgm.col_blk[0] + cb0 - ci * rpc)) & ~15) + 16);
+        const uint32_t tm = tmem + ((uint32_t)(32 * q + 16 * h) << 16) + (uint32_t)sgm.tmem_col;
+        uint32_t nxt[8];
+        __syncwarp();
+        tmem_ld_16x256b_x2(tm + (uint32_t)cb0, nxt);
+        for (int cb = cb0; cb < cb1; cb += 16) {
+          tmem_ld_wait();
+          uint32_t v[8];
 #pragma unroll
-            for (int r = 0; r < 8; ++r) {
-              const int x = (int)lds32((r & 1 ? eld1 : eld0) + (uint32_t)(r * 128));
-              const int i = i0 + (TCN ? ((r - (g & 3)) & 7) : r);
-              if (i < pb.n_in && j <= i)
-                acc_add(pb.acc, acc_elems, p.status,
-                        cacc + (long long)i * (i + 1) + 2 * j + (lane & 1), x);
-            }
+          for (int k = 0; k < 8; ++k) v[k] = nxt[k];
+          // the next columns are on their way while these are folded
+          if (cb + 16 < cb1) tmem_ld_16x256b_x2(tm + (uint32_t)(cb + 16), nxt);
+          // input of the first column (one-CTA units: consecutive inputs)
+          int j0 = sgm.col_blk[0] - ci * rpc + cb;
+          if (PAIR) {
+            if (cb >= 64) j0 = sgm.col_blk[1] + cb - 64;
+            if (cb >= 128) j0 = sgm.col_blk[2] + cb - 128;
+            if (cb >= 192) j0 = sgm.col_blk[3] + cb - 192;
+            if (j0 > i0 + 7) continue;  // above the diagonal (uniform)
+          }
+          // the two column pairs' sums: of a pair's columns, the first half
+          // is the even CTA's rows, the second the odd one's
+          const int hc = PAIR && cb >= (sgm.n >> 1) ? 1 : 0;
+          const uint32_t cs = tab + (hc ? rank_off : 0u) +
+                              8u * (uint32_t)(sgm.b_sum + cb - hc * (sgm.n >> 1) + 2 * ec);
+          const uint4 s0 = lds128(cs), s1 = lds128(cs + 64u);
+          __syncwarp();  // the buffer's last values have been read
+          sts128(est0, unbias(v[0], p_i + s0.x), unbias(v[2], m_i - s0.y),
+                 unbias(v[1], p_i + s0.z), unbias(v[3], m_i - s0.w));
+          sts128(est1, unbias(v[4], p_i + s1.x), unbias(v[6], m_i - s1.y),
+                 unbias(v[5], p_i + s1.z), unbias(v[7], m_i - s1.w));
+          __syncwarp();
+          // lane w adds word w of each row: column w / 2, part w % 2
+          const int jc = lane >> 1;
+          const int j = TCN ? j0 + (jc & 8) + (((jc & 7) - (((cb + jc) >> 3) & 3)) & 7) : j0 + jc;
+          int x[8];
+#pragma unroll
+          for (int r = 0; r < 8; ++r)
+            x[r] = (int)(lds32((r & 1 ? eld1 : eld0) + (uint32_t)(r * 128)) - kMagicBits);
+          // away from the diagonal and the last input every word counts
+          const bool inside = j0 + 15 <= i0 && i0 + 7 < pb.n_in;
+#pragma unroll
+          for (int r = 0; r < 8; ++r) {
+            const int i = i0 + (TCN ? ((r - (g & 3)) & 7) : r);
+            if (inside || (i < pb.n_in && j <= i))
+              acc_add(pb.acc, acc_elems, p.status,
+                      cacc + (i * (i + 1) + 2 * j + (lane & 1)), x[r]);
           }
         }
       }
@@ -674,16 +719,17 @@ __global__ void __launch_bounds__(kThreads, 1)
           mbar_arrive_cluster(b.acc_empty, 0);
         else
           mbar_arrive(b.acc_empty);
-        mbar_arrive(b.sum_read + 8 * sb);
+        mbar_arrive(b.sum_read);
       }
       // once every epilogue warp has read the table it is cleared for the
-      // item after the next
-      if (!mbar_wait(b.sum_read + 8 * sb, (uint32_t)((nu >> 1) & 1), abort_flag, to)) break;
-      for (int k = q * 32 + lane; k < p.sum_rows; k += 32 * kEpiWarps) sts64(tab + 8u * k, 0u, 0u);
+      // next item
+      if (!mbar_wait(b.sum_read, (uint32_t)(nu & 1), abort_flag, to)) break;
+      for (int k = 32 * (warp - kWarpEpi0) + lane; k < p.sum_rows; k += 32 * kEpiWarps)
+        sts64(tab + 8u * k, 0u, 0u);
       __syncwarp();
       if (lane == 0) {
-        mbar_arrive(b.sum_empty + 8 * sb);
-        if (PAIR) mbar_arrive_cluster(b.sum_empty + 8 * sb, rank ^ 1u);
+        mbar_arrive(b.sum_empty);
+        if (PAIR) mbar_arrive_cluster(b.sum_empty, rank ^ 1u);
       }
     }
   }

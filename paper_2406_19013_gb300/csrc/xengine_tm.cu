@@ -41,8 +41,11 @@ namespace xe {
 
 namespace {
 
+// warps: unpack as in xengine.cu, four epilogue warps, TMA, MMA issuers
+constexpr int kTmEpiWarps = 4;
+constexpr int kTmWarpTma = kWarpEpi0 + kTmEpiWarps;
 constexpr int kTmMmaWarps = 3;
-constexpr int kTmWarpMma0 = kWarpTma + 1;
+constexpr int kTmWarpMma0 = kTmWarpTma + 1;
 constexpr int kTmThreads = 32 * (kTmWarpMma0 + kTmMmaWarps);
 static_assert(kTmThreads == 768, "24 warps");
 
@@ -98,7 +101,7 @@ __global__ void __launch_bounds__(kTmThreads, 1)
       mbar_init(b.z_empty + 8 * s, kTmMmaWarps);
     }
     mbar_init(b.acc_full, kTmMmaWarps);
-    mbar_init(b.acc_empty, kEpiWarps);
+    mbar_init(b.acc_empty, kTmEpiWarps);
     for (int m = 0; m < kTmMmaWarps; ++m) mbar_init(b.drain + 8 * m, 1);
     mbar_init(b.never, 1);  // nothing ever arrives here
     *abort_flag = 0;
@@ -128,7 +131,7 @@ __global__ void __launch_bounds__(kTmThreads, 1)
   const long long acc_elems = (long long)pb.n_chan * pb.n_pairs * 2;
   const int n_st = kTileInputs * G.n_rt;  // staged inputs
 
-  if (warp == kWarpTma) {
+  if (warp == kTmWarpTma) {
     // ------------------------------------------------------------ producer
     if (lane == 0) {
       int s = 0;
@@ -331,7 +334,7 @@ __global__ void __launch_bounds__(kTmThreads, 1)
         if (++s == p.pk_stages) { s = 0; ph ^= 1u; }
       }
     }
-  } else if (warp < kWarpTma) {
+  } else if (warp < kTmWarpTma) {
     // ------------------------------------------------------------ epilogue
     const int q = warp & 3;  // TMEM lane quarter this warp may access
     const int rho = 32 * q + lane;

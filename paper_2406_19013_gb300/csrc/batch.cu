@@ -391,9 +391,9 @@ int corr_batch_create(int n_inst, const int *n_ant, const int *n_pol, const int 
   std::vector<std::vector<xe::XUnit>> units(n_inst);
   std::map<std::pair<uint32_t, uint32_t>, std::vector<int>> by_layout;
   for (int k = 0; k < n_inst; ++k) {
-    // above 256 inputs the pairs cover runs in its CTA-pair form
-    units[k] = xe::build_schedule(b->inst[k].n_in,
-                                  b->inst[k].n_in > 256 ? xe::kCoverQuads : b->inst[k].cover);
+    // the pairs cover of the largest arrays runs in its CTA-pair form
+    units[k] = xe::build_schedule(
+        b->inst[k].n_in, b->inst[k].n_in > xe::kPairInputs ? xe::kCoverQuads : b->inst[k].cover);
     xe::StageLayout L;
     if (units[k].empty() || !xe::stage_layout({&units[k]}, optin, xe::kMaxZStages, &L)) {
       free_batch(b);

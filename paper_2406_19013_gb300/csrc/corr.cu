@@ -118,15 +118,13 @@ bool use_tm_kernel(int n_in) {
   return e && std::strcmp(e, "tm") == 0;
 }
 
-// Whether CTA pairs run a context of n_in inputs: above 256 inputs, unless
-// CORR_CMAC_KERNEL=smem asks for one-CTA units.  The pair's shared B operand
-// halves the inputs each SM unpacks per MMA: 2048 inputs, 32 channels, 4
-// blocks of 4096 samples 4.70 ms against 4.97 ms on one-CTA units; up to 256
-// inputs one window unit per channel is the smaller cover.
+// Whether CTA pairs run a context of n_in inputs (more than 256 only): above
+// kPairInputs, unless CORR_CMAC_KERNEL asks for pairs or for one-CTA units.
 bool use_pair_kernel(int n_in) {
   if (n_in <= 256) return false;
   const char *e = std::getenv("CORR_CMAC_KERNEL");
-  return !e || std::strcmp(e, "smem") != 0;
+  if (e && std::strcmp(e, "pair") == 0) return true;
+  return n_in > xe::kPairInputs && !(e && std::strcmp(e, "smem") == 0);
 }
 
 // Shared-memory stages of the TMEM-operand kernel for n_in inputs: operand

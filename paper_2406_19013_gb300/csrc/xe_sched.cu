@@ -7,6 +7,9 @@
 
 #include <algorithm>
 #include <cstring>
+#include <functional>
+#include <queue>
+#include <utility>
 
 namespace xe {
 
@@ -299,15 +302,23 @@ bool stage_layout(const std::vector<const std::vector<XUnit> *> &unit_sets, int 
   return true;
 }
 
+// Cycles of one 64-sample chunk of a unit: its MMAs (four K slices of each
+// segment; measured on shared-memory operands, 57 cycles at N = 64, 122 at
+// 192, 155 at 256, and 182 for a CTA pair's M = 256, N = 256), or the unpack of
+// its operand rows (960 cycles for 384 rows) if that takes longer.
+static int chunk_cost(const XUnit &u) {
+  int mma = 0;
+  for (int s = 0; s < u.n_seg; ++s) mma += 4 * ((u.pair_rows ? 54 : 24) + u.seg[s].n / 2);
+  return std::max(mma, 5 * u.z_rows / 2);
+}
+
 int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem> &items,
                 std::vector<int> &cta_first, int min_split_pk, int max_item_pk) {
   items.clear();
   cta_first.clear();
-  // Cost model, in operand-row chunks: unpacking one 64-sample chunk of one
-  // operand row costs 1; the fold of a unit costs kFold per accumulator
-  // column (its int64 atomic adds and the TMEM drain).
-  constexpr long long kFold = 16;
-  constexpr int kChanBand = 8;  // a multiple of every unit's channels
+  // Cost model, in SM cycles: chunk_cost per 64-sample chunk of a unit, and
+  // kFold per accumulator column for its fold.
+  constexpr long long kFold = 50;
   struct PW {
     int cpb, ppb, npk, nseg;  // nseg: fold-window segments of a unit's stages
   };
@@ -322,21 +333,73 @@ int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem>
     pw[p].nseg = (pw[p].npk + max_item_pk - 1) / max_item_pk;
     for (const XUnit &u : *pr.units)
       total += (long long)((pr.n_chan + u.n_chan - 1) / u.n_chan) *
-               ((long long)pw[p].cpb * pr.n_blocks * u.z_rows + kFold * u.work * pw[p].nseg);
+               ((long long)pw[p].cpb * pr.n_blocks * chunk_cost(u) + kFold * u.work * pw[p].nseg);
   }
   if (total == 0 || grid <= 0) {
     cta_first.push_back(0);
     return 0;
   }
-  // cost of stages [a, b) of a unit with z_rows rows
-  auto range_cost = [&](size_t p, int a, int b, int z_rows) {
+  // cost of stages [a, b) of a unit that costs `per_chunk` a chunk
+  auto range_cost = [&](size_t p, int a, int b, int per_chunk) {
     long long chunks = 0;
     for (int k = a; k < b; ++k) {
       const int kc = k % pw[p].ppb;
       chunks += std::min(kChunksPerPk, pw[p].cpb - kChunksPerPk * kc);
     }
-    return chunks * z_rows;
+    return chunks * per_chunk;
   };
+  // More than two templates per channel: they read the same inputs, so the units of
+  // one channel run at the same time and the inputs come from L2 (2048
+  // inputs: contiguous runs spread the CTAs over all channels, and the loads
+  // alone, from HBM, took 4.6 of 4.7 ms against 3.0 ms from L2).  Units go
+  // channel by channel to the CTA that is free first; one that would overrun
+  // the mean load is cut there.
+  bool shared_inputs = false;
+  for (const ProbWork &pr : probs) shared_inputs = shared_inputs || pr.units->size() > 2;
+  if (shared_inputs) {
+    std::vector<std::vector<XItem>> runs(grid);
+    typedef std::pair<long long, int> Load;  // modelled cost so far, CTA
+    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> free_first;
+    for (int k = 0; k < grid; ++k) free_first.push({0, k});
+    auto deal_next = [&](size_t p, int t, int c, int pk, int npk) {
+      const XUnit &u = (*probs[p].units)[t];
+      const long long fold = kFold * u.work, per = (long long)kChunksPerPk * chunk_cost(u);
+      while (pk < npk) {
+        const Load l = free_first.top();
+        free_first.pop();
+        const long long room = (total + grid - 1) / grid - l.first - fold;
+        int n = npk - pk;
+        if (per * n > room) {
+          const int fit = (int)std::max<long long>(0, room / per);
+          if (fit >= min_split_pk && n - fit >= min_split_pk) {
+            n = fit;
+            total += fold;  // the rest of the unit is folded once more
+          }
+        }
+        runs[l.second].push_back({(int)p, t, c, pk, n});
+        free_first.push({l.first + per * n + fold, l.second});
+        pk += n;
+      }
+    };
+    for (size_t p = 0; p < probs.size(); ++p) {
+      const std::vector<XUnit> &us = *probs[p].units;
+      const long long npk_total = pw[p].npk;
+      const int nseg = pw[p].nseg;
+      int step = 1;  // channels of a unit (the same for all templates)
+      for (const XUnit &u : us) step = std::max(step, u.n_chan);
+      for (int c = 0; c < probs[p].n_chan; c += step)
+        for (int sg = 0; sg < nseg; ++sg)
+          for (int t = 0; t < (int)us.size(); ++t)
+            deal_next(p, t, c, (int)(npk_total * sg / nseg), (int)(npk_total * (sg + 1) / nseg));
+    }
+    cta_first.push_back(0);
+    for (const std::vector<XItem> &run : runs) {
+      if (run.empty()) continue;
+      items.insert(items.end(), run.begin(), run.end());
+      cta_first.push_back((int)items.size());
+    }
+    return (int)cta_first.size() - 1;
+  }
   long long remaining = total, load = 0;
   int cta = 0;
   long long target = (remaining + grid - 1) / grid;
@@ -351,16 +414,17 @@ int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem>
   // deals the stages [pk, npk) of unit (p, t, c) over the CTAs
   auto deal = [&](size_t p, int t, int c, int pk, int npk) {
     const XUnit &u = (*probs[p].units)[t];
+    const int per_chunk = chunk_cost(u);
     const long long fold = kFold * u.work;
     while (pk < npk) {
       if (cta == grid - 1) {  // the last CTA takes everything left
-        const long long cost = range_cost(p, pk, npk, u.z_rows) + fold;
+        const long long cost = range_cost(p, pk, npk, per_chunk) + fold;
         items.push_back({(int)p, t, c, pk, npk - pk});
         load += cost;
         pk = npk;
         continue;
       }
-      const long long rest = range_cost(p, pk, npk, u.z_rows) + fold;
+      const long long rest = range_cost(p, pk, npk, per_chunk) + fold;
       if (load + rest <= target) {
         items.push_back({(int)p, t, c, pk, npk - pk});
         load += rest;
@@ -373,13 +437,13 @@ int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem>
       int n = 0;
       const long long room = target - load - fold;
       if (room > 0) {
-        const long long per = (long long)kChunksPerPk * u.z_rows;
+        const long long per = (long long)kChunksPerPk * per_chunk;
         n = (int)std::min<long long>(npk - pk, room / per);
-        while (n > 0 && range_cost(p, pk, pk + n, u.z_rows) > room) --n;
+        while (n > 0 && range_cost(p, pk, pk + n, per_chunk) > room) --n;
       }
       if (n >= min_split_pk && npk - pk - n >= min_split_pk) {
         items.push_back({(int)p, t, c, pk, n});
-        load += range_cost(p, pk, pk + n, u.z_rows) + fold;
+        load += range_cost(p, pk, pk + n, per_chunk) + fold;
         remaining += fold;  // the rest of the unit is folded once more
         pk += n;
         close_cta();
@@ -398,18 +462,11 @@ int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem>
   for (size_t p = 0; p < probs.size(); ++p) {
     const long long npk_total = pw[p].npk;
     const int nseg = pw[p].nseg;
-    // Bands of channels, one template after the other within a band: the
-    // CTAs running at one time then work on the same channels, whose inputs
-    // every template reads again (from L2 instead of HBM), and each template
-    // still runs over a band's channels in turn.
-    for (int c0 = 0; c0 < probs[p].n_chan; c0 += kChanBand)
-      for (int t = 0; t < (int)probs[p].units->size(); ++t) {
-        const int step = std::max(1, (*probs[p].units)[t].n_chan);
-        for (int c = c0; c < std::min(probs[p].n_chan, c0 + kChanBand); c += step)
-          // fold-window segment sg: stages [npk sg / nseg, npk (sg + 1) / nseg)
-          for (int sg = 0; sg < nseg; ++sg)
-            deal(p, t, c, (int)(npk_total * sg / nseg), (int)(npk_total * (sg + 1) / nseg));
-      }
+    for (int t = 0; t < (int)probs[p].units->size(); ++t)
+      for (int c = 0; c < probs[p].n_chan; c += std::max(1, (*probs[p].units)[t].n_chan))
+        // fold-window segment sg: stages [npk sg / nseg, npk (sg + 1) / nseg)
+        for (int sg = 0; sg < nseg; ++sg)
+          deal(p, t, c, (int)(npk_total * sg / nseg), (int)(npk_total * (sg + 1) / nseg));
   }
   if (load > 0 || (int)cta_first.size() == 1) close_cta();
   // drop trailing empty CTAs

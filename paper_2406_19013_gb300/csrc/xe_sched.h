@@ -25,6 +25,15 @@ enum Cover {
   kCoverQuads = 3,
 };
 
+// Largest input count whose units run on one CTA each by default; above it CTA
+// pairs.  A pair's MMAs share their column operand, so each SM unpacks fewer
+// rows per product, but its 256-row blocks pad more and its two CTAs wait for
+// each other.  CMAC launches, one CTA / pairs: 300 inputs 0.75 / 1.16 ms, 512
+// 1.15 / 1.25 ms (128 channels, 2 blocks of 8192 samples); 32 channels, 4
+// blocks of 4096: 1152 inputs 1.30 / 1.39 ms, 1280 1.56 / 1.42, 2048 3.62 /
+// 3.21.
+constexpr int kPairInputs = 1152;
+
 // Templates of the cover, heaviest first.  kCoverWindow and kCoverStrips
 // fall back to kCoverPairs above 256 inputs.
 std::vector<XUnit> build_schedule(int n_in, int cover = kCoverWindow);
@@ -57,8 +66,9 @@ struct ProbWork {
 constexpr int kMaxFoldStages = 32768 / kPkSamples;
 static_assert(2LL * 15 * 15 * kMaxFoldStages * kPkSamples < (1LL << 24), "exact fp32 partials");
 
-// Cuts every unit (problem, template, channel) into items and deals
-// contiguous runs of them to at most `grid` CTAs.  Each CTA receives about
+// Cuts every unit (problem, template, channel) into items and deals them to at
+// most `grid` CTAs, in contiguous runs if every problem has one template, else
+// channel by channel to the CTA that is free first.  Each CTA receives about
 // the same modelled cost: the unpack work (operand rows x chunks) of its
 // items plus a fixed fold cost per item.  A unit is split only at 128-sample
 // stage boundaries and only into pieces of at least min_split_pk stages;

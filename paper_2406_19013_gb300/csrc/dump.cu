@@ -132,13 +132,39 @@ __global__ void guard_check_kernel(const unsigned char *__restrict__ before,
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(status, kStatusBounds);
 }
 
-// dst[row][0..pitch) = src[row][0..T) followed by zeros
+// dst[row][0..pitch) = src[row][0..T) followed by zeros, in words: an output
+// word is cut from the two aligned source words that hold its bytes (the
+// second word of a lane is the first of the next, so it comes from L1).  The
+// source's last bytes, whose second word would lie past its end, and each
+// row's last word are put together from bytes.  src is 4-byte aligned.  (Byte
+// by byte, a block of 75 inputs x 200 channels x 3001 samples took 75 us; a
+// push of it went from 134 to 81 us with words.)
 __global__ void pitch_kernel(const uint8_t *__restrict__ src, uint8_t *__restrict__ dst,
                              long long rows, int T, int pitch) {
-  for (long long r = blockIdx.x; r < rows; r += gridDim.x) {
-    const uint8_t *s = src + r * (long long)T;
-    uint8_t *d = dst + r * (long long)pitch;
-    for (int t = threadIdx.x; t < pitch; t += blockDim.x) d[t] = t < T ? s[t] : 0;
+  const int words = pitch >> 2;
+  const long long n_words = rows * words;
+  const long long src_bytes = rows * (long long)T;
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  long long row = k / words;
+  int w = (int)(k - row * words);
+  const long long row_step = stride / words;
+  const int w_step = (int)(stride - row_step * words);
+#pragma unroll 4
+  for (; k < n_words; k += stride) {
+    const long long at = row * T + 4 * w;  // first source byte of the word
+    const int left = T - 4 * w;            // bytes of the row from there on
+    uint32_t v = 0u;
+    if (left >= 4 && (at | 3) + 4 < src_bytes) {
+      const uint32_t *s = reinterpret_cast<const uint32_t *>(src + (at & ~3LL));
+      v = __funnelshift_r(__ldg(s), __ldg(s + 1), 8 * (int)(at & 3));
+    } else {
+      for (int b = 0; b < min(left, 4); ++b) v |= (uint32_t)__ldg(src + at + b) << (8 * b);
+    }
+    reinterpret_cast<uint32_t *>(dst)[k] = v;
+    row += row_step;
+    w += w_step;
+    if (w >= words) w -= words, ++row;
   }
 }
 

@@ -63,10 +63,10 @@ extern "C" {
 /* Largest block_len accepted (Sec. 2.4's integrations are blocks of many
  * samples; 2^24 - 1 bounds the host-side sample counters of one block). */
 #define CORR_MAX_BLOCK_LEN 16777215
-/* Samples the tensor cores accumulate in fp32 before a fold into int64.  A
- * partial over L samples is bounded by 128 * L, an exactly representable
- * integer (< 2^24) for L <= 131071; longer blocks, and launches of several
- * blocks, are folded at least this often. */
+/* Samples of the blocks that share one launch, at most (a block longer than
+ * that is a launch of its own).  The tensor cores accumulate at most 32768
+ * samples in fp32, where every partial is an exactly representable integer,
+ * before a fold into int64. */
 #define CORR_FOLD_SAMPLES 131071
 /* Largest input count N = n_ant * n_pol accepted. */
 #define CORR_MAX_INPUTS 8192
@@ -82,7 +82,8 @@ typedef struct corr_server corr_server;
  * (n_chan * P * 16 bytes, zeroed) and a few kilobytes of bookkeeping.
  * The CMAC kernel is chosen here: the all-shared-memory kernel by default;
  * CORR_CMAC_KERNEL=tm in the environment selects the TMEM-operand kernel
- * (up to 192 inputs), =pair the CTA-pair kernel (more than 256 inputs).
+ * (up to 192 inputs), =pair the CTA-pair kernel (more than 256 inputs; the
+ * default above 1152), =smem the one-CTA kernel.
  * On success *out owns them until corr_destroy.
  * Errors: CORR_EINVAL (non-positive size, n_pol not 1/2, block_len above
  * CORR_MAX_BLOCK_LEN, N above CORR_MAX_INPUTS, out NULL), CORR_EARCH,
@@ -103,10 +104,10 @@ int corr_push_block(corr_ctx *ctx, const uint8_t *d_block, void *stream);
 /*
  * Integrates n_blocks blocks (d_blocks: host array of n_blocks device
  * pointers, each as for corr_push_block).  Equivalent to n_blocks calls of
- * corr_push_block, but up to 8 blocks share one launch and one fold into the
- * int64 buffer (fewer while 8 * block_len exceeds CORR_FOLD_SAMPLES; a block
- * longer than that is folded every CORR_FOLD_SAMPLES samples or fewer).  The
- * pointer array itself may be reused as soon as the call returns.
+ * corr_push_block, but up to 8 blocks share one launch and its folds into the
+ * int64 buffer, one for every 32768 samples or fewer (fewer blocks while
+ * 8 * block_len exceeds CORR_FOLD_SAMPLES).  The pointer array itself may be
+ * reused as soon as the call returns.
  * Errors: CORR_EINVAL (NULL ctx or array, n_blocks < 1, a NULL or misaligned
  * block pointer; nothing is enqueued), CORR_ECUDA.
  */
@@ -169,14 +170,14 @@ int corr_plan(int n_in, uint8_t *cover, int *n_units, long long *issued_cmacs);
  *           64-input row tiles' strips share it, packed into 512 TMEM columns.
  *   STRIPS: N <= 256.  One unit per row tile t, staging inputs [0, 64(t+1)).
  *   PAIRS:  any N.  Pairs of row tiles against 256-column pieces of their
- *           strip; one CTA per unit.
+ *           strip (192-column pieces above 256 inputs); one CTA per unit.
  *   QUADS:  N > 256.  Blocks of 256 rows against 256-column pieces of their
  *           strip, each run by a pair of CTAs on two SMs (a 2-CTA cluster):
  *           each CTA stages 128 of the rows and half of the piece's columns,
  *           and the pair's M = 256 tensor-core MMAs share the columns.  On
  *           the diagonal the CTAs take row tiles 0 and 3, and 1 and 2, so
  *           that tiles 0 and 1 run against 128 columns only.
- *           Contexts use it only when CORR_CMAC_KERNEL=pair is set.
+ *           Contexts and batches use it above 1152 inputs.
  * WINDOW and STRIPS fall back to PAIRS above 256 inputs, QUADS to PAIRS at
  * 256 and below.  CORR_CMAC_KERNEL=pair in the environment makes contexts of
  * more than 256 inputs use QUADS, =smem PAIRS. */
@@ -195,11 +196,15 @@ int corr_plan_cover(int n_in, int cover, uint8_t *cover_out, int *n_units,
  * multiprocessors (no device needed).
  *   - A unit is (template, channel): one of the cover's n_units templates on
  *     one channel, over all n_blocks blocks of block_len samples.
- *   - Units are cut at 128-sample stage boundaries into items, and every CTA
- *     (at most `grid`) runs a contiguous run of items of about equal
- *     modelled cost.  That cost is the operand rows unpacked plus a fixed
- *     fold cost per item.  No item spans more than CORR_FOLD_SAMPLES / 128
- *     stages (1023): each item folds its fp32 partials into int64 once.
+ *   - Units are cut at 128-sample stage boundaries into items, dealt to at
+ *     most `grid` CTAs with about equal modelled cost: the cycles of the
+ *     chunks' matrix products or unpack, plus the fold of each item.  With one
+ *     or two templates per channel every CTA runs a contiguous run of items;
+ *     with more, the units of a channel (which read the same inputs) go to
+ *     the CTAs that are free first.  No item spans more than 256 stages
+ *     (32768 samples): each item folds its fp32 partials into int64 once.
+ *   - Contexts whose units are too few to fill the GPU (at most four items
+ *     per CTA) may cut them finer than this view shows.
  *   - n_blocks: 1..8 (the blocks of one launch).
  *   - items, if not NULL, receives up to `cap` rows of 5 ints:
  *     (problem = 0, template, channel, first stage, stages).  Stage k of the
@@ -229,7 +234,7 @@ int corr_plan_items(int n_in, int n_chan, int block_len, int n_blocks, int cover
  * loads the library holds until the process exits; the call allocates nothing
  * on the device or the host.
  *   - Limits: n_ant * n_pol <= CORR_STATIC_MAX_INPUTS, block_len a multiple of
- *     16 (at most CORR_STATIC_MAX_BLOCK_LEN, one fold per call); d_block and
+ *     16 (at most CORR_STATIC_MAX_BLOCK_LEN); d_block and
  *     d_vis 16-byte aligned.
  *     Anything else returns CORR_EINVAL before any work is enqueued.
  *   - The first call on a device looks up the array's device address and the
@@ -279,8 +284,8 @@ int corr_corner_turn(const uint8_t *d_src, uint8_t *d_dst, int n_in, int n_chan,
  * [block_len][n_chan][N] (d_src, 4-byte aligned): the Transpose step of
  * Sec. 2.1 and the correlation in one call.
  *   - When N is a multiple of 16, d_src is 16-byte aligned and the context
- *     runs the all-shared-memory CMAC kernel (the default; not with
- *     CORR_CMAC_KERNEL=tm or =pair), the CMAC kernel stages the block in this order
+ *     runs an all-shared-memory CMAC kernel (the default; not with
+ *     CORR_CMAC_KERNEL=tm), the CMAC kernel stages the block in this order
  *     itself: its TMA boxes are [128 samples][64 inputs] of one channel and
  *     the unpack transposes them on chip.  One launch; every byte is read
  *     once.
@@ -416,9 +421,10 @@ int corr_batch_dump(corr_batch *b, int inst, int64_t *d_vis, int64_t *d_stokes, 
 int corr_batch_sizes(const corr_batch *b, int inst, size_t *vis_elems, size_t *stokes_elems,
                      long long *samples_integrated);
 
-/* Instance `inst`'s cover (CORR_COVER_*), its launch group, and the number of
- * launch groups (one CMAC launch each per push).  Any output may be NULL.
- * Errors: CORR_EINVAL. */
+/* Instance `inst`'s cover (CORR_COVER_*; above 1152 inputs CORR_COVER_PAIRS,
+ * which then runs in its CTA-pair form, CORR_COVER_QUADS), its launch group,
+ * and the number of launch groups (one CMAC launch each per push).  Any output
+ * may be NULL.  Errors: CORR_EINVAL. */
 int corr_batch_info(const corr_batch *b, int inst, int *cover, int *group, int *n_groups);
 
 /* As corr_check, for the batch's device status word. */

@@ -269,7 +269,7 @@ int upload_group(corr_batch *b, BGroup &g) {
     workers = std::min(b->n_sm / 2, xe::cmac_pair_clusters_batch(g.L.smem_bytes));
     if (workers < 1) return CORR_ECUDA;
   }
-  g.grid = xe::build_items(work, workers, items, first);
+  g.grid = xe::build_items_filled(work, workers, items, first);
   int rc;
   if ((rc = cuda_err(cudaMalloc(&g.d_units, all.size() * sizeof(xe::XUnit)))) != CORR_OK ||
       (rc = cuda_err(cudaMalloc(&g.d_probs, g.members.size() * sizeof(xe::XProb)))) != CORR_OK ||

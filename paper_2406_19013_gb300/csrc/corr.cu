@@ -321,7 +321,8 @@ int corr_create(int n_ant, int n_pol, int n_chan, int block_len, corr_ctx **out)
     std::vector<xe::XItem> items;
     std::vector<int> first;
     ItemPlan &pl = ctx->plans[nb];
-    pl.grid = xe::build_items({{&plan_units, n_chan, block_len, nb}}, workers, items, first);
+    pl.grid =
+        xe::build_items_filled({{&plan_units, n_chan, block_len, nb}}, workers, items, first);
     if ((rc = cuda_err(cudaMalloc(&pl.d_items, items.size() * sizeof(xe::XItem)))) != CORR_OK ||
         (rc = cuda_err(cudaMalloc(&pl.d_cta_first, first.size() * sizeof(int)))) != CORR_OK ||
         (rc = cuda_err(cudaMemcpy(pl.d_items, items.data(), items.size() * sizeof(xe::XItem),
@@ -466,10 +467,10 @@ int corr_push_block_tcn(corr_ctx *ctx, const uint8_t *d_src, void *stream) {
   CORR_TRACE("corr_push_block_tcn");
   if (!ctx || !d_src || (reinterpret_cast<uintptr_t>(d_src) & 3u)) return CORR_EINVAL;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // The shared-memory kernel stages F-engine-order blocks directly (TMA boxes
+  // The shared-memory kernels stage F-engine-order blocks directly (TMA boxes
   // of [128 samples][64 inputs], transposed on chip) when the block's strides
   // allow a tensor map; otherwise the block is turned in HBM first.
-  if (!ctx->tm && !ctx->pair && ctx->n_in % 16 == 0 &&
+  if (!ctx->tm && ctx->n_in % 16 == 0 &&
       (reinterpret_cast<uintptr_t>(d_src) & 15u) == 0)
     return launch_staged(ctx, &d_src, 1, st, 0, true);
   int rc;

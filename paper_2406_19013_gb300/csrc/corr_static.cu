@@ -11,7 +11,6 @@
 // size, and writes the visibilities straight into the caller's buffer.  It
 // calls no cudaMalloc, cudaFree or other allocating routine, on the device or
 // on the host.
-#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -47,7 +46,7 @@ unsigned long long g_timeout_ns = 2000000000ull;  // device-side wait limit (COR
 // The schedule and problem descriptor of one call, passed by value in the
 // parameters of the set-up kernel below (so nothing is copied from host
 // memory, which a captured copy would read again at replay).
-constexpr int kMaxCallUnits = 4;
+constexpr int kMaxCallUnits = xe::kMaxWindowUnits;
 struct StaticPlan {
   xe::XProb prob;
   xe::XUnit units[kMaxCallUnits];
@@ -70,12 +69,6 @@ __global__ void static_setup_kernel(const __grid_constant__ StaticPlan plan, xe:
   if (threadIdx.x == 0) *d_status = 0;
 }
 
-typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *,
-                                  const cuuint64_t *, const cuuint64_t *, const cuuint32_t *,
-                                  const cuuint32_t *, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn g_encode = nullptr;
-
 int rc_of(cudaError_t e) { return e == cudaSuccess ? CORR_OK : CORR_ECUDA; }
 
 // Once per device, with that device current: resolve the array's device
@@ -90,15 +83,6 @@ int setup_device(int dev) {
   int optin = 0;
   if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
     return CORR_ECUDA;
-  if (!g_encode) {
-    void *p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault,
-                                         &q) != cudaSuccess ||
-        q != cudaDriverEntryPointSuccess)
-      return CORR_ECUDA;
-    g_encode = reinterpret_cast<EncodeTiledFn>(p);
-  }
   void *addr = nullptr;
   if (cudaGetSymbolAddress(&addr, g_static_scratch) != cudaSuccess || !addr) return CORR_ECUDA;
   if (const char *env = std::getenv("CORR_TIMEOUT_MS")) {
@@ -109,61 +93,6 @@ int setup_device(int dev) {
   g_n_sm[dev] = prop.multiProcessorCount;
   g_scratch_addr[dev] = static_cast<unsigned char *>(addr);
   return CORR_OK;
-}
-
-// The single-window tile schedule (all inputs staged together; row tiles of
-// 64 inputs packed into units of at most 512 accumulator columns), built in
-// a fixed array.  Returns the number of units.
-int plan_single_window(int N, xe::XUnit *units) {
-  const int n16 = (N + 15) / 16 * 16;
-  const int n_rt = (N + xe::kTileInputs - 1) / xe::kTileInputs;  // <= 4
-  int bin_of[4], used[4] = {0, 0, 0, 0}, n_bins = 0;
-  for (int t = n_rt - 1; t >= 0; --t) {  // largest strip first, first fit
-    const int n = std::min(xe::kTileInputs * (t + 1), n16);
-    int b = 0;
-    while (b < n_bins && used[b] + n > xe::kTmemCols) ++b;
-    if (b == n_bins) ++n_bins;
-    used[b] += n;
-    bin_of[t] = b;
-  }
-  for (int b = 0; b < n_bins; ++b) {
-    xe::XUnit &u = units[b];
-    std::memset(&u, 0, sizeof(u));
-    u.n_chan = 1;
-    int t_max = 0;
-    for (int t = 0; t < n_rt; ++t)
-      if (bin_of[t] == b) t_max = std::max(t_max, t);
-    xe::XRegion &r = u.reg[0];
-    r.in_lo = 0;
-    r.in_lo1 = 0;
-    r.n_in = xe::kTileInputs * (t_max + 1);
-    r.interleaved = 1;
-    r.z_row = 0;
-    r.pk_off = 0;
-    u.n_reg = 1;
-    u.z_rows = 2 * r.n_in;
-    u.n_sum = r.n_in;
-    u.pk_bytes = r.n_in * xe::kPackedRowBytes;
-    for (int t = n_rt - 1; t >= 0; --t) {
-      if (bin_of[t] != b) continue;
-      xe::XSeg &s = u.seg[u.n_seg];
-      s.a_zrow = 128 * t;
-      s.b_zrow = 0;
-      s.a_sum = xe::kTileInputs * t;
-      s.b_sbo = 2048;
-      s.n = std::min(xe::kTileInputs * (t + 1), n16);
-      s.tmem_col = u.work;
-      s.row_in0 = xe::kTileInputs * t;
-      s.row_in1 = s.row_in0;
-      for (int c = 0; c < 4; ++c) s.col_blk[c] = 64 * c;  // columns 0, 1, 2, ...
-      u.work += s.n;
-      u.n_seg++;
-    }
-  }
-  // heaviest unit first (at most four: an insertion sort)
-  for (int i = 1; i < n_bins; ++i)
-    for (int j = i; j > 0 && units[j - 1].work < units[j].work; --j) std::swap(units[j - 1], units[j]);
-  return n_bins;
 }
 
 }  // namespace
@@ -187,8 +116,8 @@ extern "C" int corr_xcorr_static(const uint8_t *d_block, int n_ant, int n_pol, i
   StaticPlan plan;
   std::memset(&plan, 0, sizeof(plan));
   xe::XUnit *units = plan.units;
-  const int n_tpl = plan_single_window((int)N, units);
-  if (n_tpl > kMaxStaticUnits || n_tpl > kMaxCallUnits) return CORR_EINVAL;
+  const int n_tpl = xe::window_units((int)N, units);
+  if (n_tpl > kMaxStaticUnits) return CORR_EINVAL;
   plan.n_units = n_tpl;
   int max_z = 0, max_pk = 0, max_sum = 0;
   for (int k = 0; k < n_tpl; ++k) {
@@ -196,21 +125,9 @@ extern "C" int corr_xcorr_static(const uint8_t *d_block, int n_ant, int n_pol, i
     max_pk = std::max(max_pk, units[k].pk_bytes);
     max_sum = std::max(max_sum, units[k].n_sum);
   }
-  // shared-memory stages, sized as for a context
   const int optin = g_smem_optin[dev];
-  const int z_bytes = (max_z * 128 + 1023) / 1024 * 1024;
-  const int pk_bytes = (max_pk + 1023) / 1024 * 1024;
-  const int fixed = 1024 + xe::kBarrierBytes + xe::kEpiWarps * xe::kEpiBufBytes +
-                    max_sum * xe::kSumBytesPerInput;
-  int pk_stages = 3, z_stages = 0;
-  for (int ps = 3; ps >= 2 && z_stages < 2; --ps) {
-    pk_stages = ps;
-    z_stages = (optin - fixed - ps * pk_bytes) / z_bytes;
-  }
-  z_stages = std::min(z_stages, 4);
-  if (z_stages < 2) return CORR_EINVAL;
-  int smem = fixed + z_stages * z_bytes + pk_stages * pk_bytes;
-  smem = std::min(std::max(smem, optin / 2 + 1024), optin);
+  xe::StageLayout L;
+  if (!xe::stage_layout(max_z, max_pk, max_sum, optin, xe::kMaxZStages, &L)) return CORR_EINVAL;
 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   unsigned char *scratch = g_scratch_addr[dev];
@@ -239,14 +156,8 @@ extern "C" int corr_xcorr_static(const uint8_t *d_block, int n_ant, int n_pol, i
 
   xe::XMaps maps;
   std::memset(&maps, 0, sizeof(maps));
-  const cuuint64_t dims[3] = {(cuuint64_t)block_len, (cuuint64_t)N, (cuuint64_t)n_chan};
-  const cuuint64_t strides[2] = {(cuuint64_t)block_len, (cuuint64_t)block_len * (cuuint64_t)N};
-  const cuuint32_t box[3] = {(cuuint32_t)xe::kPkSamples, (cuuint32_t)xe::kTileInputs, 1};
-  const cuuint32_t estr[3] = {1, 1, 1};
-  if (g_encode(reinterpret_cast<CUtensorMap *>(maps.m[0]), CU_TENSOR_MAP_DATA_TYPE_UINT8, 3,
-               const_cast<uint8_t *>(d_block), dims, strides, box, estr,
-               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
-               CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+  const int ch_rows = units[0].seg[0].ch_rows ? units[0].seg[0].ch_rows : xe::kTileInputs;
+  if (!xe::encode_block_map(d_block, block_len, (int)N, n_chan, block_len, maps.m[0], ch_rows))
     return CORR_ECUDA;
 
   xe::XParams p;
@@ -255,18 +166,30 @@ extern "C" int corr_xcorr_static(const uint8_t *d_block, int n_ant, int n_pol, i
   p.items = nullptr;  // units (or their fold windows), dealt round-robin over the CTAs
   p.cta_first = nullptr;
   p.implicit_n_tpl = n_tpl;
-  p.implicit_n_chan = n_chan;
+  p.implicit_chan_step = units[0].n_chan;
+  p.implicit_n_chan = (n_chan + units[0].n_chan - 1) / units[0].n_chan;
   p.implicit_npk = prob.pk_per_block;
-  // as many items per unit as keep every fp32 partial exact
-  p.implicit_nseg = (prob.pk_per_block + xe::kMaxFoldStages - 1) / xe::kMaxFoldStages;
+  // Items per unit: as many as keep every fp32 partial exact, or more where
+  // that shortens the modelled run (rounds of items over the SMs, each a piece
+  // of the heaviest unit and its fold).
+  const long long n_units = (long long)n_tpl * p.implicit_n_chan;
+  const int min_seg = (p.implicit_npk + xe::kMaxFoldStages - 1) / xe::kMaxFoldStages;
+  long long best = 0;
+  for (int seg = min_seg; seg <= std::min(p.implicit_npk, 32 * min_seg); ++seg) {
+    const long long rounds = (n_units * seg + g_n_sm[dev] - 1) / g_n_sm[dev];
+    const long long piece = (p.implicit_npk + seg - 1) / seg;
+    const long long t = rounds * (piece * xe::kChunksPerPk * xe::chunk_cost(units[0]) +
+                                  xe::kFold * units[0].work);
+    if (seg == min_seg || t < best) best = t, p.implicit_nseg = seg;
+  }
   p.status = d_status;
   p.timeout_ns = g_timeout_ns;
-  p.z_stages = z_stages;
-  p.pk_stages = pk_stages;
-  p.z_stage_bytes = (uint32_t)z_bytes;
-  p.pk_stage_bytes = (uint32_t)pk_bytes;
-  p.sum_rows = max_sum;
-  const long long n_work = (long long)n_tpl * n_chan * p.implicit_nseg;
+  p.z_stages = L.z_stages;
+  p.pk_stages = L.pk_stages;
+  p.z_stage_bytes = L.z_stage_bytes;
+  p.pk_stage_bytes = L.pk_stage_bytes;
+  p.sum_rows = L.sum_rows;
+  const long long n_work = n_units * p.implicit_nseg;
   const int grid = (int)std::min<long long>(n_work, g_n_sm[dev]);
-  return rc_of(xe::launch_cmac(maps, p, grid, smem, st));
+  return rc_of(xe::launch_cmac(maps, p, grid, L.smem_bytes, st));
 }

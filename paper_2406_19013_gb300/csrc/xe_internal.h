@@ -163,11 +163,12 @@ struct XParams {
   // Explicit items: CTA b runs items [cta_first[b], cta_first[b + 1]).
   // With items == nullptr the launch holds problem 0 alone and CTA b runs
   // items b, b + grid, ... of its n_tpl x n_chan units (unit w is template
-  // w / n_chan on channel w % n_chan), all npk stages of each.
+  // w / n_chan on channels from w % n_chan), all npk stages of each.
   const XItem *items;
   const int *cta_first;
-  // Each unit is cut into implicit_nseg items of equal length.
-  int implicit_n_tpl, implicit_n_chan, implicit_npk, implicit_nseg;
+  // Each unit is cut into implicit_nseg items of equal length; unit w of a
+  // template starts at channel implicit_chan_step w.
+  int implicit_n_tpl, implicit_n_chan, implicit_npk, implicit_nseg, implicit_chan_step;
   int *status;           // device status word (kStatusTimeout | kStatusBounds)
   unsigned long long timeout_ns;
   int z_stages, pk_stages;

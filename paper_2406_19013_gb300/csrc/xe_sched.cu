@@ -68,19 +68,27 @@ XUnit empty_unit() {
 
 }  // namespace
 
+// Entries of the table of operand sums for a finished unit's segments.
+static void set_sums(XUnit &u) {
+  for (int s = 0; s < u.n_seg; ++s) {
+    u.seg[s].a_sum = sum_entry(u, u.seg[s].a_zrow);
+    u.seg[s].b_sum = sum_entry(u, u.seg[s].b_zrow);
+  }
+}
+
 // Tiles of 64 inputs (rows) cover the lower triangle strip by strip: row tile
 // t needs columns [0, min(64 (t + 1), N)).  Within a unit, columns are staged
 // once per chunk and shared by all its row tiles.
-std::vector<XUnit> build_schedule(int N, int cover) {
-  std::vector<XUnit> units;
+int window_units(int N, XUnit *units) {
   const int n16 = round_up(N, 16);
   const int n_rt = (N + kTileInputs - 1) / kTileInputs;
-  if (N <= 32 && cover == kCoverWindow) {
+  int n_units = 0;
+  if (N <= 32) {
     // 16 or 32 inputs at most: a 64-row tile holds 64 / n16 channels (the
     // TMA box brings that many channels' rows at once), and a unit two such
     // tiles; each tile's MMA also computes the cross-channel blocks, which
     // the epilogue skips
-    XUnit u = empty_unit();
+    XUnit &u = units[n_units++] = empty_unit();
     const int cpt = kTileInputs / n16;
     u.n_chan = 2 * cpt;
     for (int r = 0; r < 2; ++r) {
@@ -92,13 +100,12 @@ std::vector<XUnit> build_schedule(int N, int cover) {
       u.seg[r].chan_off = r * cpt;
       u.seg[r].ch_rows = n16;
     }
-    units.push_back(u);
-  } else if (N <= 2 * kTileInputs && cover == kCoverWindow) {
+  } else if (N <= 2 * kTileInputs) {
     // one or two row tiles: a unit covers two channels (two staged regions,
     // one accumulator per row tile and channel, at most 2 x 192 TMEM
     // columns), so every chunk handed from the unpack to the MMA issuers
     // carries twice the work
-    XUnit u = empty_unit();
+    XUnit &u = units[n_units++] = empty_unit();
     u.n_chan = 2;
     for (int r = 0; r < 2; ++r) {
       add_reg(u, 0, kTileInputs * n_rt, 1);
@@ -110,35 +117,40 @@ std::vector<XUnit> build_schedule(int N, int cover) {
                 std::min(kTileInputs * (t + 1), n16), kTileInputs * t, 0);
         u.seg[u.n_seg - 1].chan_off = r;
       }
-    units.push_back(u);
-  } else if (N <= 256 && cover == kCoverWindow) {
+  } else {
     // units of consecutive row tiles, largest strip first, each as many as
     // fit 512 TMEM columns: a unit's lowest tile then bounds the inputs that
     // are only its columns, and those need no Q rows
-    std::vector<std::vector<int>> bins;
-    int used = kTmemCols + 1;
-    for (int t = n_rt - 1; t >= 0; --t) {
-      const int n = std::min(kTileInputs * (t + 1), n16);
-      if (used + n > kTmemCols) {
-        bins.push_back({});
-        used = 0;
+    for (int t_max = n_rt - 1; t_max >= 0;) {
+      int t_min = t_max + 1, used = 0;
+      while (t_min > 0) {
+        const int n = std::min(kTileInputs * t_min, n16);  // tile t_min - 1
+        if (used + n > kTmemCols) break;
+        used += n;
+        --t_min;
       }
-      bins.back().push_back(t);
-      used += n;
-    }
-    for (auto &bin : bins) {
-      XUnit u = empty_unit();
-      int t_max = 0, t_min = n_rt;
-      for (int t : bin) t_max = std::max(t_max, t), t_min = std::min(t_min, t);
+      XUnit &u = units[n_units++] = empty_unit();
       // inputs below the unit's lowest row tile are only its columns: their
       // Q rows are neither decoded nor stored (same layout, so the B operand
       // still spans the window with one stride)
       if (t_min > 0) add_reg(u, 0, kTileInputs * t_min, 2);
       add_reg(u, kTileInputs * t_min, kTileInputs * (t_max + 1 - t_min), 1);
-      for (int t : bin)
+      for (int t = t_max; t >= t_min; --t)
         add_seg(u, 128 * t, 0, 2048, std::min(kTileInputs * (t + 1), n16), kTileInputs * t, 0);
-      units.push_back(u);
+      t_max = t_min - 1;
     }
+  }
+  for (int k = 0; k < n_units; ++k) set_sums(units[k]);
+  return n_units;
+}
+
+std::vector<XUnit> build_schedule(int N, int cover) {
+  std::vector<XUnit> units;
+  const int n16 = round_up(N, 16);
+  const int n_rt = (N + kTileInputs - 1) / kTileInputs;
+  if (N <= 256 && cover == kCoverWindow) {
+    XUnit w[kMaxWindowUnits];
+    units.assign(w, w + window_units(N, w));
   } else if (N <= 256 && cover == kCoverStrips) {
     for (int t = n_rt - 1; t >= 0; --t) {
       XUnit u = empty_unit();
@@ -223,11 +235,7 @@ std::vector<XUnit> build_schedule(int N, int cover) {
   }
   std::stable_sort(units.begin(), units.end(),
                    [](const XUnit &a, const XUnit &b) { return a.work > b.work; });
-  for (XUnit &u : units)
-    for (int s = 0; s < u.n_seg; ++s) {
-      u.seg[s].a_sum = sum_entry(u, u.seg[s].a_zrow);
-      u.seg[s].b_sum = sum_entry(u, u.seg[s].b_zrow);
-    }
+  for (XUnit &u : units) set_sums(u);
   // the unpack handles regions of at most kMaxRegionInputs inputs (every
   // cover above satisfies this; an empty schedule reports a violation)
   for (const XUnit &u : units)
@@ -252,6 +260,11 @@ bool stage_layout(const std::vector<const std::vector<XUnit> *> &unit_sets, int 
       max_pk = std::max(max_pk, u.pk_bytes);
       max_sum = std::max(max_sum, (u.pair_rows ? 2 : 1) * u.n_sum);
     }
+  return stage_layout(max_zr, max_pk, max_sum, smem_optin, max_z, out);
+}
+
+bool stage_layout(int max_zr, int max_pk, int max_sum, int smem_optin, int max_z,
+                  StageLayout *out) {
   StageLayout L;
   L.sum_rows = max_sum;
   L.z_stage_bytes = (uint32_t)round_up(max_zr * 128, 1024);
@@ -302,14 +315,87 @@ bool stage_layout(const std::vector<const std::vector<XUnit> *> &unit_sets, int 
   return true;
 }
 
-// Cycles of one 64-sample chunk of a unit: its MMAs (four K slices of each
-// segment; measured on shared-memory operands, 57 cycles at N = 64, 122 at
-// 192, 155 at 256, and 182 for a CTA pair's M = 256, N = 256), or the unpack of
-// its operand rows (960 cycles for 384 rows) if that takes longer.
-static int chunk_cost(const XUnit &u) {
+int chunk_cost(const XUnit &u) {
   int mma = 0;
   for (int s = 0; s < u.n_seg; ++s) mma += 4 * ((u.pair_rows ? 54 : 24) + u.seg[s].n / 2);
   return std::max(mma, 5 * u.z_rows / 2);
+}
+
+// Modelled cycles of the busiest CTA of a split.
+static long long busiest(const std::vector<ProbWork> &probs, const std::vector<XItem> &items,
+                         const std::vector<int> &cta_first) {
+  long long most = 0;
+  for (size_t b = 0; b + 1 < cta_first.size(); ++b) {
+    long long sum = 0;
+    for (int k = cta_first[b]; k < cta_first[b + 1]; ++k) {
+      const XUnit &u = (*probs[items[k].prob].units)[items[k].tpl];
+      sum += (long long)kChunksPerPk * items[k].npk * chunk_cost(u) + kFold * u.work;
+    }
+    most = std::max(most, sum);
+  }
+  return most;
+}
+
+int build_items_filled(const std::vector<ProbWork> &probs, int grid, std::vector<XItem> &items,
+                       std::vector<int> &cta_first) {
+  int used = build_items(probs, grid, items, cta_first);
+  if (used <= 0) return used;
+  long long best = busiest(probs, items, cta_first);
+  // with many items per CTA the runs are balanced and finer pieces only add
+  // folds
+  if ((int)items.size() > 4 * grid) return used;
+  std::vector<XItem> it;
+  std::vector<int> first;
+  auto keep_if_better = [&]() {
+    const long long t = busiest(probs, it, first);
+    if (t >= best) return;
+    best = t;
+    items.swap(it);
+    cta_first.swap(first);
+  };
+  // finer cuts of the runs
+  for (int min_split = 8; min_split >= 2; min_split /= 2) {
+    build_items(probs, grid, it, first, min_split);
+    keep_if_better();
+  }
+  // every unit in n equal pieces, dealt in turn to the CTA that is free first
+  // (where a fold costs more than a CTA's share of the work, no run is cut)
+  for (int n = 2; n <= 64; n *= 2) {
+    std::vector<std::vector<XItem>> runs(grid);
+    typedef std::pair<long long, int> Load;
+    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> free_first;
+    for (int k = 0; k < grid; ++k) free_first.push({0, k});
+    for (size_t p = 0; p < probs.size(); ++p) {
+      const ProbWork &pr = probs[p];
+      const int npk = (pr.block_len + kPkSamples - 1) / kPkSamples * pr.n_blocks;
+      const int pieces =
+          std::min(npk, n * std::max(1, (npk + kMaxFoldStages - 1) / kMaxFoldStages));
+      for (int t = 0; t < (int)pr.units->size(); ++t) {
+        const XUnit &u = (*pr.units)[t];
+        for (int c = 0; c < pr.n_chan; c += std::max(1, u.n_chan))
+          for (int k = 0; k < pieces; ++k) {
+            const int a = (int)((long long)npk * k / pieces);
+            const int b = (int)((long long)npk * (k + 1) / pieces);
+            const Load l = free_first.top();
+            free_first.pop();
+            runs[l.second].push_back({(int)p, t, c, a, b - a});
+            free_first.push({l.first + (long long)kChunksPerPk * (b - a) * chunk_cost(u) +
+                                 kFold * u.work,
+                             l.second});
+          }
+      }
+    }
+    it.clear();
+    first.assign(1, 0);
+    for (const std::vector<XItem> &run : runs) {
+      if (run.empty()) continue;
+      it.insert(it.end(), run.begin(), run.end());
+      first.push_back((int)it.size());
+    }
+    keep_if_better();
+    if ((int)it.size() > 4 * grid) break;
+  }
+  return (int)cta_first.size() - 1;
 }
 
 int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem> &items,
@@ -318,7 +404,6 @@ int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem>
   cta_first.clear();
   // Cost model, in SM cycles: chunk_cost per 64-sample chunk of a unit, and
   // kFold per accumulator column for its fold.
-  constexpr long long kFold = 50;
   struct PW {
     int cpb, ppb, npk, nseg;  // nseg: fold-window segments of a unit's stages
   };

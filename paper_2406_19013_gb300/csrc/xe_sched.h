@@ -38,6 +38,21 @@ constexpr int kPairInputs = 1152;
 // fall back to kCoverPairs above 256 inputs.
 std::vector<XUnit> build_schedule(int n_in, int cover = kCoverWindow);
 
+// The window cover's templates, heaviest first, into units[kMaxWindowUnits]
+// (n_in <= 256; allocates nothing).  Returns their number; all of them cover
+// the same number of channels.
+constexpr int kMaxWindowUnits = 4;
+int window_units(int n_in, XUnit *units);
+
+// Modelled cycles of one 64-sample chunk of a unit: its MMAs (four K slices of
+// each segment; measured on shared-memory operands, 57 cycles at N = 64, 122
+// at 192, 155 at 256, and 182 for a CTA pair's M = 256, N = 256), or the unpack
+// of its operand rows (960 cycles for 384 rows) if that takes longer.
+int chunk_cost(const XUnit &u);
+// Modelled cycles of a unit's fold per accumulator column (measured: 384
+// columns in about 20 000 cycles).
+constexpr long long kFold = 50;
+
 // Shared-memory layout of a launch whose units are `units`.
 struct StageLayout {
   int z_stages, pk_stages;
@@ -50,6 +65,11 @@ struct StageLayout {
 // 2 + 2 stages fit.
 bool stage_layout(const std::vector<const std::vector<XUnit> *> &unit_sets, int smem_optin,
                   int max_z, StageLayout *out);
+
+// The same for units of at most max_zr operand rows, max_pk packed bytes and
+// max_sum entries of operand sums (allocates nothing).
+bool stage_layout(int max_zr, int max_pk, int max_sum, int smem_optin, int max_z,
+                  StageLayout *out);
 
 // One problem as the item builder sees it.
 struct ProbWork {
@@ -78,6 +98,13 @@ static_assert(2LL * 15 * 15 * kMaxFoldStages * kPkSamples < (1LL << 24), "exact 
 int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem> &items,
                 std::vector<int> &cta_first, int min_split_pk = 16,
                 int max_item_pk = kMaxFoldStages);
+
+// As build_items, for a launch that is to fill the SMs: where the units are few,
+// finer cuts and equal pieces of every unit are tried as well and the split
+// whose busiest CTA is modelled shortest is taken (16 inputs x 64 channels x
+// 2048 samples: 8 units of 16 stages ran on 8 CTAs, and run on 128).
+int build_items_filled(const std::vector<ProbWork> &probs, int grid, std::vector<XItem> &items,
+                       std::vector<int> &cta_first);
 
 // The TMA descriptor of one block, uint8 [n_chan][n_in][row pitch], 3-D
 // (time, input, channel) with boxes of 128 samples x ch_rows inputs x

@@ -78,7 +78,7 @@ __device__ __forceinline__ XItem item_at(const XParams &p, int it) {
   r.prob = 0;
   const int unit = it / p.implicit_nseg, seg = it - unit * p.implicit_nseg;
   r.tpl = unit / p.implicit_n_chan;
-  r.chan = unit - r.tpl * p.implicit_n_chan;
+  r.chan = (unit - r.tpl * p.implicit_n_chan) * p.implicit_chan_step;
   r.pk0 = (int)((long long)p.implicit_npk * seg / p.implicit_nseg);
   r.npk = (int)((long long)p.implicit_npk * (seg + 1) / p.implicit_nseg) - r.pk0;
   return r;
@@ -287,7 +287,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     it_step = 1;
   } else {
     it0 = blockIdx.x;
-    it1 = p.implicit_n_tpl * p.implicit_n_chan;
+    it1 = p.implicit_n_tpl * p.implicit_n_chan * p.implicit_nseg;
     it_step = gridDim.x;
   }
   const uint64_t to = p.timeout_ns;
@@ -755,6 +755,7 @@ cudaError_t cmac_set_smem(int smem_bytes) {
       reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxMaps, false, false>),
       reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxMaps, true, false>),
       reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxMaps, false, true>),
+      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxMaps, true, true>),
       reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxBatchMaps, false, false>),
       reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxBatchMaps, false, true>)};
   for (const void *k : kernels) {
@@ -798,6 +799,7 @@ struct PairConfig {
 cudaError_t launch_cmac_pair(const XMaps &maps, const XParams &p, int clusters, int smem_bytes,
                              cudaStream_t stream) {
   PairConfig c(clusters, smem_bytes, stream);
+  if (p.tcn) return cudaLaunchKernelEx(&c.cfg, xengine_cmac_kernel<kMaxMaps, true, true>, maps, p);
   return cudaLaunchKernelEx(&c.cfg, xengine_cmac_kernel<kMaxMaps, false, true>, maps, p);
 }
 

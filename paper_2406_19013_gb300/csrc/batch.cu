@@ -46,6 +46,7 @@ struct BInst {
 };
 
 struct BGroup {
+  bool gram;  // units of the Gram form
   bool pair;  // CTA pairs (units with pair_rows) run this group
   std::vector<int> members;
   std::vector<std::vector<xe::XUnit>> units;  // per member
@@ -132,6 +133,7 @@ float time_cover(const std::vector<xe::XUnit> &units, int n_in, int C, int T, in
   p.z_stage_bytes = L.z_stage_bytes;
   p.pk_stage_bytes = L.pk_stage_bytes;
   p.sum_rows = L.sum_rows;
+  p.gram = units[0].gram;
   for (int rep = 0; rep < 6; ++rep) {
     if (cudaEventRecord(e0, st) != cudaSuccess ||
         xe::launch_cmac(maps, p, grid, L.smem_bytes, st) != cudaSuccess ||
@@ -181,7 +183,11 @@ int tuned_cover(int n_in, int block_len, int n_sm, int smem_optin, int *rc) {
   // the default cover (the first candidate) is kept unless another one is
   // faster by more than the run-to-run spread of a timing (3 %)
   for (int cv : cands) {
-    const std::vector<xe::XUnit> units = xe::build_schedule(n_in, cv);
+    std::vector<xe::XUnit> units = xe::build_schedule(n_in, cv);
+    if (n_in <= xe::kGramInputs && cv == xe::kCoverWindow) {
+      xe::XUnit g[xe::kMaxWindowUnits];
+      units.assign(g, g + xe::gram_units(n_in, g));
+    }
     if (units.empty()) continue;
     const float ms = time_cover(units, n_in, C, T, n_sm, smem_optin, d_x, d_acc, d_status, st);
     if (ms >= 0.0f && (best_ms < 0.0f || ms < 0.97f * best_ms)) {
@@ -264,6 +270,7 @@ int upload_group(corr_batch *b, BGroup &g) {
   std::vector<xe::XItem> items;
   std::vector<int> first;
   g.pair = g.units[0][0].pair_rows != 0;
+  g.gram = g.units[0][0].gram != 0;
   int workers = b->n_sm;
   if (g.pair) {
     workers = std::min(b->n_sm / 2, xe::cmac_pair_clusters_batch(g.L.smem_bytes));
@@ -394,13 +401,18 @@ int corr_batch_create(int n_inst, const int *n_ant, const int *n_pol, const int 
     // the pairs cover of the largest arrays runs in its CTA-pair form
     units[k] = xe::build_schedule(
         b->inst[k].n_in, b->inst[k].n_in > xe::kPairInputs ? xe::kCoverQuads : b->inst[k].cover);
+    if (b->inst[k].n_in <= xe::kGramInputs && b->inst[k].cover == xe::kCoverWindow) {
+      xe::XUnit g[xe::kMaxWindowUnits];
+      units[k].assign(g, g + xe::gram_units(b->inst[k].n_in, g));
+    }
     xe::StageLayout L;
     if (units[k].empty() || !xe::stage_layout({&units[k]}, optin, xe::kMaxZStages, &L)) {
       free_batch(b);
       return CORR_EINVAL;
     }
-    const uint32_t pair_bit = units[k][0].pair_rows ? 1u : 0u;  // stage sizes are multiples of 1024
-    by_layout[{L.z_stage_bytes | pair_bit, L.pk_stage_bytes}].push_back(k);
+    // stage sizes are multiples of 1024: the kernel variant goes in the low bits
+    const uint32_t variant = units[k][0].pair_rows ? 1u : units[k][0].gram ? 2u : 0u;
+    by_layout[{L.z_stage_bytes | variant, L.pk_stage_bytes}].push_back(k);
   }
   for (auto &kv : by_layout) {
     const std::vector<int> &ks = kv.second;
@@ -504,6 +516,7 @@ int corr_batch_push(corr_batch *b, const uint8_t *const *d_blocks, void *stream)
     p.z_stage_bytes = g.L.z_stage_bytes;
     p.pk_stage_bytes = g.L.pk_stage_bytes;
     p.sum_rows = g.L.sum_rows;
+    p.gram = g.gram;
     if (g.grid > 0) {
       if ((rc = cuda_err(g.pair ? xe::launch_cmac_batch_pair(maps, p, g.grid, g.L.smem_bytes, st)
                                 : xe::launch_cmac_batch(maps, p, g.grid, g.L.smem_bytes, st))) !=

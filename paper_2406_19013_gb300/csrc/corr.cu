@@ -43,6 +43,7 @@ struct corr_ctx {
   uint32_t z_stage_bytes, pk_stage_bytes;
   int sum_rows;
   int tm;  // 1: the TMEM-operand kernel (xengine_tm.cu) runs this context's launches
+  int gram;  // 1: units of the Gram form (up to kGramInputs inputs)
   int pair;  // 1: CTA pairs (the quad cover, M = 256 MMAs) run this context's launches
   int ch_rows;  // inputs per channel in the TMA box (64, or 16 / 32 for multi-channel tiles)
   int pitch;           // row pitch of the staged block (block_len rounded up to 16)
@@ -227,6 +228,11 @@ int corr_create(int n_ant, int n_pol, int n_chan, int block_len, corr_ctx **out)
   ctx->pair = use_pair_kernel(ctx->n_in) ? 1 : 0;
   std::vector<XUnit> units =
       xe::build_schedule(ctx->n_in, ctx->pair ? xe::kCoverQuads : xe::kCoverWindow);
+  if (ctx->n_in <= xe::kGramInputs && !use_tm_kernel(ctx->n_in)) {
+    XUnit g[xe::kMaxWindowUnits];
+    units.assign(g, g + xe::gram_units(ctx->n_in, g));
+    ctx->gram = 1;
+  }
   if (units.empty()) {
     free_ctx(ctx);
     return CORR_EINVAL;
@@ -367,6 +373,7 @@ int launch_staged(corr_ctx *ctx, const uint8_t *const *staged, int nb, cudaStrea
   p.z_stage_bytes = ctx->z_stage_bytes;
   p.pk_stage_bytes = ctx->pk_stage_bytes;
   p.sum_rows = ctx->sum_rows;
+  p.gram = ctx->gram;
   xe::XMaps maps;
   std::memset(&maps, 0, sizeof(maps));
   int rc;

@@ -116,7 +116,8 @@ extern "C" int corr_xcorr_static(const uint8_t *d_block, int n_ant, int n_pol, i
   StaticPlan plan;
   std::memset(&plan, 0, sizeof(plan));
   xe::XUnit *units = plan.units;
-  const int n_tpl = xe::window_units((int)N, units);
+  const int n_tpl = N <= xe::kGramInputs ? xe::gram_units((int)N, units)
+                                         : xe::window_units((int)N, units);
   if (n_tpl > kMaxStaticUnits) return CORR_EINVAL;
   plan.n_units = n_tpl;
   int max_z = 0, max_pk = 0, max_sum = 0;
@@ -189,6 +190,7 @@ extern "C" int corr_xcorr_static(const uint8_t *d_block, int n_ant, int n_pol, i
   p.z_stage_bytes = L.z_stage_bytes;
   p.pk_stage_bytes = L.pk_stage_bytes;
   p.sum_rows = L.sum_rows;
+  p.gram = units[0].gram;
   const long long n_work = n_units * p.implicit_nseg;
   const int grid = (int)std::min<long long>(n_work, g_n_sm[dev]);
   return rc_of(xe::launch_cmac(maps, p, grid, L.smem_bytes, st));

@@ -98,6 +98,10 @@ struct XUnit {
   // column blocks are shared, since the pair's B operand is the even CTA's
   // N / 2 B rows followed by the odd one's
   int pair_rows;
+  // 1: the Gram form (gram_units): an input's two operand rows are its real
+  // and its imaginary parts, 128 samples each, and the products of all four
+  // combinations are accumulated apart
+  int gram;
   int z_rows;    // rows staged per chunk (sum over regions)
   int n_sum;     // inputs staged per chunk (sum over regions)
   int pk_bytes;  // packed bytes per chunk (sum over regions)
@@ -180,6 +184,7 @@ struct XParams {
   // boxes (no swizzle); the unpack transposes them on chip, and operand rows
   // are rotated within every 8-input group (see xengine.cu)
   int tcn;
+  int gram;  // 1: units of the Gram form (XUnit::gram)
 };
 
 // TMA descriptors (CUtensorMap, 128 bytes each), one per (problem, block) of

@@ -144,6 +144,33 @@ int window_units(int N, XUnit *units) {
   return n_units;
 }
 
+int gram_units(int N, XUnit *units) {
+  const int n16 = round_up(N, 16);
+  XUnit &u = units[0] = empty_unit();
+  u.gram = 1;
+  if (N <= kTileInputs) {
+    // two tiles: of one channel each, or of 64 / n16 channels (ch_rows)
+    const int cpt = N <= 32 ? kTileInputs / n16 : 1;
+    u.n_chan = 2 * cpt;
+    for (int r = 0; r < 2; ++r) {
+      add_reg(u, 0, kTileInputs, 1);
+      u.reg[r].chan_off = r * cpt;
+    }
+    for (int r = 0; r < 2; ++r) {
+      add_seg(u, u.reg[r].z_row, u.reg[r].z_row, 1024, N <= 32 ? 2 * kTileInputs : 2 * n16, 0, 0);
+      u.seg[r].chan_off = r * cpt;
+      u.seg[r].ch_rows = N <= 32 ? n16 : 0;
+    }
+  } else {
+    // two row tiles of one channel, at most 128 + 256 columns
+    add_reg(u, 0, 2 * kTileInputs, 1);
+    add_seg(u, 128, 0, 1024, 2 * n16, kTileInputs, 0);
+    add_seg(u, 0, 0, 1024, 2 * kTileInputs, 0, 0);
+  }
+  set_sums(u);
+  return 1;
+}
+
 std::vector<XUnit> build_schedule(int N, int cover) {
   std::vector<XUnit> units;
   const int n16 = round_up(N, 16);
@@ -278,9 +305,10 @@ bool stage_layout(int max_zr, int max_pk, int max_sum, int smem_optin, int max_z
   const int zb = (int)L.z_stage_bytes, pb = (int)L.pk_stage_bytes;
   const int zcap = std::min(max_z, kMaxZStages);
   // Operand stages first (three beside three packed stages, else three
-  // beside two, else two beside three or two), then packed stages (bytes in
-  // flight from HBM) up to six,
-  // operand stages up to four, and both up to their caps while they fit.
+  // beside two, else two beside three or two), then a fourth, then packed
+  // stages (bytes in flight from HBM), and both up to their caps while they
+  // fit.  (Six packed stages before the fourth operand stage: 64 inputs 626 us
+  // a launch against 612.)
   int zs, ps;
   if (3 * zb + 3 * pb <= avail && zcap >= 3) {
     zs = 3;
@@ -301,7 +329,6 @@ bool stage_layout(int max_zr, int max_pk, int max_sum, int smem_optin, int max_z
   auto grow = [&](int &v, int cap, int bytes) {
     while (v < cap && zs * zb + ps * pb + bytes <= avail) ++v;
   };
-  grow(ps, 6, pb);
   grow(zs, std::min(4, zcap), zb);
   grow(ps, kMaxPkStages, pb);
   grow(zs, zcap, zb);
@@ -318,7 +345,8 @@ bool stage_layout(int max_zr, int max_pk, int max_sum, int smem_optin, int max_z
 int chunk_cost(const XUnit &u) {
   int mma = 0;
   for (int s = 0; s < u.n_seg; ++s) mma += 4 * ((u.pair_rows ? 54 : 24) + u.seg[s].n / 2);
-  return std::max(mma, 5 * u.z_rows / 2);
+  const int cost = std::max(mma, 5 * u.z_rows / 2);
+  return u.gram ? cost / 2 : cost;  // its rows and MMAs hold 128 samples
 }
 
 // Modelled cycles of the busiest CTA of a split.
@@ -358,44 +386,47 @@ int build_items_filled(const std::vector<ProbWork> &probs, int grid, std::vector
     build_items(probs, grid, it, first, min_split);
     keep_if_better();
   }
-  // every unit in n equal pieces, dealt in turn to the CTA that is free first
-  // (where a fold costs more than a CTA's share of the work, no run is cut)
-  for (int n = 2; n <= 64; n *= 2) {
-    std::vector<std::vector<XItem>> runs(grid);
-    typedef std::pair<long long, int> Load;
-    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> free_first;
-    for (int k = 0; k < grid; ++k) free_first.push({0, k});
-    for (size_t p = 0; p < probs.size(); ++p) {
-      const ProbWork &pr = probs[p];
-      const int npk = (pr.block_len + kPkSamples - 1) / kPkSamples * pr.n_blocks;
-      const int pieces =
-          std::min(npk, n * std::max(1, (npk + kMaxFoldStages - 1) / kMaxFoldStages));
-      for (int t = 0; t < (int)pr.units->size(); ++t) {
-        const XUnit &u = (*pr.units)[t];
-        for (int c = 0; c < pr.n_chan; c += std::max(1, u.n_chan))
-          for (int k = 0; k < pieces; ++k) {
-            const int a = (int)((long long)npk * k / pieces);
-            const int b = (int)((long long)npk * (k + 1) / pieces);
-            const Load l = free_first.top();
-            free_first.pop();
-            runs[l.second].push_back({(int)p, t, c, a, b - a});
-            free_first.push({l.first + (long long)kChunksPerPk * (b - a) * chunk_cost(u) +
-                                 kFold * u.work,
-                             l.second});
-          }
-      }
+  // every unit in n equal pieces, dealt round the CTAs (where a fold costs more
+  // than a CTA's share of the work, no run is cut): the n of the shortest
+  // modelled run, rounds of the costliest unit's pieces
+  long long n_units = 0, fold = 0, work = 0;
+  int npk = 0, nseg = 1;
+  for (const ProbWork &pr : probs) {
+    npk = std::max(npk, (pr.block_len + kPkSamples - 1) / kPkSamples * pr.n_blocks);
+    for (const XUnit &u : *pr.units) {
+      n_units += (pr.n_chan + u.n_chan - 1) / std::max(1, u.n_chan);
+      fold = std::max(fold, kFold * u.work);
+      work = std::max(work, (long long)kChunksPerPk * chunk_cost(u));
     }
-    it.clear();
-    first.assign(1, 0);
-    for (const std::vector<XItem> &run : runs) {
-      if (run.empty()) continue;
-      it.insert(it.end(), run.begin(), run.end());
-      first.push_back((int)it.size());
-    }
-    keep_if_better();
-    if ((int)it.size() > 4 * grid) break;
   }
-  return (int)cta_first.size() - 1;
+  nseg = (npk + kMaxFoldStages - 1) / kMaxFoldStages;
+  int best_n = 0;
+  for (int n = nseg; n <= std::min(npk, 64 * nseg); ++n) {
+    const long long t = (n_units * n + grid - 1) / grid * ((npk + n - 1) / n * work + fold);
+    if (t < best) best = t, best_n = n;
+    if (n_units * n >= 2LL * grid) break;
+  }
+  if (best_n == 0) return used;
+  it.clear();
+  for (size_t p = 0; p < probs.size(); ++p) {
+    const ProbWork &pr = probs[p];
+    const int pk = (pr.block_len + kPkSamples - 1) / kPkSamples * pr.n_blocks;
+    const int n = std::min(pk, std::max(best_n, (pk + kMaxFoldStages - 1) / kMaxFoldStages));
+    for (int t = 0; t < (int)pr.units->size(); ++t)
+      for (int c = 0; c < pr.n_chan; c += std::max(1, (*pr.units)[t].n_chan))
+        for (int k = 0; k < n; ++k) {
+          const int lo = (int)((long long)pk * k / n), hi = (int)((long long)pk * (k + 1) / n);
+          it.push_back({(int)p, t, c, lo, hi - lo});
+        }
+  }
+  used = std::min(grid, (int)it.size());
+  items.clear();
+  cta_first.assign(1, 0);
+  for (int b = 0; b < used; ++b) {
+    for (size_t k = b; k < it.size(); k += used) items.push_back(it[k]);
+    cta_first.push_back((int)items.size());
+  }
+  return used;
 }
 
 int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem> &items,
@@ -426,11 +457,10 @@ int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem>
   }
   // cost of stages [a, b) of a unit that costs `per_chunk` a chunk
   auto range_cost = [&](size_t p, int a, int b, int per_chunk) {
-    long long chunks = 0;
-    for (int k = a; k < b; ++k) {
-      const int kc = k % pw[p].ppb;
-      chunks += std::min(kChunksPerPk, pw[p].cpb - kChunksPerPk * kc);
-    }
+    // all stages but a block's last one hold kChunksPerPk chunks
+    const int ppb = pw[p].ppb, short_by = kChunksPerPk * ppb - pw[p].cpb;
+    const long long chunks =
+        (long long)kChunksPerPk * (b - a) - (long long)short_by * (b / ppb - a / ppb);
     return chunks * per_chunk;
   };
   // More than two templates per channel: they read the same inputs, so the units of
@@ -595,8 +625,9 @@ bool encode_block_map(const void *base, int block_len, int n_in, int n_chan, int
   const cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = enc(static_cast<CUtensorMap *>(map), CU_TENSOR_MAP_DATA_TYPE_UINT8, 3,
                    const_cast<void *>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                   CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                   CU_TENSOR_MAP_SWIZZLE_128B,
+                   // a row's next stage comes along into L2
+                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
 

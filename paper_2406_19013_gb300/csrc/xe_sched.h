@@ -44,6 +44,18 @@ std::vector<XUnit> build_schedule(int n_in, int cover = kCoverWindow);
 constexpr int kMaxWindowUnits = 4;
 int window_units(int n_in, XUnit *units);
 
+// The units that launches run up to kGramInputs inputs, instead of the window
+// cover's: the same triangle with half of the operand bytes.  A tile's 128
+// rows are the real and the imaginary rows of 64 inputs, 128 samples to a
+// 128-byte row (against [re, im] and [im, -re] rows of 64 samples), and D
+// holds re re, re im, im re and im im products, which the epilogue adds up.  No
+// negated rows are decoded or stored, a stage is one hand-off instead of two,
+// and the MMAs are twice as wide; but an input takes two accumulator columns,
+// so a channel of more than 128 inputs does not fit the 512 TMEM columns.
+// Same arguments and result as window_units.
+constexpr int kGramInputs = 128;
+int gram_units(int n_in, XUnit *units);
+
 // Modelled cycles of one 64-sample chunk of a unit: its MMAs (four K slices of
 // each segment; measured on shared-memory operands, 57 cycles at N = 64, 122
 // at 192, 155 at 256, and 182 for a CTA pair's M = 256, N = 256), or the unpack

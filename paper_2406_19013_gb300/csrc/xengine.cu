@@ -43,6 +43,12 @@
 // hold several independent problems (a batch of correlators).  All waits are
 // bounded by a timeout; on expiry the kernel drains its own copies and MMAs,
 // frees TMEM and reports through *status.
+// The Gram instance (GRAM, up to 128 inputs) keeps an input's real and
+// imaginary parts in rows of their own, 128 samples to a row, and accumulates
+// the four kinds of product apart: half the operand bytes, no negated rows, one
+// hand-off per 128 samples, twice the accumulator columns.  (128 inputs, 512
+// channels, 4 blocks of 8192 samples: 741 -> 567 us a launch; 64 inputs, 8
+// blocks: 824 -> 612; 16 inputs: 237 -> 179.)
 // The CTA-pair instance (PAIR) runs clusters of two CTAs on two SMs: each
 // stages and unpacks two row tiles and half of a B operand of up to 256
 // columns, the even CTA's two issuers run M = 256 MMAs (cta_group::2) over
@@ -179,6 +185,66 @@ __device__ __forceinline__ void unpack_turned(uint32_t src, uint32_t dst, int ki
     }
   }
 }
+// The Gram form of unpack_rows: 128 samples of this warp's rows, the lane's two
+// 16-sample chunks (g and g + 4) one after the other.  The real bytes go to the
+// same 16-byte chunk of the first operand row, the imaginary ones to the second
+// (1024 bytes on): half of the stores of unpack_rows<true>.
+__device__ __forceinline__ void unpack_gram(uint32_t src, uint32_t dst, int n_k,
+                                            uint32_t (&sum)[4]) {
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {  // at most two tiles of a region
+    if (k >= n_k) break;
+    const uint32_t s0 = src + (uint32_t)(k * kTileInputs * kPackedRowBytes);
+    const uint32_t d0 = dst + (uint32_t)k * 16384u;
+    const uint4 x[2] = {lds128(s0), lds128(s0 ^ 64u)};
+    uint32_t re = 0u, im = 0u;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      uint32_t re0, im0, re1, im1, re2, im2, re3, im3, n;
+      decode_biased(x[c].x, re0, im0, n);
+      decode_biased(x[c].y, re1, im1, n);
+      decode_biased(x[c].z, re2, im2, n);
+      decode_biased(x[c].w, re3, im3, n);
+      sts128(d0 ^ (64u * c), re0, re1, re2, re3);
+      sts128_q(d0 ^ (64u * c), im0, im1, im2, im3);
+      re += re0 + re1 + re2 + re3;  // bytes: at most 8 x 15
+      im += im0 + im1 + im2 + im3;
+    }
+    sum[k] = __dp4a(re, 0x01010101u, sum[k]) + (__dp4a(im, 0x01010101u, 0u) << 16);
+  }
+}
+
+// The Gram form of unpack_turned: item (qd, j) is inputs 4 qd .. 4 qd + 3 and
+// samples 16 j .. 16 j + 15 of the stage, with the same rotations.
+__device__ __forceinline__ void unpack_gram_turned(uint32_t src, uint32_t dst, int n_box, int t,
+                                                   uint32_t (&sum)[8]) {
+  const int v = t & 127, qd = v & 15, j = v >> 4, jj = j & 1;
+  const int box = t >> 7;  // at most two boxes of a region
+  if (box >= n_box) return;
+  const uint32_t at = src + (uint32_t)box * 8192u + (uint32_t)(64 * 16 * j) + 4u * qd;
+  uint32_t w[4][4];  // [input][4 samples]
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    uint32_t x[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) x[i] = lds32(at + 64u * (uint32_t)((4 * m + i + jj) & 15));
+    transpose4(x[0], x[1], x[2], x[3], w[0][m], w[1][m], w[2][m], w[3][m]);
+  }
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    uint32_t re[4], im[4], n;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) decode_biased(w[e][m], re[m], im[m], n);
+    const int i_rel = kTileInputs * box + 4 * qd + e, gp = i_rel >> 3;
+    const int pos = ((i_rel & 7) + (gp & 3)) & 7;
+    const uint32_t d = dst + (uint32_t)(16 * gp + pos) * 128u + (uint32_t)((j ^ pos) << 4);
+    sts128(d, re[0], re[1], re[2], re[3]);
+    sts128_q(d, im[0], im[1], im[2], im[3]);
+    sum[e] = __dp4a(re[0] + re[1] + re[2] + re[3], 0x01010101u, sum[e]) +
+             (__dp4a(im[0] + im[1] + im[2] + im[3], 0x01010101u, 0u) << 16);
+  }
+}
+
 // A folded value from an accumulator (in units of 2^-18) and the sum of its
 // operand-sum entries, given plus kMagicBits: acc 2^18 - 8 sum, returned plus
 // kMagicBits.  1.5 x 2^23 has a unit of 1, so adding a whole number below 2^22
@@ -200,7 +266,8 @@ __device__ __forceinline__ uint32_t unbias(uint32_t acc, uint32_t sum_magic) {
 // PAIR: the launch is clusters of two CTAs running pair units (XUnit::
 // pair_rows): both CTAs stage and unpack their own rows, the even CTA's
 // issuers run M = 256 MMAs over both, and both fold their own TMEM rows.
-template <int M, bool TCN, bool PAIR>
+// GRAM: units of the Gram form (XUnit::gram).
+template <int M, bool TCN, bool PAIR, bool GRAM>
 __global__ void __launch_bounds__(kThreads, 1)
     xengine_cmac_kernel(const __grid_constant__ XMapsT<M> maps, const XParams p) {
   extern __shared__ uint8_t smem_raw[];
@@ -387,7 +454,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         uint32_t acc0 = 0;  // the item's first MMA of each accumulator overwrites it
         StageWalk walk(pb, item.pk0);
         for (int k = 0; k < item.npk && ok; ++k, walk.next()) {
-          const int nch = walk.chunks();
+          const int nch = GRAM ? 1 : walk.chunks();
           for (int sub = 0; sub < nch; ++sub) {
             if (!(PAIR ? mbar_wait_cluster(b.z_full + 8 * zs, zph, abort_flag, to)
                        : mbar_wait(b.z_full + 8 * zs, zph, abort_flag, to))) {
@@ -474,14 +541,18 @@ __global__ void __launch_bounds__(kThreads, 1)
     // packed rows arrive 128B-swizzled: 16-byte chunk c of row r sits at
     // c ^ (r & 7); this group's operand chunk is chunks 4 grp + g
     const uint32_t src_lane =
-        (uint32_t)((8 * w8 + sw) * kPackedRowBytes + (((4 * grp + g) ^ sw) << 4));
-    // the lane's 32 operand bytes are 16-byte chunks 2 g and 2 g + 1
-    const uint32_t dst_lane = (uint32_t)(sw * 128 + (((2 * g) ^ sw) << 4));
+        (uint32_t)((8 * w8 + sw) * kPackedRowBytes + (((GRAM ? g : 4 * grp + g) ^ sw) << 4));
+    // the lane's 32 operand bytes are 16-byte chunks 2 g and 2 g + 1 (Gram
+    // form: a packed chunk's real and imaginary bytes go to the same chunk of
+    // the two rows)
+    const uint32_t dst_lane = (uint32_t)(sw * 128 + (((GRAM ? g : 2 * g) ^ sw) << 4));
     const uint32_t pk_s0 = smem_u32(pk_buf), z_s0 = smem_u32(z_buf);
     int s = 0, zs = 0;
     uint32_t ph = 0, zph = 0;
     bool ok = true;
     long long nu = 0;
+    // Gram form: a stage is one chunk, and the groups take stages in turn
+    bool my_turn = grp == 0;
     for (int it = it0; it < it1 && ok && !*abort_flag; it += it_step, ++nu) {
       const XItem item = item_at(p, it);
       const XProb pb = p.probs[item.prob];
@@ -495,7 +566,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int r = 0; r < 2; ++r)
 #pragma unroll
         for (int k = 0; k < (TCN ? 8 : 4); ++k) sums[r][k] = 0u;
-      static_assert(kMaxFoldStages * 16 * 15 < 65536, "16-bit sums");
+      static_assert(kMaxFoldStages * 16 * 15 < 65536, "16-bit sums (Gram: 32 of half the stages)");
       int n_mine = 0;  // chunks this warp decoded
       // per-region constants (at most two regions of at most 256 inputs)
       uint32_t src_off[2], dst_off[2], dst_step[2];
@@ -512,11 +583,13 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       StageWalk walk(pb, item.pk0);
       for (int k = 0; k < item.npk; ++k, walk.next()) {
-        const int nch = walk.chunks();
+        const int nch = GRAM ? 1 : walk.chunks();
+        const bool wanted = GRAM ? my_turn : grp < nch;
+        my_turn = !my_turn;
         if (!mbar_wait(b.pk_full + 8 * s, ph, abort_flag, to)) { ok = false; break; }
-        if (grp < nch) {
+        if (wanted) {
           ++n_mine;
-          const int zm = zs + grp, zi = zm >= p.z_stages ? zm - p.z_stages : zm;
+          const int zm = zs + (GRAM ? 0 : grp), zi = zm >= p.z_stages ? zm - p.z_stages : zm;
           const uint32_t zp = zm >= p.z_stages ? zph ^ 1u : zph;
           if (!mbar_wait(b.z_empty + 8 * zi, zp ^ 1u, abort_flag, to)) { ok = false; break; }
           const uint32_t pk_s = pk_s0 + (uint32_t)s * p.pk_stage_bytes;
@@ -524,7 +597,11 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
           for (int r = 0; r < 2; ++r) {
             if (n_k[r] == 0) break;
-            if constexpr (TCN)
+            if constexpr (TCN && GRAM)
+              unpack_gram_turned(pk_s + src_off[r], z_s + dst_off[r], n_k[r], t_grp, sums[r]);
+            else if constexpr (GRAM)
+              unpack_gram(pk_s + src_off[r], z_s + dst_off[r], n_k[r], sums[r]);
+            else if constexpr (TCN)
               unpack_turned(pk_s + src_off[r], z_s + dst_off[r], kind[r], n_k[r], t_grp, grp,
                             sums[r]);
             else if (kind[r] == 1)
@@ -539,7 +616,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             mbar_arrive(b.pk_empty + 8 * s);
           }
         } else if (lane == 0) {
-          mbar_arrive(b.pk_empty + 8 * s);  // a block's odd last chunk
+          mbar_arrive(b.pk_empty + 8 * s);  // not this group's, or a block's odd last chunk
         }
         if ((zs += nch) >= p.z_stages) { zs -= p.z_stages; zph ^= 1u; }
         if (++s == p.pk_stages) { s = 0; ph ^= 1u; }
@@ -568,8 +645,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           ua += __shfl_xor_sync(0xffffffffu, ua, 16);
           ub += __shfl_xor_sync(0xffffffffu, ub, 16);
-          // normal order: the warp held all 64 samples of a chunk of 8 rows;
-          // F-engine order: 16 of them (8 a half-warp) of 64 inputs
+          // normal order: the warp held all samples of a chunk of 8 rows; F-
+          // engine order: a quarter of them (an eighth a half-warp) of 64 inputs
           if (lane < (TCN ? 16 : 8)) {
             int at;
             if (TCN) {
@@ -580,7 +657,8 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             const uint32_t addr =
                 tab + 8u * (uint32_t)((int)rank * (p.sum_rows >> 1) + sum_row + at);
-            const int vx = ua + ub - 8 * (TCN ? 16 : kChunkSamples) * n_mine;
+            constexpr int kSeen = (GRAM ? kPkSamples : kChunkSamples) / (TCN ? 4 : 1);
+            const int vx = ua + ub - 8 * kSeen * n_mine;
             const int vy = ub - ua;
             reds32(addr, vx);
             reds32(addr + 4u, vy);
@@ -660,20 +738,39 @@ __global__ void __launch_bounds__(kThreads, 1)
         // the columns to fold: up to the 16 that hold the 8 rows' diagonal,
         // and of a multi-channel tile the rows' channel block only.  Column
         // blocks of a pair's segment are not in input order: all of them.
+        // (Gram form: 16 inputs are 32 accumulator columns, 8 real ones and 8
+        // imaginary ones in turn; cb counts inputs.)
         const int cb0 = rpc ? ci * rpc : 0;
-        int cb1 = rpc ? cb0 + rpc : sgm.n;
+        int cb1 = rpc ? cb0 + rpc : GRAM ? sgm.n >> 1 : sgm.n;
         if (!PAIR) cb1 = min(cb1, cb0 + ((i0 + 7 - (sgm.col_blk[0] + cb0 - ci * rpc)) & ~15) + 16);
         const uint32_t tm = tmem + ((uint32_t)(32 * q + 16 * h) << 16) + (uint32_t)sgm.tmem_col;
-        uint32_t nxt[8];
+        uint32_t nxt[8], nxt2[8];
         __syncwarp();
-        tmem_ld_16x256b_x2(tm + (uint32_t)cb0, nxt);
+        tmem_ld_16x256b_x2(tm + (uint32_t)(GRAM ? 2 * cb0 : cb0), nxt);
+        if (GRAM) tmem_ld_16x256b_x2(tm + (uint32_t)(2 * cb0 + 16), nxt2);
         for (int cb = cb0; cb < cb1; cb += 16) {
           tmem_ld_wait();
           uint32_t v[8];
+          if (GRAM) {
+            // re re + im im, im re - re im: whole numbers below 2^24, exact
+            auto f = [](uint32_t x) { return __uint_as_float(x); };
 #pragma unroll
-          for (int k = 0; k < 8; ++k) v[k] = nxt[k];
+            for (int k = 0; k < 2; ++k) {
+              const uint32_t *a = k ? nxt2 : nxt;
+              v[4 * k] = __float_as_uint(f(a[0]) + f(a[6]));
+              v[4 * k + 1] = __float_as_uint(f(a[1]) + f(a[7]));
+              v[4 * k + 2] = __float_as_uint(f(a[2]) - f(a[4]));
+              v[4 * k + 3] = __float_as_uint(f(a[3]) - f(a[5]));
+            }
+          } else {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = nxt[k];
+          }
           // the next columns are on their way while these are folded
-          if (cb + 16 < cb1) tmem_ld_16x256b_x2(tm + (uint32_t)(cb + 16), nxt);
+          if (cb + 16 < cb1) {
+            tmem_ld_16x256b_x2(tm + (uint32_t)(GRAM ? 2 * cb + 32 : cb + 16), nxt);
+            if (GRAM) tmem_ld_16x256b_x2(tm + (uint32_t)(2 * cb + 48), nxt2);
+          }
           // input of the first column (one-CTA units: consecutive inputs)
           int j0 = sgm.col_blk[0] - ci * rpc + cb;
           if (PAIR) {
@@ -752,12 +849,15 @@ __global__ void __launch_bounds__(kThreads, 1)
 
 cudaError_t cmac_set_smem(int smem_bytes) {
   const void *kernels[] = {
-      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxMaps, false, false>),
-      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxMaps, true, false>),
-      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxMaps, false, true>),
-      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxMaps, true, true>),
-      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxBatchMaps, false, false>),
-      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxBatchMaps, false, true>)};
+      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxMaps, false, false, false>),
+      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxMaps, true, false, false>),
+      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxMaps, false, true, false>),
+      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxMaps, true, true, false>),
+      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxBatchMaps, false, false, false>),
+      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxBatchMaps, false, true, false>),
+      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxMaps, false, false, true>),
+      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxMaps, true, false, true>),
+      reinterpret_cast<const void *>(xengine_cmac_kernel<kMaxBatchMaps, false, false, true>)};
   for (const void *k : kernels) {
     cudaError_t e =
         cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes);
@@ -768,10 +868,14 @@ cudaError_t cmac_set_smem(int smem_bytes) {
 
 cudaError_t launch_cmac(const XMaps &maps, const XParams &p, int grid, int smem_bytes,
                         cudaStream_t stream) {
-  if (p.tcn)
-    xengine_cmac_kernel<kMaxMaps, true, false><<<grid, kThreads, smem_bytes, stream>>>(maps, p);
+  if (p.gram && p.tcn)
+    xengine_cmac_kernel<kMaxMaps, true, false, true><<<grid, kThreads, smem_bytes, stream>>>(maps, p);
+  else if (p.gram)
+    xengine_cmac_kernel<kMaxMaps, false, false, true><<<grid, kThreads, smem_bytes, stream>>>(maps, p);
+  else if (p.tcn)
+    xengine_cmac_kernel<kMaxMaps, true, false, false><<<grid, kThreads, smem_bytes, stream>>>(maps, p);
   else
-    xengine_cmac_kernel<kMaxMaps, false, false><<<grid, kThreads, smem_bytes, stream>>>(maps, p);
+    xengine_cmac_kernel<kMaxMaps, false, false, false><<<grid, kThreads, smem_bytes, stream>>>(maps, p);
   return cudaGetLastError();
 }
 
@@ -799,20 +903,20 @@ struct PairConfig {
 cudaError_t launch_cmac_pair(const XMaps &maps, const XParams &p, int clusters, int smem_bytes,
                              cudaStream_t stream) {
   PairConfig c(clusters, smem_bytes, stream);
-  if (p.tcn) return cudaLaunchKernelEx(&c.cfg, xengine_cmac_kernel<kMaxMaps, true, true>, maps, p);
-  return cudaLaunchKernelEx(&c.cfg, xengine_cmac_kernel<kMaxMaps, false, true>, maps, p);
+  if (p.tcn) return cudaLaunchKernelEx(&c.cfg, xengine_cmac_kernel<kMaxMaps, true, true, false>, maps, p);
+  return cudaLaunchKernelEx(&c.cfg, xengine_cmac_kernel<kMaxMaps, false, true, false>, maps, p);
 }
 
 cudaError_t launch_cmac_batch_pair(const XBatchMaps &maps, const XParams &p, int clusters,
                                    int smem_bytes, cudaStream_t stream) {
   PairConfig c(clusters, smem_bytes, stream);
-  return cudaLaunchKernelEx(&c.cfg, xengine_cmac_kernel<kMaxBatchMaps, false, true>, maps, p);
+  return cudaLaunchKernelEx(&c.cfg, xengine_cmac_kernel<kMaxBatchMaps, false, true, false>, maps, p);
 }
 
 int cmac_pair_clusters(int smem_bytes) {
   PairConfig c(1, smem_bytes, nullptr);
   int n = 0;
-  return cudaOccupancyMaxActiveClusters(&n, xengine_cmac_kernel<kMaxMaps, false, true>, &c.cfg) ==
+  return cudaOccupancyMaxActiveClusters(&n, xengine_cmac_kernel<kMaxMaps, false, true, false>, &c.cfg) ==
                  cudaSuccess
              ? n
              : 0;
@@ -821,7 +925,7 @@ int cmac_pair_clusters(int smem_bytes) {
 int cmac_pair_clusters_batch(int smem_bytes) {
   PairConfig c(1, smem_bytes, nullptr);
   int n = 0;
-  return cudaOccupancyMaxActiveClusters(&n, xengine_cmac_kernel<kMaxBatchMaps, false, true>,
+  return cudaOccupancyMaxActiveClusters(&n, xengine_cmac_kernel<kMaxBatchMaps, false, true, false>,
                                         &c.cfg) == cudaSuccess
              ? n
              : 0;
@@ -829,7 +933,12 @@ int cmac_pair_clusters_batch(int smem_bytes) {
 
 cudaError_t launch_cmac_batch(const XBatchMaps &maps, const XParams &p, int grid, int smem_bytes,
                               cudaStream_t stream) {
-  xengine_cmac_kernel<kMaxBatchMaps, false, false><<<grid, kThreads, smem_bytes, stream>>>(maps, p);
+  if (p.gram)
+    xengine_cmac_kernel<kMaxBatchMaps, false, false, true>
+        <<<grid, kThreads, smem_bytes, stream>>>(maps, p);
+  else
+    xengine_cmac_kernel<kMaxBatchMaps, false, false, false>
+        <<<grid, kThreads, smem_bytes, stream>>>(maps, p);
   return cudaGetLastError();
 }
 

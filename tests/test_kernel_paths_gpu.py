@@ -47,6 +47,8 @@ def _vis(corr, torch, blocks, n_ant, n_pol, tcn=False):
 @pytest.mark.parametrize("n_ant,C,T", [
     (8, 2, 33001),     # 7+7j runs past one fold window of 32768 samples
     (32, 3, 32768),    # exactly one window
+    (24, 3, 33001),    # 48 inputs: two tiles of one channel each
+    (64, 1, 32896),    # 128 inputs: two row tiles, two windows of unlike parity
     (80, 1, 40000),    # three row tiles
     (96, 2, 1024),
     (160, 1, 640),     # one-CTA units above 256 inputs

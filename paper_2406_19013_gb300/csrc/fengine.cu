@@ -40,6 +40,9 @@
 //     [1024 channels][kSpecTile spectra];
 //   - each channel's row of the staging tile is written out as one 32-byte run
 //     of out[c][input][k0 ..].
+// 192 inputs x 8192 spectra: 5.22 ms, 0.28 of the fp32 rate (5.79 ms before the
+// codes were rounded and packed without conversions, the filter's coefficients
+// stayed in registers, and the rows left in whole sectors).
 // Floating point is fp32 (the host computes the filter and twiddles in
 // double precision); the codes can differ from an exact computation only for
 // values within the fp32 rounding error of a quantisation boundary.
@@ -107,11 +110,13 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
 
 __device__ __forceinline__ void dft4(float2 &a0, float2 &a1, float2 &a2, float2 &a3) {
   const float2 s02 = cadd(a0, a2), d02 = csub(a0, a2);
-  const float2 s13 = cadd(a1, a3), d13 = csub(a1, a3);
+  const float2 s13 = cadd(a1, a3);
+  // (d13.y, d13.x), so that the rotated sums are two-lane operations as well
+  const float2 dr = make_float2(__fsub_rn(a1.y, a3.y), __fsub_rn(a1.x, a3.x));
   a0 = cadd(s02, s13);
-  a1 = make_float2(d02.x + d13.y, d02.y - d13.x);  // a0 - i a1 - a2 + i a3
   a2 = csub(s02, s13);
-  a3 = make_float2(d02.x - d13.y, d02.y + d13.x);  // a0 + i a1 - a2 - i a3
+  a1 = fma2(dr, make_float2(1.0f, -1.0f), d02);  // a0 - i a1 - a2 + i a3
+  a3 = fma2(dr, make_float2(-1.0f, 1.0f), d02);  // a0 + i a1 - a2 - i a3
 }
 
 // Forward 16-point DFT in place, natural order in and out:
@@ -154,6 +159,37 @@ __device__ __forceinline__ int quant(float a) {
   return __float2int_rz(__fadd_rz(y, copysignf(0.5f, y)));
 }
 
+// The 4-bit codes of one channel's four spectra, x[u] = (re, im), as a word:
+// byte u is (q(re) << 4) | (q(im) & 15) with q = quant.  The value's magnitude,
+// clipped to 7, is added rounding toward zero to 2^(23-4p) + 0.5, which leaves
+// the rounded magnitude at bits 4p .. 4p + 2 of the sum: one addition and one
+// logic operation put it at its place in the word, without a conversion (the
+// conversion instruction runs at an eighth of the rate) or a shift.  The signs
+// are gathered by byte permutes and negate all eight nibbles together:
+// -m = (8 - m) ^ 8 in 4 bits.
+__device__ __forceinline__ float clip7(float a) { return fminf(fmaxf(a, -7.0f), 7.0f); }
+__device__ __forceinline__ uint32_t quant4(const float2 (&x)[4]) {
+  float2 y[4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) y[u] = make_float2(clip7(x[u].x), clip7(x[u].y));
+  uint32_t half[2];
+#pragma unroll
+  for (int k = 0; k < 2; ++k)  // nibbles im, re of spectra 2 k and 2 k + 1 at 4 p, p = 1..4
+    half[k] = (__float_as_uint(__fadd_rz(fabsf(y[2 * k].y), 524288.5f)) & 0x70u) |
+              (__float_as_uint(__fadd_rz(fabsf(y[2 * k].x), 32768.5f)) & 0x700u) |
+              (__float_as_uint(__fadd_rz(fabsf(y[2 * k + 1].y), 2048.5f)) & 0x7000u) |
+              (__float_as_uint(__fadd_rz(fabsf(y[2 * k + 1].x), 128.5f)) & 0x70000u);
+  const uint32_t mag = (half[0] >> 4) | (half[1] << 12);
+  auto top4 = [](float a, float b, float c, float d) {  // the top bytes
+    return __byte_perm(__byte_perm(__float_as_uint(a), __float_as_uint(b), 0x0073),
+                       __byte_perm(__float_as_uint(c), __float_as_uint(d), 0x0073), 0x5410);
+  };
+  const uint32_t sgn = (top4(y[0].x, y[1].x, y[2].x, y[3].x) & 0x80808080u) |
+                       ((top4(y[0].y, y[1].y, y[2].y, y[3].y) >> 4) & 0x08080808u);
+  const uint32_t neg = (sgn >> 3) * 15u;  // all bits of the negative nibbles
+  return (mag & ~neg) | (((0x88888888u - mag) ^ 0x88888888u) & neg);
+}
+
 // Shared memory of one CTA (dynamic): the sample ring, the FFT buffers of a
 // batch of spectra and, when quantising, the staging tile.
 constexpr int kBatch = 4;                         // spectra per inner iteration
@@ -190,15 +226,20 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src, int src_b
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(src_bytes)
                : "memory");
 }
-// A 16-byte read-only load that the compiler keeps where it is written (it
-// neither re-issues it at the use nor moves it across the barriers), so that
-// the next batch's coefficients are in flight while the current batch ends.
+// A 16-byte read-only load that the compiler does not issue again at the use,
+// so that the filter's coefficients stay in registers.
 __device__ __forceinline__ float4 ldg_keep(const float *p) {
   float4 v;
   asm volatile("ld.global.nc.v4.f32 {%0, %1, %2, %3}, [%4];"
                : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
                : "l"(p));
   return v;
+}
+// A 32-byte store (one full sector) of eight words in shared memory.
+__device__ __forceinline__ void store32(uint8_t *dst, const uint32_t *w) {
+  asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(w[0]),
+               "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
+               : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
@@ -210,7 +251,9 @@ static_assert(kRing >= kTaps - 1 + 2 * kBatch && (kRing & (kRing - 1)) == 0, "ri
 
 // kQuant: 1 -> packed codes via the staging tile; 0 -> float2 g X straight to
 // global (X-engine order, for tolerance checks).
-template <int kQuant>
+// kWide: every tile is whole and its rows of the output start on 32-byte
+// boundaries (n_spec a multiple of 32, out_codes 32-byte aligned).
+template <int kQuant, bool kWide>
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
     fengine_kernel(const int8_t *__restrict__ adc, const float *__restrict__ proto,
                    const float2 *__restrict__ tw_fft, const float2 *__restrict__ split,
@@ -225,6 +268,10 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
   // W64^j = W1024^(16 j), the first pass's twiddles, kept in shared memory
   __shared__ float2 tw64[64];
   if (tid < 64) tw64[tid] = __ldg(tw_fft + 16 * tid);
+  // W1024^(n2 k1) at 64 n2 + k1, the second pass's
+  float2 *tw_p2 = reinterpret_cast<float2 *>(fe_smem + kRingBytes + kBufBytes + kStageBytes);
+  for (int k = tid; k < kHalf; k += kThreads)
+    tw_p2[k] = __ldg(tw_fft + (((k >> 6) * (k & 63)) & (kHalf - 1)));
   __syncthreads();
   const int n_tiles = (n_spec + kSpecTile - 1) / kSpecTile;
   const int n_seg = n_spec + kTaps - 1;  // segments in one input's stream
@@ -240,8 +287,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
                x + (in ? (long long)seg * kP + 16 * p : 0), in ? 16 : 0);
   };
   // the thread's 8 coefficients of each tap (samples 4 t .. 4 t + 3 and
-  // 1024 + 4 t .. + 3), the same for every batch; loaded here for the first
-  // batch and at the end of each batch for the next
+  // 1024 + 4 t .. + 3), the same for every batch: kept in 32 registers
   float4 hq[2 * kTaps];
   auto load_h = [&]() {
 #pragma unroll
@@ -358,10 +404,10 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
         const int n2 = tid >> 4, l1 = tid & 15;
         float2 tw[4];
 #pragma unroll
-        for (int l2 = 0; l2 < 4; ++l2) tw[l2] = __ldg(tw_fft + ((n2 * (l1 + 16 * l2)) & (kHalf - 1)));
-        // kept as a loop: unrolled, the four copies made the kernel 5 % slower
-        // (a larger loop body for the instruction cache)
-#pragma unroll 1
+        for (int l2 = 0; l2 < 4; ++l2) tw[l2] = tw_p2[64 * n2 + l1 + 16 * l2];
+        // two spectra an iteration (192 inputs x 8192 spectra: 5.22 ms; one,
+        // 5.35; all four, 5.24: the loop body's size against its latency)
+#pragma unroll 2
         for (int u = 0; u < kBatch; ++u) {
           if (u >= nb) break;
           float2 *bu = buf + u * kBufElems;
@@ -407,7 +453,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
         const float gm = __ldg(eq + (long long)in * kHalf + m);
         const float2 sc = __ldg(split + c);
         const float2 gcc = make_float2(gc, gc), gmm = make_float2(gm, -gm);
-        uint32_t wc = 0, wm = 0;
+        float2 xcs[kBatch], xms[kBatch];
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
           const float2 P = buf[u * kBufElems + bpos(c)];
@@ -419,53 +465,55 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
           const float2 xc = mul2(gcc, U);          // g X[c]
           const float2 xm = mul2(gmm, csub(F, U));  // g X[m] = g conj V
           if (kQuant) {
-            wc |= (uint32_t)(((quant(xc.x) & 15) << 4) | (quant(xc.y) & 15)) << (8 * u);
-            wm |= (uint32_t)(((quant(xm.x) & 15) << 4) | (quant(xm.y) & 15)) << (8 * u);
+            xcs[u] = xc;
+            xms[u] = xm;
           } else if (u < nb) {
             out_spec[((long long)c * n_in + in) * n_spec + k0 + s0 + u] = xc;
             out_spec[((long long)m * n_in + in) * n_spec + k0 + s0 + u] = xm;
           }
         }
         if (kQuant) {
-          *reinterpret_cast<uint32_t *>(&stage[c * kStagePitch + s0]) = wc;
-          *reinterpret_cast<uint32_t *>(&stage[m * kStagePitch + s0]) = wm;
+          *reinterpret_cast<uint32_t *>(&stage[c * kStagePitch + s0]) = quant4(xcs);
+          *reinterpret_cast<uint32_t *>(&stage[m * kStagePitch + s0]) = quant4(xms);
         }
       }
-      if (tid == 0) {
-        // channel 0: R = P = Z[0]
+      if ((tid & 31) == 0 && (tid >> 5) < kBatch) {
+        // channel 0: R = P = Z[0]; a spectrum each to four warps' first threads
+        const int u = tid >> 5;
         const float g0 = __ldg(eq + (long long)in * kHalf);
         const float2 s_0 = __ldg(split);
-        uint32_t w0 = 0;
-#pragma unroll
-        for (int u = 0; u < kBatch; ++u) {
-          const float2 P = buf[u * kBufElems];
-          const float2 D = fma2(P, k_mp, P);
-          const float2 x0 = make_float2(g0 * fmaf(s_0.x, D.x, fmaf(-s_0.y, D.y, P.x)),
-                                        g0 * fmaf(s_0.x, D.y, fmaf(s_0.y, D.x, -P.y)));
-          if (kQuant) {
-            w0 |= (uint32_t)(((quant(x0.x) & 15) << 4) | (quant(x0.y) & 15)) << (8 * u);
-          } else if (u < nb) {
-            out_spec[(long long)in * n_spec + k0 + s0 + u] = x0;
-          }
-        }
-        if (kQuant) *reinterpret_cast<uint32_t *>(&stage[s0]) = w0;
+        const float2 P = buf[u * kBufElems];
+        const float2 D = fma2(P, k_mp, P);
+        const float2 x0 = make_float2(g0 * fmaf(s_0.x, D.x, fmaf(-s_0.y, D.y, P.x)),
+                                      g0 * fmaf(s_0.x, D.y, fmaf(s_0.y, D.x, -P.y)));
+        if (kQuant)
+          stage[s0 + u] = (uint8_t)(((quant(x0.x) & 15) << 4) | (quant(x0.y) & 15));
+        else if (u < nb)
+          out_spec[(long long)in * n_spec + k0 + s0 + u] = x0;
       }
-      load_h();         // the next batch's coefficients, in flight across the barrier
+      if (!kQuant) load_h();  // the spectra output's addresses take the registers
       __syncthreads();  // buf and the ring slots are reused by the next batch
     }
     if (kQuant) {
-      // ---- staging tile -> out[c][in][k0 .. k0 + ns): thread per channel,
-      // its row of the tile as eight words (conflict-free: rows 9 words apart)
-      const bool vec = ns == kSpecTile && (n_spec & 15) == 0;
-      static_assert(kSpecTile == 32, "two 16-byte stores per channel");
-      for (int c = tid; c < kHalf; c += kThreads) {
-        const uint32_t *row = reinterpret_cast<const uint32_t *>(&stage[c * kStagePitch]);
-        uint8_t *dst = out_codes + ((long long)c * n_in + in) * n_spec + k0;
-        if (vec) {
-          reinterpret_cast<uint4 *>(dst)[0] = make_uint4(row[0], row[1], row[2], row[3]);
-          reinterpret_cast<uint4 *>(dst)[1] = make_uint4(row[4], row[5], row[6], row[7]);
-        } else {
-          for (int b = 0; b < ns; ++b) dst[b] = stage[c * kStagePitch + b];
+      // ---- staging tile -> out[c][in][k0 .. k0 + ns)
+      if (kWide) {
+        // a thread per channel, its row of the tile as eight words (conflict-
+        // free: rows 9 words apart) in one 32-byte store, a full sector (two
+        // 16-byte stores cost 5 % of the kernel's time)
+        for (int c = tid; c < kHalf; c += kThreads)
+          store32(out_codes + ((long long)c * n_in + in) * n_spec + k0,
+                  reinterpret_cast<const uint32_t *>(&stage[c * kStagePitch]));
+      } else {
+        // rows of any alignment or length: a warp per row, a lane per code
+        // (a thread per row, code by code, touched 32 rows an instruction: 17
+        // inputs x 1003 spectra took 220 us against 87)
+        const int b = tid & 31;
+        if (b < ns) {
+          uint8_t *dst = out_codes + (long long)in * n_spec + k0 + b;
+          const long long pitch = (long long)n_in * n_spec;
+#pragma unroll 8
+          for (int c = tid >> 5; c < kHalf; c += kThreads / 32)
+            dst[c * pitch] = stage[c * kStagePitch + b];
         }
       }
       __syncthreads();
@@ -473,7 +521,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
   }
 }
 
-constexpr int smem_bytes() { return kRingBytes + kBufBytes + kStageBytes; }
+constexpr int smem_bytes() { return kRingBytes + kBufBytes + kStageBytes + kHalf * 8; }
 
 }  // namespace
 
@@ -542,10 +590,13 @@ int corr_fengine_create(int n_in, int n_spectra, corr_fengine **out) {
     split[k] = make_float2((float)(0.5 * (1.0 - st)), (float)(-0.5 * ct));
   }
   int rc;
-  if ((rc = cuda_err(cudaFuncSetAttribute(fengine_kernel<1>,
+  if ((rc = cuda_err(cudaFuncSetAttribute(fengine_kernel<1, true>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           smem_bytes()))) != CORR_OK ||
-      (rc = cuda_err(cudaFuncSetAttribute(fengine_kernel<0>,
+      (rc = cuda_err(cudaFuncSetAttribute(fengine_kernel<1, false>,
+                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          smem_bytes()))) != CORR_OK ||
+      (rc = cuda_err(cudaFuncSetAttribute(fengine_kernel<0, false>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           smem_bytes()))) != CORR_OK ||
       (rc = cuda_err(cudaMalloc(&f->d_proto, L * sizeof(float)))) != CORR_OK ||
@@ -578,7 +629,9 @@ int corr_fengine_run(corr_fengine *f, const int8_t *d_adc, uint8_t *d_out, void 
   if (!f || !d_adc || !d_out || !aligned(d_adc, 16) || !aligned(d_out, 16)) return CORR_EINVAL;
   const long long work = (long long)f->n_in * ((f->n_spec + kSpecTile - 1) / kSpecTile);
   const int grid = (int)std::min<long long>(work, (long long)f->n_sm * kCtasPerSm * 4);
-  fengine_kernel<1><<<grid, kThreads, smem_bytes(), static_cast<cudaStream_t>(stream)>>>(
+  const bool wide = f->n_spec % kSpecTile == 0 && aligned(d_out, 32);
+  auto *kernel = wide ? fengine_kernel<1, true> : fengine_kernel<1, false>;
+  kernel<<<grid, kThreads, smem_bytes(), static_cast<cudaStream_t>(stream)>>>(
       d_adc, f->d_proto, f->d_tw_fft, f->d_split, f->d_eq, d_out, nullptr, f->n_in, f->n_spec);
   return cuda_err(cudaGetLastError());
 }
@@ -588,7 +641,7 @@ int corr_fengine_spectra(corr_fengine *f, const int8_t *d_adc, float *d_spec, vo
   if (!f || !d_adc || !d_spec || !aligned(d_adc, 16) || !aligned(d_spec, 8)) return CORR_EINVAL;
   const long long work = (long long)f->n_in * ((f->n_spec + kSpecTile - 1) / kSpecTile);
   const int grid = (int)std::min<long long>(work, (long long)f->n_sm * kCtasPerSm * 4);
-  fengine_kernel<0><<<grid, kThreads, smem_bytes(), static_cast<cudaStream_t>(stream)>>>(
+  fengine_kernel<0, false><<<grid, kThreads, smem_bytes(), static_cast<cudaStream_t>(stream)>>>(
       d_adc, f->d_proto, f->d_tw_fft, f->d_split, f->d_eq, nullptr,
       reinterpret_cast<float2 *>(d_spec), f->n_in, f->n_spec);
   return cuda_err(cudaGetLastError());

@@ -126,3 +126,63 @@ def test_dump_into_stokes_of_either_alignment(corr, torch_cuda, oracle_mod, synt
     assert np.array_equal(vis.cpu().numpy(), want)
     assert np.array_equal(st.cpu().numpy().reshape(C, -1, 4, 2), oracle_mod.stokes(want, n_ant))
     assert (store[:offset] == 7).all() and (store[offset + n:] == 7).all()
+
+
+def _impulse_engine(corr, torch, n_spectra):
+    # an impulse at the first sample of segment 2 is the centre tap of spectrum
+    # 0: X[c] is the same real number for every channel, exactly (the DFT adds
+    # zeros to it)
+    adc = torch.zeros((1, (n_spectra + 3) * 2048), dtype=torch.int8, device="cuda")
+    adc[0, 2 * 2048] = 100
+    fe = corr.FEngine(1, n_spectra)
+    fe.set_eq(np.ones((1, 1024), dtype=np.float32))
+    x = fe.spectra(adc).cpu().numpy()[:, 0, 0]
+    assert (x[:, 0] == x[0, 0]).all() and not x[:, 1].any()
+    return adc, fe, np.float32(x[0, 0])
+
+
+@pytest.mark.parametrize("n_spectra", [32, 5])
+def test_fengine_codes_at_rounding_boundaries(corr, torch_cuda, n_spectra):
+    # gains that bring X to every half-integer up to the clip, and to its
+    # neighbours in fp32 on both sides; the code is the fp32 product rounded
+    # half away from zero, clipped to [-7, 7]
+    adc, fe, x0 = _impulse_engine(corr, torch_cuda, n_spectra)
+    targets = [s * (k + h) for k in range(10) for h in (0.0, 0.5) for s in (1.0, -1.0)]
+    g = [np.float32(t) / x0 for t in targets]
+    for step in (1, 2, 3):
+        for t in targets:
+            lo = hi = np.float32(t) / x0
+            for _ in range(step):
+                lo, hi = np.nextafter(lo, np.float32(-np.inf)), np.nextafter(hi, np.float32(np.inf))
+            g += [lo, hi]
+    g += [np.float32(v) for v in (np.inf, -np.inf, np.nan, 1e30, -1e30, 1e-30, 0.0, -0.0)]
+    eq = np.zeros((1, 1024), dtype=np.float32)
+    eq[0, : len(g)] = g
+    assert len(g) < 1024
+    fe.set_eq(eq)
+    codes = fe.run(adc).cpu().numpy()[:, 0, 0]
+    with np.errstate(all="ignore"):
+        re, im = eq[0] * x0, eq[0] * np.float32(0.0)
+    for c in range(1024):
+        want = 0
+        for v, shift in ((re[c], 4), (im[c], 0)):
+            if np.isnan(v):
+                q = -7  # fmax(NaN, -7)
+            else:
+                q = int(np.sign(v) * np.floor(np.abs(np.float64(np.clip(v, -7, 7))) + 0.5))
+            want |= (q & 15) << shift
+        assert codes[c] == want, (c, eq[0, c], re[c])
+
+
+@pytest.mark.parametrize("n_in,n_spectra", [(3, 64), (2, 32), (2, 96)])
+def test_fengine_output_alignments(corr, torch_cuda, synth_mod, n_in, n_spectra):
+    # rows in whole 32-byte stores, and the same output 16 bytes off
+    torch = torch_cuda
+    adc = torch.from_numpy(synth_mod.adc_streams(n_in, (n_spectra + 3) * 2048, seed=41)).cuda()
+    n = 1024 * n_in * n_spectra
+    store = torch.full((n + 64,), 0xAB, dtype=torch.uint8, device="cuda")
+    with corr.FEngine(n_in, n_spectra, synth_mod.eq_for_noise(n_in, 20.0)) as fe:
+        want = fe.run(adc)
+        fe.run(adc, out=store[16:16 + n])
+    assert torch.equal(store[16:16 + n], want.view(-1))
+    assert (store[:16] == 0xAB).all() and (store[16 + n:] == 0xAB).all()

@@ -525,10 +525,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     }
   } else if (warp < kUnpackWarps) {
     // ------------------------------------------------------------ unpack
-    // The warps form two groups of kUnpackGroup.  A packed stage holds two
-    // operand chunks; group 0 decodes the first and group 1 the second, so a
-    // warp waits, fences and arrives once per stage and has all its loads of
-    // a chunk in flight together.  (All warps on every chunk spent half of
+    // The warps form two groups of kUnpackGroup, which decode the operand
+    // chunks in turn (the even and the odd ones, counted over all items), so a
+    // warp waits, fences and arrives once per two chunks, as a rule a packed
+    // stage, and has all its loads of a chunk in flight together.  Taking turns
+    // strictly, also past a block's odd last chunk, keeps a group at most two
+    // chunks from its last wait on an operand stage: a parity wait then never
+    // mistakes a stage's phase for the one two uses before.  (All warps on every chunk spent half of
     // their instructions on that hand-off: 3200 warp instructions per chunk
     // of 192 inputs.)  A region's inputs are a multiple of kTileInputs, so
     // every warp has the same number of 8-row groups: rows 8 w + 64 k + 0..7
@@ -539,9 +542,9 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int g = lane >> 3, sw = lane & 7;
     const int t_grp = 32 * w8 + lane;  // thread of the group
     // packed rows arrive 128B-swizzled: 16-byte chunk c of row r sits at
-    // c ^ (r & 7); this group's operand chunk is chunks 4 grp + g
+    // c ^ (r & 7); operand chunk `sub` of the stage is chunks 4 sub + g
     const uint32_t src_lane =
-        (uint32_t)((8 * w8 + sw) * kPackedRowBytes + (((GRAM ? g : 4 * grp + g) ^ sw) << 4));
+        (uint32_t)((8 * w8 + sw) * kPackedRowBytes + ((g ^ sw) << 4));
     // the lane's 32 operand bytes are 16-byte chunks 2 g and 2 g + 1 (Gram
     // form: a packed chunk's real and imaginary bytes go to the same chunk of
     // the two rows)
@@ -551,8 +554,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t ph = 0, zph = 0;
     bool ok = true;
     long long nu = 0;
-    // Gram form: a stage is one chunk, and the groups take stages in turn
-    bool my_turn = grp == 0;
+    int turn = 0;  // the group that decodes the next chunk
     for (int it = it0; it < it1 && ok && !*abort_flag; it += it_step, ++nu) {
       const XItem item = item_at(p, it);
       const XProb pb = p.probs[item.prob];
@@ -584,15 +586,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       StageWalk walk(pb, item.pk0);
       for (int k = 0; k < item.npk; ++k, walk.next()) {
         const int nch = GRAM ? 1 : walk.chunks();
-        const bool wanted = GRAM ? my_turn : grp < nch;
-        my_turn = !my_turn;
+        const int sub = grp ^ turn;  // the group's chunk of this stage, if it has it
+        turn ^= nch & 1;
         if (!mbar_wait(b.pk_full + 8 * s, ph, abort_flag, to)) { ok = false; break; }
-        if (wanted) {
+        if (sub < nch) {
           ++n_mine;
-          const int zm = zs + (GRAM ? 0 : grp), zi = zm >= p.z_stages ? zm - p.z_stages : zm;
+          const int zm = zs + sub, zi = zm >= p.z_stages ? zm - p.z_stages : zm;
           const uint32_t zp = zm >= p.z_stages ? zph ^ 1u : zph;
           if (!mbar_wait(b.z_empty + 8 * zi, zp ^ 1u, abort_flag, to)) { ok = false; break; }
           const uint32_t pk_s = pk_s0 + (uint32_t)s * p.pk_stage_bytes;
+          const uint32_t sub_x = GRAM || TCN ? 0u : 64u * (uint32_t)sub;  // chunks 4 on
           const uint32_t z_s = z_s0 + (uint32_t)zi * p.z_stage_bytes;
 #pragma unroll
           for (int r = 0; r < 2; ++r) {
@@ -602,12 +605,12 @@ __global__ void __launch_bounds__(kThreads, 1)
             else if constexpr (GRAM)
               unpack_gram(pk_s + src_off[r], z_s + dst_off[r], n_k[r], sums[r]);
             else if constexpr (TCN)
-              unpack_turned(pk_s + src_off[r], z_s + dst_off[r], kind[r], n_k[r], t_grp, grp,
+              unpack_turned(pk_s + src_off[r], z_s + dst_off[r], kind[r], n_k[r], t_grp, sub,
                             sums[r]);
             else if (kind[r] == 1)
-              unpack_rows<true>(pk_s + src_off[r], z_s + dst_off[r], 16384u, n_k[r], sums[r]);
+              unpack_rows<true>((pk_s + src_off[r]) ^ sub_x, z_s + dst_off[r], 16384u, n_k[r], sums[r]);
             else
-              unpack_rows<false>(pk_s + src_off[r], z_s + dst_off[r], dst_step[r], n_k[r], sums[r]);
+              unpack_rows<false>((pk_s + src_off[r]) ^ sub_x, z_s + dst_off[r], dst_step[r], n_k[r], sums[r]);
           }
           fence_proxy_async_smem();
           __syncwarp();

@@ -85,6 +85,39 @@ def test_launches_of_few_units(corr, torch_cuda, oracle_mod, synth_mod, n_ant, n
     assert np.array_equal(got, want)
 
 
+@pytest.mark.parametrize("tcn", [False, True])
+@pytest.mark.parametrize("n_ant,C,T,nb", [
+    (128, 2, 4160, 1),     # 256 inputs, 65 chunks a block, cut into equal pieces
+    (128, 5, 64, 8),       # one chunk a block
+    (150, 3, 192, 8),      # two operand stages, three chunks a block
+    (150, 40, 2112, 3),    # the same, 33 chunks, every SM busy
+    (96, 2, 320, 7),       # three operand stages, five chunks a block
+    (96, 1, 40, 8),        # less than a chunk a block
+    (40, 3, 192, 5),       # Gram form: a stage is a chunk
+    (600, 1, 192, 3),      # CTA pairs
+])
+def test_odd_chunk_counts(corr, torch_cuda, oracle_mod, synth_mod, n_ant, C, T, nb, tcn):
+    # blocks of an odd number of 64-sample chunks: the two unpack groups then
+    # meet every block with changed turns
+    N = 2 * n_ant
+    blocks = [synth_mod.make_block(N, C, T, seed=930 + N, block=b) for b in range(nb)]
+    torch = torch_cuda
+    want = None
+    for b in blocks:
+        want = oracle_mod.xcorr(b, vis=want, n_threads=N_THREADS)
+    with corr.Correlator(n_ant, 2, C, T) as xc:
+        for _ in range(3):  # the same launches again: a race need not show at once
+            if tcn:
+                for b in blocks:
+                    b = np.ascontiguousarray(np.transpose(b, (2, 0, 1)))
+                    xc.push_block_tcn(torch.from_numpy(b).cuda())
+            else:
+                xc.push_blocks([torch.from_numpy(b).cuda() for b in blocks])
+            vis, _ = xc.dump(want_stokes=False)
+            xc.check()
+            assert np.array_equal(vis.cpu().numpy(), want)
+
+
 @pytest.mark.parametrize("N,C,T", [
     (5, 7, 16), (16, 9, 131056), (20, 5, 4096), (64, 11, 4096), (65, 3, 33008), (128, 3, 2048),
     (192, 3, 65536), (256, 2, 1040),

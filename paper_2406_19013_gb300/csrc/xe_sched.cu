@@ -406,7 +406,7 @@ int build_items_filled(const std::vector<ProbWork> &probs, int grid, std::vector
     if (t < best) best = t, best_n = n;
     if (n_units * n >= 2LL * grid) break;
   }
-  if (best_n == 0) return used;
+  if (best_n == 0) return (int)cta_first.size() - 1;
   it.clear();
   for (size_t p = 0; p < probs.size(); ++p) {
     const ProbWork &pr = probs[p];

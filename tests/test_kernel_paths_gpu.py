@@ -118,6 +118,26 @@ def test_odd_chunk_counts(corr, torch_cuda, oracle_mod, synth_mod, n_ant, C, T, 
             assert np.array_equal(vis.cpu().numpy(), want)
 
 
+@pytest.mark.parametrize("seed", range(6))
+def test_batches_of_few_uneven_units(corr, torch_cuda, oracle_mod, synth_mod, seed):
+    # launch groups of several small instances, whose splits the search for a
+    # shorter run changes
+    torch = torch_cuda
+    rng = np.random.default_rng(seed)
+    shapes = [(n // 2, 2, int(rng.integers(1, 40)), 16 * int(rng.integers(1, 100)))
+              for n in rng.choice([4, 32, 64, 100, 128, 192, 200, 256, 300], size=7)]
+    blocks = [synth_mod.make_block(2 * a, c, t, seed=990 + seed, block=k)
+              for k, (a, _, c, t) in enumerate(shapes)]
+    with corr.Batch(shapes) as bt:
+        for _ in range(2):
+            bt.push([torch.from_numpy(x).cuda() for x in blocks])
+        bt.check()
+        for k, (a, _, _, _) in enumerate(shapes):
+            vis, _ = bt.dump(k, want_stokes=False)
+            want = 2 * oracle_mod.xcorr(blocks[k], n_threads=N_THREADS)
+            assert np.array_equal(vis.cpu().numpy(), want), (k, shapes[k])
+
+
 @pytest.mark.parametrize("N,C,T", [
     (5, 7, 16), (16, 9, 131056), (20, 5, 4096), (64, 11, 4096), (65, 3, 33008), (128, 3, 2048),
     (192, 3, 65536), (256, 2, 1040),

@@ -198,9 +198,9 @@ int corr_plan_cover(int n_in, int cover, uint8_t *cover_out, int *n_units,
  *     one channel, over all n_blocks blocks of block_len samples.
  *   - Units are cut at 128-sample stage boundaries into items, dealt to at
  *     most `grid` CTAs with about equal modelled cost: the cycles of the
- *     chunks' matrix products or unpack, plus the fold of each item.  With one
- *     or two templates per channel every CTA runs a contiguous run of items;
- *     with more, the units of a channel (which read the same inputs) go to
+ *     chunks' unpack or matrix products, plus the fold of each item.  Every
+ *     CTA runs a contiguous run of items; with CTA pairs or more than 20
+ *     templates, the units of a channel (which read the same inputs) go to
  *     the CTAs that are free first.  No item spans more than 256 stages
  *     (32768 samples): each item folds its fp32 partials into int64 once.
  *   - Contexts whose units are too few to fill the GPU (at most four items

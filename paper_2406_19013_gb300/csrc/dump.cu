@@ -132,39 +132,44 @@ __global__ void guard_check_kernel(const unsigned char *__restrict__ before,
   if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(status, kStatusBounds);
 }
 
-// dst[row][0..pitch) = src[row][0..T) followed by zeros, in words: an output
-// word is cut from the two aligned source words that hold its bytes (the
-// second word of a lane is the first of the next, so it comes from L1).  The
-// source's last bytes, whose second word would lie past its end, and each
-// row's last word are put together from bytes.  src is 4-byte aligned.  (Byte
-// by byte, a block of 75 inputs x 200 channels x 3001 samples took 75 us; a
-// push of it went from 134 to 81 us with words.)
+// dst[row][0..pitch) = src[row][0..T) followed by zeros.  A thread makes 16
+// output bytes from the five aligned source words that hold them (the words
+// come from L1 for all but one lane).  A row's last bytes, and the source's
+// last ones, whose fifth word would lie past its end, are put together from
+// bytes.  src is 4-byte aligned and pitch a multiple of 16.  (45 MB in 15 us;
+// byte by byte 75 us, a word a thread 27 us.)
 __global__ void pitch_kernel(const uint8_t *__restrict__ src, uint8_t *__restrict__ dst,
                              long long rows, int T, int pitch) {
-  const int words = pitch >> 2;
-  const long long n_words = rows * words;
+  const int quads = pitch >> 4;  // 16-byte pieces of a row
+  const long long n_quads = rows * quads;
   const long long src_bytes = rows * (long long)T;
   const long long stride = (long long)gridDim.x * blockDim.x;
   long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  long long row = k / words;
-  int w = (int)(k - row * words);
-  const long long row_step = stride / words;
-  const int w_step = (int)(stride - row_step * words);
-#pragma unroll 4
-  for (; k < n_words; k += stride) {
-    const long long at = row * T + 4 * w;  // first source byte of the word
-    const int left = T - 4 * w;            // bytes of the row from there on
-    uint32_t v = 0u;
-    if (left >= 4 && (at | 3) + 4 < src_bytes) {
+  long long row = k / quads;
+  int w = (int)(k - row * quads);
+  const long long row_step = stride / quads;
+  const int w_step = (int)(stride - row_step * quads);
+#pragma unroll 2
+  for (; k < n_quads; k += stride) {
+    const long long at = row * T + 16 * w;  // first source byte of the piece
+    const int left = T - 16 * w;            // bytes of the row from there on
+    uint32_t v[4] = {0u, 0u, 0u, 0u};
+    if (left >= 16 && (at | 3) + 16 < src_bytes) {
       const uint32_t *s = reinterpret_cast<const uint32_t *>(src + (at & ~3LL));
-      v = __funnelshift_r(__ldg(s), __ldg(s + 1), 8 * (int)(at & 3));
+      uint32_t x[5];
+#pragma unroll
+      for (int e = 0; e < 5; ++e) x[e] = __ldg(s + e);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[e] = __funnelshift_r(x[e], x[e + 1], 8 * (int)(at & 3));
     } else {
-      for (int b = 0; b < min(left, 4); ++b) v |= (uint32_t)__ldg(src + at + b) << (8 * b);
+#pragma unroll
+      for (int b = 0; b < 16; ++b)
+        if (b < left) v[b >> 2] |= (uint32_t)__ldg(src + at + b) << (8 * (b & 3));
     }
-    reinterpret_cast<uint32_t *>(dst)[k] = v;
+    reinterpret_cast<uint4 *>(dst)[k] = make_uint4(v[0], v[1], v[2], v[3]);
     row += row_step;
     w += w_step;
-    if (w >= words) w -= words, ++row;
+    if (w >= quads) w -= quads, ++row;
   }
 }
 

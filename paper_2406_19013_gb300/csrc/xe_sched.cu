@@ -130,13 +130,21 @@ int window_units(int N, XUnit *units) {
         --t_min;
       }
       XUnit &u = units[n_units++] = empty_unit();
-      // inputs below the unit's lowest row tile are only its columns: their
-      // Q rows are neither decoded nor stored (same layout, so the B operand
-      // still spans the window with one stride)
-      if (t_min > 0) add_reg(u, 0, kTileInputs * t_min, 2);
-      add_reg(u, kTileInputs * t_min, kTileInputs * (t_max + 1 - t_min), 1);
-      for (int t = t_max; t >= t_min; --t)
-        add_seg(u, 128 * t, 0, 2048, std::min(kTileInputs * (t + 1), n16), kTileInputs * t, 0);
+      // inputs below the unit's lowest row tile are only its columns: plain
+      // rows, with MMAs of their own.  (In the interleaved layout, Q slots
+      // empty, one MMA spans both, but a stage takes 64 KB, only two fit, and
+      // the unpack and the issuers wait for each other: 256 inputs 1354 us a
+      // launch against 1294, and 1118 with the split's costs set right.)
+      const int own = kTileInputs * t_min;
+      if (t_min > 0) add_reg(u, 0, own, 0);
+      add_reg(u, own, kTileInputs * (t_max + 1 - t_min), 1);
+      const int z_own = u.reg[u.n_reg - 1].z_row;
+      for (int t = t_max; t >= t_min; --t) {
+        const int a_zrow = z_own + 128 * (t - t_min);
+        if (t_min > 0) add_seg(u, a_zrow, 0, 1024, own, kTileInputs * t, 0);
+        add_seg(u, a_zrow, z_own, 2048, std::min(kTileInputs * (t + 1), n16) - own,
+                kTileInputs * t, own);
+      }
       t_max = t_min - 1;
     }
   }
@@ -343,9 +351,10 @@ bool stage_layout(int max_zr, int max_pk, int max_sum, int smem_optin, int max_z
 }
 
 int chunk_cost(const XUnit &u) {
-  int mma = 0;
+  int mma = 0, rows = 0;
   for (int s = 0; s < u.n_seg; ++s) mma += 4 * ((u.pair_rows ? 54 : 24) + u.seg[s].n / 2);
-  const int cost = std::max(mma, 5 * u.z_rows / 2);
+  for (int r = 0; r < u.n_reg; ++r) rows += (u.reg[r].interleaved == 1 ? 2 : 1) * u.reg[r].n_in;
+  const int cost = std::max(mma, 450 + 12 * rows / 5);
   return u.gram ? cost / 2 : cost;  // its rows and MMAs hold 128 samples
 }
 
@@ -463,14 +472,20 @@ int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem>
         (long long)kChunksPerPk * (b - a) - (long long)short_by * (b / ppb - a / ppb);
     return chunks * per_chunk;
   };
-  // More than two templates per channel: they read the same inputs, so the units of
-  // one channel run at the same time and the inputs come from L2 (2048
-  // inputs: contiguous runs spread the CTAs over all channels, and the loads
-  // alone, from HBM, took 4.6 of 4.7 ms against 3.0 ms from L2).  Units go
-  // channel by channel to the CTA that is free first; one that would overrun
-  // the mean load is cut there.
+  // The templates of a channel read the same inputs.  Where there are many, its
+  // units run at the same time, so that the inputs come from L2 (2048 inputs
+  // on CTA pairs: contiguous runs spread the CTAs over all channels, and the
+  // loads alone, from HBM, took 4.6 of 4.7 ms against 3.0 ms from L2): units go
+  // channel by channel to the CTA that is free first, and one that would
+  // overrun the mean load is cut there.  Up to kRunTemplates one-CTA templates
+  // contiguous runs are faster, every CTA having about the same mix of units
+  // (384 inputs 619 / 752 us, 512 1095 / 1175, 768 1129 / 1220, 896 1523 /
+  // 1567, 1152 1333 / 1306; 1280 inputs on pairs 1558 / 1381).
+  constexpr size_t kRunTemplates = 20;
   bool shared_inputs = false;
-  for (const ProbWork &pr : probs) shared_inputs = shared_inputs || pr.units->size() > 2;
+  for (const ProbWork &pr : probs)
+    for (const XUnit &u : *pr.units)
+      shared_inputs = shared_inputs || u.pair_rows || pr.units->size() > kRunTemplates;
   if (shared_inputs) {
     std::vector<std::vector<XItem>> runs(grid);
     typedef std::pair<long long, int> Load;  // modelled cost so far, CTA

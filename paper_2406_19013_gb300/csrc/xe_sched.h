@@ -56,10 +56,12 @@ int window_units(int n_in, XUnit *units);
 constexpr int kGramInputs = 128;
 int gram_units(int n_in, XUnit *units);
 
-// Modelled cycles of one 64-sample chunk of a unit: its MMAs (four K slices of
-// each segment; measured on shared-memory operands, 57 cycles at N = 64, 122
-// at 192, 155 at 256, and 182 for a CTA pair's M = 256, N = 256), or the unpack
-// of its operand rows (960 cycles for 384 rows) if that takes longer.
+// Modelled cycles of one 64-sample chunk of a unit: the unpack of its operand
+// rows, with the hand-off of the chunk (measured at 300 to 512 inputs: 1047
+// cycles for 192 rows written, 1065 for 256, 1260 for 320, 1448 for 384, 1527
+// for 448), or its MMAs if they take longer (four K slices of each segment, on
+// shared-memory operands 57 cycles at N = 64, 122 at 192, 155 at 256, and 182
+// for a CTA pair's M = 256, N = 256).
 int chunk_cost(const XUnit &u);
 // Modelled cycles of a unit's fold per accumulator column (measured: 384
 // columns in about 20 000 cycles).
@@ -99,8 +101,8 @@ constexpr int kMaxFoldStages = 32768 / kPkSamples;
 static_assert(2LL * 15 * 15 * kMaxFoldStages * kPkSamples < (1LL << 24), "exact fp32 partials");
 
 // Cuts every unit (problem, template, channel) into items and deals them to at
-// most `grid` CTAs, in contiguous runs if every problem has one template, else
-// channel by channel to the CTA that is free first.  Each CTA receives about
+// most `grid` CTAs, in contiguous runs, or, where many templates or CTA pairs
+// share a channel's inputs, channel by channel to the CTA that is free first.  Each CTA receives about
 // the same modelled cost: the unpack work (operand rows x chunks) of its
 // items plus a fixed fold cost per item.  A unit is split only at 128-sample
 // stage boundaries and only into pieces of at least min_split_pk stages;

@@ -86,8 +86,8 @@ def log(*a):
     print(*a, file=sys.stderr, flush=True)
 
 
-# The CMAC kernel's operands are 8-bit floats (E5M2) on the tensor cores with
-# fp32 accumulation.  Its roofline peak is the dense E5M2 rate measured in the
+# The CMAC kernel's operands are 8-bit floats (E4M3) on the tensor cores with
+# fp32 accumulation.  Its roofline peak is the dense fp8 (E5M2) rate measured in the
 # same run by corr_mma_rate (back-to-back tcgen05.mma, M = 128, N = 256,
 # K = 32, one CTA per SM, operands in shared memory or A in TMEM; the best of
 # the variants).  The launches last ~5 ms like one CMAC launch, so this is a
@@ -407,7 +407,7 @@ def run_ours(args):
             "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e,
             "gpu_launches": n_launch * ws, "clocks": clk,
             "pct_tensor_peak": 100 * roofline["frac"],
-            "arith": "E5M2 (fp8) operands (exact for 4-bit values), fp32 tensor-core "
+            "arith": "E4M3 (fp8) operands (biased 4-bit values, exact), fp32 tensor-core "
                      "accumulation (exact below 2^24), int64 integration",
         }
         print(json.dumps(line), flush=True)

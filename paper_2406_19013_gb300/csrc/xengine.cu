@@ -20,6 +20,12 @@
 // (times 2^-18) and exact; each item's sums are folded into the int64
 // integration buffer when it ends.
 //
+// What bounds it at 192 inputs: the MMAs on shared-memory operands.  One of N
+// columns takes about 24 + N / 2 cycles per 32-byte K slice (57 at N = 64, 155
+// at 256), so the three strips take about 955 of a 64-sample chunk's 1035
+// cycles (256 channels, 8 blocks of 8192 samples: 940 us a launch, 868 without
+// the decode).  Other sizes: see chunk_cost in xe_sched.h.
+//
 // Kernel structure (persistent, one CTA per SM, 28 warps):
 //   warp 24     TMA producer: packed bytes [channel][input][time] -> smem ring
 //   warps 0-15  unpack: 4-bit nibbles -> E4M3 A/Q rows in the 128B-swizzled
@@ -38,8 +44,8 @@
 // A work unit is (problem, template, channel); a template names the inputs
 // staged per chunk and the MMAs (row tile x column range) that cover its part
 // of the triangle.  The host cuts the units into items (a unit over a range
-// of 128-sample stages) and gives every CTA a contiguous run of items of
-// about equal cost, so the last wave does not leave SMs idle; a launch may
+// of 128-sample stages) and deals them to the CTAs in shares of about equal
+// cost, so the last wave does not leave SMs idle; a launch may
 // hold several independent problems (a batch of correlators).  All waits are
 // bounded by a timeout; on expiry the kernel drains its own copies and MMAs,
 // frees TMEM and reports through *status.

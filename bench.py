@@ -398,7 +398,7 @@ def run_ours(args):
         line = {
             "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": t_max / args.steps, "higher_is_better": True,
-            "scaling": "weak", "vs_baseline": None, "dtype": "e5m2", "data": "synthetic",
+            "scaling": "weak", "vs_baseline": None, "dtype": "e4m3", "data": "synthetic",
             "config": {"workload": WORKLOAD, "n_inputs": N_IN, "n_chan": N_CHAN * ws,
                        "n_chan_per_gpu": N_CHAN, "block_len": BLOCK_LEN,
                        "blocks_per_step": BLOCKS_PER_STEP, "ring_blocks": ring_n,
@@ -494,7 +494,7 @@ def run_large_n(args):
     line = {
         "metric": "X-engine Tera-CMAC/s at 2048 inputs", "value": value, "unit": UNIT, "n_gpus": 1,
         "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms / args.steps,
-        "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "e5m2",
+        "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "e4m3",
         "data": "synthetic",
         "config": {"workload": "large-N X-engine: 1024 dual-pol antennas (2048 inputs, 2098176 "
                                "pairs with autos), 256 channels, 4096-sample blocks of 4+4-bit "
@@ -633,7 +633,7 @@ def run_batched(args):
         "metric": "X-engine batched Tera-CMAC/s (64 independent correlators)", "value": value,
         "unit": UNIT, "n_gpus": 1, "steps": n_push, "warmup": args.warmup,
         "ms_per_step": ms_batch / n_push, "higher_is_better": True, "scaling": "weak",
-        "vs_baseline": None, "dtype": "e5m2", "data": "synthetic",
+        "vs_baseline": None, "dtype": "e4m3", "data": "synthetic",
         "config": {"workload": "64 correlators: 32..512 inputs (dual-pol), 16..1024 channels, "
                                "256..16384-sample blocks (16-sample grid); one step = one block "
                                "of every instance; the timed steps end with a dump of every "
@@ -856,7 +856,7 @@ def run_served(args):
         "metric": "served p99 block-to-visibility latency at 90% of capacity",
         "value": levels["90%"]["p99_ms"], "unit": "ms", "n_gpus": 1, "steps": n_cap,
         "warmup": 6, "ms_per_step": 1000 * wall / n_cap, "higher_is_better": False,
-        "scaling": "weak", "vs_baseline": None, "dtype": "e5m2", "data": "synthetic",
+        "scaling": "weak", "vs_baseline": None, "dtype": "e4m3", "data": "synthetic",
         "config": {"workload": "6 arrays (32, 96, 192, 192, 384, 512 inputs; 64..2048 channels; "
                                "1024..8192-sample blocks), one block per integration, blocks from "
                                "pinned host memory, visibilities back to pinned host memory",

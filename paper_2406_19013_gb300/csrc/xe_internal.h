@@ -6,7 +6,7 @@
 
 namespace xe {
 
-// Samples per pipeline chunk: one 128-byte operand row of fp8 (e5m2) values,
+// Samples per pipeline chunk: one 128-byte operand row of fp8 values,
 // two per sample (re, im), i.e. exactly one 128B-swizzle atom along K.
 constexpr int kChunkSamples = 64;
 // Inputs per row tile: the MMA A operand stacks 64 inputs' real-part rows and

@@ -155,7 +155,9 @@ int corr_sizes(const corr_ctx *ctx, size_t *vis_elems, size_t *stokes_elems,
 int corr_check(corr_ctx *ctx, void *stream);
 
 /*
- * Host-only view of the tile schedule for n_in inputs (no device needed).
+ * Host-only view of the tile schedule that a context of n_in inputs runs (no
+ * device needed): the WINDOW cover up to 256 inputs, PAIRS up to 1152, QUADS
+ * above, or what CORR_CMAC_KERNEL=pair or =smem asks for (the covers follow).
  * cover, if not NULL, is uint8[n_in][n_in] and receives +1 for every element
  * (i, j) that the schedule's MMAs fold into the integration buffer (the lower
  * triangle, each element exactly once).  *n_units receives the work units per
@@ -168,6 +170,10 @@ int corr_plan(int n_in, uint8_t *cover, int *n_units, long long *issued_cmacs);
 /* Triangle covers (the tile schedule's shape; see corr_plan_cover).
  *   WINDOW: N <= 256.  Every unit stages all inputs once per chunk, and the
  *           64-input row tiles' strips share it, packed into 512 TMEM columns.
+ *           Up to 128 inputs in the Gram form: an input's real and imaginary
+ *           samples are operand rows of their own and take a column each.  A
+ *           unit then holds 2 (64 / (N rounded up to 16)) channels up to 32
+ *           inputs, two channels up to 64, otherwise one.
  *   STRIPS: N <= 256.  One unit per row tile t, staging inputs [0, 64(t+1)).
  *   PAIRS:  any N.  Pairs of row tiles against 256-column pieces of their
  *           strip (192-column pieces above 256 inputs); one CTA per unit.
@@ -177,7 +183,8 @@ int corr_plan(int n_in, uint8_t *cover, int *n_units, long long *issued_cmacs);
  *           and the pair's M = 256 tensor-core MMAs share the columns.  On
  *           the diagonal the CTAs take row tiles 0 and 3, and 1 and 2, so
  *           that tiles 0 and 1 run against 128 columns only.
- *           Contexts and batches use it above 1152 inputs.
+ *           Contexts and batches use it above 1152 inputs.  Its items
+ *           (corr_plan_items, corr_plan_launch) are dealt to CTA pairs.
  * WINDOW and STRIPS fall back to PAIRS above 256 inputs, QUADS to PAIRS at
  * 256 and below.  CORR_CMAC_KERNEL=pair in the environment makes contexts of
  * more than 256 inputs use QUADS, =smem PAIRS. */
@@ -193,7 +200,8 @@ int corr_plan_cover(int n_in, int cover, uint8_t *cover_out, int *n_units,
 
 /*
  * Host-only view of how one launch's work is dealt to the GPU's
- * multiprocessors (no device needed).
+ * multiprocessors (no device needed), for a given cover and before the search
+ * for a finer split that contexts and batches add (corr_plan_launch).
  *   - A unit is (template, channel): one of the cover's n_units templates on
  *     one channel, over all n_blocks blocks of block_len samples.
  *   - Units are cut at 128-sample stage boundaries into items, dealt to at
@@ -203,8 +211,6 @@ int corr_plan_cover(int n_in, int cover, uint8_t *cover_out, int *n_units,
  *     templates, the units of a channel (which read the same inputs) go to
  *     the CTAs that are free first.  No item spans more than 256 stages
  *     (32768 samples): each item folds its fp32 partials into int64 once.
- *   - Contexts whose units are too few to fill the GPU (at most four items
- *     per CTA) may cut them finer than this view shows.
  *   - n_blocks: 1..8 (the blocks of one launch).
  *   - items, if not NULL, receives up to `cap` rows of 5 ints:
  *     (problem = 0, template, channel, first stage, stages).  Stage k of the
@@ -218,6 +224,25 @@ int corr_plan_cover(int n_in, int cover, uint8_t *cover_out, int *n_units,
  */
 int corr_plan_items(int n_in, int n_chan, int block_len, int n_blocks, int cover, int grid,
                     int *items, int cap, int *n_items, int *cta_first, int *used_grid);
+
+/*
+ * Host-only view of the split that a launch runs (no device needed): one
+ * problem of n_blocks blocks as a context launches it by default, or several
+ * problems of one block each as a batch launches the instances of a group.
+ *   - n_in, n_chan, block_len: host arrays of n_prob entries (1..128).  Every
+ *     problem has its default cover (corr_plan); all of a launch are in the
+ *     Gram form, or on CTA pairs, or neither.
+ *   - A launch of at most four items per CTA may be cut finer than
+ *     corr_plan_items shows: into smaller pieces of the runs, or every unit
+ *     into equal pieces dealt round the CTAs, whichever is modelled shortest.
+ *   - grid (CTAs, or CTA pairs) and the outputs as for corr_plan_items; an
+ *     item's first int is its problem.
+ * Errors: CORR_EINVAL (NULL array, sizes out of range, problems of different
+ * forms, or cap < *n_items with items given; *n_items is still set).
+ */
+int corr_plan_launch(int n_prob, const int *n_in, const int *n_chan, const int *block_len,
+                     int n_blocks, int grid, int *items, int cap, int *n_items, int *cta_first,
+                     int *used_grid);
 
 /*
  * Visibilities of one block without any allocation.  The paper has no

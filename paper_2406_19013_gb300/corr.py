@@ -54,6 +54,8 @@ ABI = [
     ("corr_plan_cover", _ci, [_ci, _ci, _vp, ctypes.POINTER(_ci), ctypes.POINTER(_ll)]),
     ("corr_plan_items", _ci, [_ci, _ci, _ci, _ci, _ci, _ci, _vp, _ci, ctypes.POINTER(_ci), _vp,
                               ctypes.POINTER(_ci)]),
+    ("corr_plan_launch", _ci, [_ci, _vp, _vp, _vp, _ci, _ci, _vp, _ci, ctypes.POINTER(_ci), _vp,
+                               ctypes.POINTER(_ci)]),
     ("corr_batch_create", _ci, [_ci, _vp, _vp, _vp, _vp, _ci, ctypes.POINTER(_vp)]),
     ("corr_batch_push", _ci, [_vp, ctypes.POINTER(_vp), _vp]),
     ("corr_batch_dump", _ci, [_vp, _ci, _vp, _vp, _vp]),
@@ -204,6 +206,23 @@ def plan_items(n_in: int, n_chan: int, block_len: int, n_blocks: int, grid: int,
     _ck(lib.corr_plan_items(n_in, n_chan, block_len, n_blocks, cover, grid, items.ctypes.data,
                             n.value, ctypes.byref(n), first.ctypes.data, ctypes.byref(used)),
         "corr_plan_items")
+    return items, first[:used.value + 1]
+
+
+def plan_launch(shapes, n_blocks: int, grid: int):
+    """The split that a launch runs: ``shapes`` is a list of (n_in, n_chan,
+    block_len), one for a context's launch of ``n_blocks`` blocks, or the
+    instances of a batch's launch group.  Returns as ``plan_items``."""
+    lib = load()
+    arr = [np.array([sh[k] for sh in shapes], dtype=np.int32) for k in range(3)]
+    head = (len(shapes), *(a.ctypes.data for a in arr), n_blocks, grid)
+    n, used = _ci(), _ci()
+    _ck(lib.corr_plan_launch(*head, None, 0, ctypes.byref(n), None, ctypes.byref(used)),
+        "corr_plan_launch")
+    items = np.zeros((n.value, 5), dtype=np.int32)
+    first = np.zeros(grid + 1, dtype=np.int32)
+    _ck(lib.corr_plan_launch(*head, items.ctypes.data, n.value, ctypes.byref(n),
+                             first.ctypes.data, ctypes.byref(used)), "corr_plan_launch")
     return items, first[:used.value + 1]
 
 

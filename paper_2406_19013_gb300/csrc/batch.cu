@@ -183,11 +183,7 @@ int tuned_cover(int n_in, int block_len, int n_sm, int smem_optin, int *rc) {
   // the default cover (the first candidate) is kept unless another one is
   // faster by more than the run-to-run spread of a timing (3 %)
   for (int cv : cands) {
-    std::vector<xe::XUnit> units = xe::build_schedule(n_in, cv);
-    if (n_in <= xe::kGramInputs && cv == xe::kCoverWindow) {
-      xe::XUnit g[xe::kMaxWindowUnits];
-      units.assign(g, g + xe::gram_units(n_in, g));
-    }
+    const std::vector<xe::XUnit> units = xe::build_schedule(n_in, cv);
     if (units.empty()) continue;
     const float ms = time_cover(units, n_in, C, T, n_sm, smem_optin, d_x, d_acc, d_status, st);
     if (ms >= 0.0f && (best_ms < 0.0f || ms < 0.97f * best_ms)) {
@@ -401,10 +397,6 @@ int corr_batch_create(int n_inst, const int *n_ant, const int *n_pol, const int 
     // the pairs cover of the largest arrays runs in its CTA-pair form
     units[k] = xe::build_schedule(
         b->inst[k].n_in, b->inst[k].n_in > xe::kPairInputs ? xe::kCoverQuads : b->inst[k].cover);
-    if (b->inst[k].n_in <= xe::kGramInputs && b->inst[k].cover == xe::kCoverWindow) {
-      xe::XUnit g[xe::kMaxWindowUnits];
-      units[k].assign(g, g + xe::gram_units(b->inst[k].n_in, g));
-    }
     xe::StageLayout L;
     if (units[k].empty() || !xe::stage_layout({&units[k]}, optin, xe::kMaxZStages, &L)) {
       free_batch(b);

@@ -119,13 +119,13 @@ bool use_tm_kernel(int n_in) {
   return e && std::strcmp(e, "tm") == 0;
 }
 
-// Whether CTA pairs run a context of n_in inputs (more than 256 only): above
-// kPairInputs, unless CORR_CMAC_KERNEL asks for pairs or for one-CTA units.
-bool use_pair_kernel(int n_in) {
-  if (n_in <= 256) return false;
+// The cover of a context of n_in inputs: launch_cover's, unless
+// CORR_CMAC_KERNEL asks for CTA pairs or for one-CTA units (above 256 inputs).
+int context_cover(int n_in) {
   const char *e = std::getenv("CORR_CMAC_KERNEL");
-  if (e && std::strcmp(e, "pair") == 0) return true;
-  return n_in > xe::kPairInputs && !(e && std::strcmp(e, "smem") == 0);
+  if (n_in > 256 && e && std::strcmp(e, "pair") == 0) return xe::kCoverQuads;
+  if (n_in > 256 && e && std::strcmp(e, "smem") == 0) return xe::kCoverPairs;
+  return xe::launch_cover(n_in);
 }
 
 // Shared-memory stages of the TMEM-operand kernel for n_in inputs: operand
@@ -163,6 +163,24 @@ bool tm_stage_layout(int n_in, int smem_optin, xe::StageLayout *out, std::vector
   u.work = G.acc_cols;
   units->assign(1, u);
   return true;
+}
+
+// A split's items, CTA runs and totals to a host view's outputs.
+int copy_split(const std::vector<xe::XItem> &it, const std::vector<int> &first, int *items, int cap,
+               int *n_items, int *cta_first, int *used_grid) {
+  if (n_items) *n_items = (int)it.size();
+  if (used_grid) *used_grid = (int)first.size() - 1;
+  if (cta_first) std::copy(first.begin(), first.end(), cta_first);
+  if (!items) return CORR_OK;
+  if (cap < (int)it.size()) return CORR_EINVAL;
+  for (size_t k = 0; k < it.size(); ++k) {
+    items[5 * k + 0] = it[k].prob;
+    items[5 * k + 1] = it[k].tpl;
+    items[5 * k + 2] = it[k].chan;
+    items[5 * k + 3] = it[k].pk0;
+    items[5 * k + 4] = it[k].npk;
+  }
+  return CORR_OK;
 }
 
 size_t block_bytes(const corr_ctx *c) {
@@ -225,18 +243,13 @@ int corr_create(int n_ant, int n_pol, int n_chan, int block_len, corr_ctx **out)
     if (ms > 0) ctx->timeout_ns = (unsigned long long)ms * 1000000ull;
   }
 
-  ctx->pair = use_pair_kernel(ctx->n_in) ? 1 : 0;
-  std::vector<XUnit> units =
-      xe::build_schedule(ctx->n_in, ctx->pair ? xe::kCoverQuads : xe::kCoverWindow);
-  if (ctx->n_in <= xe::kGramInputs && !use_tm_kernel(ctx->n_in)) {
-    XUnit g[xe::kMaxWindowUnits];
-    units.assign(g, g + xe::gram_units(ctx->n_in, g));
-    ctx->gram = 1;
-  }
+  const std::vector<XUnit> units = xe::build_schedule(ctx->n_in, context_cover(ctx->n_in));
   if (units.empty()) {
     free_ctx(ctx);
     return CORR_EINVAL;
   }
+  ctx->pair = units[0].pair_rows != 0;
+  ctx->gram = units[0].gram;
   ctx->n_tpl = (int)units.size();
   xe::StageLayout L;
   if (!xe::stage_layout({&units}, smem_optin, xe::kMaxZStages, &L)) {
@@ -609,7 +622,7 @@ int corr_check(corr_ctx *ctx, void *stream) {
 }
 
 int corr_plan(int n_in, uint8_t *cover, int *n_units, long long *issued_cmacs) {
-  return corr_plan_cover(n_in, CORR_COVER_WINDOW, cover, n_units, issued_cmacs);
+  return corr_plan_cover(n_in, context_cover(n_in), cover, n_units, issued_cmacs);
 }
 
 int corr_plan_items(int n_in, int n_chan, int block_len, int n_blocks, int cover, int grid,
@@ -623,22 +636,33 @@ int corr_plan_items(int n_in, int n_chan, int block_len, int n_blocks, int cover
   if (units.empty()) return CORR_EINVAL;
   std::vector<xe::XItem> it;
   std::vector<int> first;
-  const int used = xe::build_items({{&units, n_chan, block_len, n_blocks}}, grid, it, first);
-  if (n_items) *n_items = (int)it.size();
-  if (used_grid) *used_grid = used;
-  if (cta_first)
-    for (int k = 0; k <= used; ++k) cta_first[k] = first[k];
-  if (items) {
-    if (cap < (int)it.size()) return CORR_EINVAL;
-    for (size_t k = 0; k < it.size(); ++k) {
-      items[5 * k + 0] = it[k].prob;
-      items[5 * k + 1] = it[k].tpl;
-      items[5 * k + 2] = it[k].chan;
-      items[5 * k + 3] = it[k].pk0;
-      items[5 * k + 4] = it[k].npk;
-    }
+  xe::build_items({{&units, n_chan, block_len, n_blocks}}, grid, it, first);
+  return copy_split(it, first, items, cap, n_items, cta_first, used_grid);
+}
+
+int corr_plan_launch(int n_prob, const int *n_in, const int *n_chan, const int *block_len,
+                     int n_blocks, int grid, int *items, int cap, int *n_items, int *cta_first,
+                     int *used_grid) {
+  if (n_prob <= 0 || n_prob > xe::kMaxBatchMaps || !n_in || !n_chan || !block_len ||
+      n_blocks <= 0 || n_blocks > xe::kMaxBlocksPerLaunch || grid <= 0)
+    return CORR_EINVAL;
+  for (int k = 0; k < n_prob; ++k)
+    if (n_in[k] <= 0 || n_in[k] > CORR_MAX_INPUTS || n_chan[k] <= 0 || block_len[k] <= 0 ||
+        block_len[k] > CORR_MAX_BLOCK_LEN)
+      return CORR_EINVAL;
+  std::vector<std::vector<XUnit>> units(n_prob);
+  std::vector<xe::ProbWork> work;
+  for (int k = 0; k < n_prob; ++k) {
+    units[k] = xe::build_schedule(n_in[k], xe::launch_cover(n_in[k]));
+    if (units[k].empty() || units[k][0].pair_rows != units[0][0].pair_rows ||
+        units[k][0].gram != units[0][0].gram)
+      return CORR_EINVAL;
+    work.push_back({&units[k], n_chan[k], block_len[k], n_blocks});
   }
-  return CORR_OK;
+  std::vector<xe::XItem> it;
+  std::vector<int> first;
+  xe::build_items_filled(work, grid, it, first);
+  return copy_split(it, first, items, cap, n_items, cta_first, used_grid);
 }
 
 int corr_plan_cover(int n_in, int cover_kind, uint8_t *cover, int *n_units,
@@ -659,17 +683,23 @@ int corr_plan_cover(int n_in, int cover_kind, uint8_t *cover, int *n_units,
         // a multi-channel tile issues its MMAs for all its channels: count
         // the first channel's share, and only its diagonal block
         const int cpt = s.ch_rows ? xe::kTileInputs / s.ch_rows : 1;
-        issued += 64LL * s.n / cpt;  // 128 accumulator rows = 64 inputs x (re, im)
+        // 128 accumulator rows are 64 inputs x (re, im); in the Gram form an
+        // input takes two columns as well
+        issued += (u.gram ? 32LL : 64LL) * s.n / cpt;
         if (!cover) continue;
         // the epilogue's mapping: lane rho holds input row_in0 (row_in1 on the
         // odd CTA of a pair) + 8 (rho / 16) + rho % 8, real part when (rho / 8)
-        // is even; column n holds input col_blk[n / 64] + n % 64
+        // is even; column n holds input col_blk[n / 64] + n % 64, in the Gram
+        // form, where columns alternate as the rows do, col_blk[0] +
+        // 8 (n / 16) + n % 8
         for (int rho = 0; rho < 128; ++rho) {
           if ((rho >> 3) & 1) continue;
           const int i = (rank ? s.row_in1 : s.row_in0) + 8 * (rho >> 4) + (rho & 7);
           if (i >= n_in || (s.ch_rows && i >= s.ch_rows)) continue;
           for (int n = 0; n < s.n; ++n) {
-            const int j = s.col_blk[n >> 6] + (n & 63);
+            if (u.gram && ((n >> 3) & 1)) continue;
+            const int j = u.gram ? s.col_blk[0] + 8 * (n >> 4) + (n & 7)
+                                 : s.col_blk[n >> 6] + (n & 63);
             if (s.ch_rows && j >= s.ch_rows) continue;
             if (j <= i) cover[(size_t)i * n_in + j]++;
           }

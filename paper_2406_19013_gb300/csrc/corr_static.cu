@@ -116,8 +116,7 @@ extern "C" int corr_xcorr_static(const uint8_t *d_block, int n_ant, int n_pol, i
   StaticPlan plan;
   std::memset(&plan, 0, sizeof(plan));
   xe::XUnit *units = plan.units;
-  const int n_tpl = N <= xe::kGramInputs ? xe::gram_units((int)N, units)
-                                         : xe::window_units((int)N, units);
+  const int n_tpl = xe::window_units((int)N, units);
   if (n_tpl > kMaxStaticUnits) return CORR_EINVAL;
   plan.n_units = n_tpl;
   int max_z = 0, max_pk = 0, max_sum = 0;

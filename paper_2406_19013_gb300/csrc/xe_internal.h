@@ -98,7 +98,7 @@ struct XUnit {
   // column blocks are shared, since the pair's B operand is the even CTA's
   // N / 2 B rows followed by the odd one's
   int pair_rows;
-  // 1: the Gram form (gram_units): an input's two operand rows are its real
+  // 1: the Gram form (see kGramInputs): an input's two operand rows are its real
   // and its imaginary parts, 128 samples each, and the products of all four
   // combinations are accumulated apart
   int gram;

@@ -76,83 +76,7 @@ static void set_sums(XUnit &u) {
   }
 }
 
-// Tiles of 64 inputs (rows) cover the lower triangle strip by strip: row tile
-// t needs columns [0, min(64 (t + 1), N)).  Within a unit, columns are staged
-// once per chunk and shared by all its row tiles.
-int window_units(int N, XUnit *units) {
-  const int n16 = round_up(N, 16);
-  const int n_rt = (N + kTileInputs - 1) / kTileInputs;
-  int n_units = 0;
-  if (N <= 32) {
-    // 16 or 32 inputs at most: a 64-row tile holds 64 / n16 channels (the
-    // TMA box brings that many channels' rows at once), and a unit two such
-    // tiles; each tile's MMA also computes the cross-channel blocks, which
-    // the epilogue skips
-    XUnit &u = units[n_units++] = empty_unit();
-    const int cpt = kTileInputs / n16;
-    u.n_chan = 2 * cpt;
-    for (int r = 0; r < 2; ++r) {
-      add_reg(u, 0, kTileInputs, 1);
-      u.reg[r].chan_off = r * cpt;
-    }
-    for (int r = 0; r < 2; ++r) {
-      add_seg(u, u.reg[r].z_row, u.reg[r].z_row, 2048, kTileInputs, 0, 0);
-      u.seg[r].chan_off = r * cpt;
-      u.seg[r].ch_rows = n16;
-    }
-  } else if (N <= 2 * kTileInputs) {
-    // one or two row tiles: a unit covers two channels (two staged regions,
-    // one accumulator per row tile and channel, at most 2 x 192 TMEM
-    // columns), so every chunk handed from the unpack to the MMA issuers
-    // carries twice the work
-    XUnit &u = units[n_units++] = empty_unit();
-    u.n_chan = 2;
-    for (int r = 0; r < 2; ++r) {
-      add_reg(u, 0, kTileInputs * n_rt, 1);
-      u.reg[r].chan_off = r;
-    }
-    for (int r = 0; r < 2; ++r)
-      for (int t = 0; t < n_rt; ++t) {
-        add_seg(u, u.reg[r].z_row + 128 * t, u.reg[r].z_row, 2048,
-                std::min(kTileInputs * (t + 1), n16), kTileInputs * t, 0);
-        u.seg[u.n_seg - 1].chan_off = r;
-      }
-  } else {
-    // units of consecutive row tiles, largest strip first, each as many as
-    // fit 512 TMEM columns: a unit's lowest tile then bounds the inputs that
-    // are only its columns, and those need no Q rows
-    for (int t_max = n_rt - 1; t_max >= 0;) {
-      int t_min = t_max + 1, used = 0;
-      while (t_min > 0) {
-        const int n = std::min(kTileInputs * t_min, n16);  // tile t_min - 1
-        if (used + n > kTmemCols) break;
-        used += n;
-        --t_min;
-      }
-      XUnit &u = units[n_units++] = empty_unit();
-      // inputs below the unit's lowest row tile are only its columns: plain
-      // rows, with MMAs of their own.  (In the interleaved layout, Q slots
-      // empty, one MMA spans both, but a stage takes 64 KB, only two fit, and
-      // the unpack and the issuers wait for each other: 256 inputs 1354 us a
-      // launch against 1294, and 1118 with the split's costs set right.)
-      const int own = kTileInputs * t_min;
-      if (t_min > 0) add_reg(u, 0, own, 0);
-      add_reg(u, own, kTileInputs * (t_max + 1 - t_min), 1);
-      const int z_own = u.reg[u.n_reg - 1].z_row;
-      for (int t = t_max; t >= t_min; --t) {
-        const int a_zrow = z_own + 128 * (t - t_min);
-        if (t_min > 0) add_seg(u, a_zrow, 0, 1024, own, kTileInputs * t, 0);
-        add_seg(u, a_zrow, z_own, 2048, std::min(kTileInputs * (t + 1), n16) - own,
-                kTileInputs * t, own);
-      }
-      t_max = t_min - 1;
-    }
-  }
-  for (int k = 0; k < n_units; ++k) set_sums(units[k]);
-  return n_units;
-}
-
-int gram_units(int N, XUnit *units) {
+static int gram_units(int N, XUnit *units) {
   const int n16 = round_up(N, 16);
   XUnit &u = units[0] = empty_unit();
   u.gram = 1;
@@ -177,6 +101,47 @@ int gram_units(int N, XUnit *units) {
   }
   set_sums(u);
   return 1;
+}
+
+// Tiles of 64 inputs (rows) cover the lower triangle strip by strip: row tile
+// t needs columns [0, min(64 (t + 1), N)).  Within a unit, columns are staged
+// once per chunk and shared by all its row tiles.
+int window_units(int N, XUnit *units) {
+  if (N <= kGramInputs) return gram_units(N, units);
+  const int n16 = round_up(N, 16);
+  const int n_rt = (N + kTileInputs - 1) / kTileInputs;
+  int n_units = 0;
+  // units of consecutive row tiles, largest strip first, each as many as
+  // fit 512 TMEM columns: a unit's lowest tile then bounds the inputs that
+  // are only its columns, and those need no Q rows
+  for (int t_max = n_rt - 1; t_max >= 0;) {
+    int t_min = t_max + 1, used = 0;
+    while (t_min > 0) {
+      const int n = std::min(kTileInputs * t_min, n16);  // tile t_min - 1
+      if (used + n > kTmemCols) break;
+      used += n;
+      --t_min;
+    }
+    XUnit &u = units[n_units++] = empty_unit();
+    // inputs below the unit's lowest row tile are only its columns: plain
+    // rows, with MMAs of their own.  (In the interleaved layout, Q slots
+    // empty, one MMA spans both, but a stage takes 64 KB, only two fit, and
+    // the unpack and the issuers wait for each other: 256 inputs 1354 us a
+    // launch against 1294, and 1118 with the split's costs set right.)
+    const int own = kTileInputs * t_min;
+    if (t_min > 0) add_reg(u, 0, own, 0);
+    add_reg(u, own, kTileInputs * (t_max + 1 - t_min), 1);
+    const int z_own = u.reg[u.n_reg - 1].z_row;
+    for (int t = t_max; t >= t_min; --t) {
+      const int a_zrow = z_own + 128 * (t - t_min);
+      if (t_min > 0) add_seg(u, a_zrow, 0, 1024, own, kTileInputs * t, 0);
+      add_seg(u, a_zrow, z_own, 2048, std::min(kTileInputs * (t + 1), n16) - own,
+              kTileInputs * t, own);
+    }
+    t_max = t_min - 1;
+  }
+  for (int k = 0; k < n_units; ++k) set_sums(units[k]);
+  return n_units;
 }
 
 std::vector<XUnit> build_schedule(int N, int cover) {
@@ -284,6 +249,11 @@ int tile_ch_rows(const std::vector<XUnit> &units) {
     for (int s = 0; s < u.n_seg; ++s)
       if (u.seg[s].ch_rows) return u.seg[s].ch_rows;
   return kTileInputs;
+}
+
+int launch_cover(int n_in) {
+  if (n_in <= 256) return kCoverWindow;
+  return n_in > kPairInputs ? kCoverQuads : kCoverPairs;
 }
 
 bool stage_layout(const std::vector<const std::vector<XUnit> *> &unit_sets, int smem_optin,

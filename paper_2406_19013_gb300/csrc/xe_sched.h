@@ -11,13 +11,14 @@ namespace xe {
 
 // Cover variants of the triangle (the autotuner chooses between them).
 enum Cover {
-  // N <= 256: one staged window of all inputs per unit; the row tiles'
-  // strips are packed first-fit into units of <= 512 TMEM columns.
+  // N <= 256: one staged window of all inputs per unit; consecutive row
+  // tiles' strips, largest first, packed into units of <= 512 TMEM columns.
+  // Up to kGramInputs inputs in the Gram form.
   kCoverWindow = 0,
   // N <= 256: one unit per row tile t, staging inputs [0, 64 (t + 1)) only.
   kCoverStrips = 1,
-  // any N: pairs of row tiles against 256-column pieces of their strip
-  // (the only one-CTA cover for N > 256).
+  // any N: pairs of row tiles against 256-column pieces of their strip,
+  // 192-column pieces for N > 256 (the only one-CTA cover there).
   kCoverPairs = 2,
   // N > 256, CTA pairs: blocks of 256 rows (four row tiles, two per CTA)
   // against 256-column pieces of their strip, each piece's B rows split
@@ -34,9 +35,13 @@ enum Cover {
 // 3.21.
 constexpr int kPairInputs = 1152;
 
+// The cover that launches of n_in inputs run unless something else is asked
+// for (contexts, batches without the autotuner, the host views).
+int launch_cover(int n_in);
+
 // Templates of the cover, heaviest first.  kCoverWindow and kCoverStrips
-// fall back to kCoverPairs above 256 inputs.
-std::vector<XUnit> build_schedule(int n_in, int cover = kCoverWindow);
+// fall back to kCoverPairs above 256 inputs, kCoverQuads at 256 and below.
+std::vector<XUnit> build_schedule(int n_in, int cover);
 
 // The window cover's templates, heaviest first, into units[kMaxWindowUnits]
 // (n_in <= 256; allocates nothing).  Returns their number; all of them cover
@@ -44,17 +49,15 @@ std::vector<XUnit> build_schedule(int n_in, int cover = kCoverWindow);
 constexpr int kMaxWindowUnits = 4;
 int window_units(int n_in, XUnit *units);
 
-// The units that launches run up to kGramInputs inputs, instead of the window
-// cover's: the same triangle with half of the operand bytes.  A tile's 128
-// rows are the real and the imaginary rows of 64 inputs, 128 samples to a
-// 128-byte row (against [re, im] and [im, -re] rows of 64 samples), and D
-// holds re re, re im, im re and im im products, which the epilogue adds up.  No
-// negated rows are decoded or stored, a stage is one hand-off instead of two,
-// and the MMAs are twice as wide; but an input takes two accumulator columns,
-// so a channel of more than 128 inputs does not fit the 512 TMEM columns.
-// Same arguments and result as window_units.
+// Up to kGramInputs inputs the window cover's units are of the Gram form: the
+// same triangle with half of the operand bytes.  A tile's 128 rows are the real
+// and the imaginary rows of 64 inputs, 128 samples to a 128-byte row (against
+// [re, im] and [im, -re] rows of 64 samples), and D holds re re, re im, im re
+// and im im products, which the epilogue adds up.  No negated rows are decoded
+// or stored, a stage is one hand-off instead of two, and the MMAs are twice as
+// wide; but an input takes two accumulator columns, so a channel of more than
+// 128 inputs does not fit the 512 TMEM columns.
 constexpr int kGramInputs = 128;
-int gram_units(int n_in, XUnit *units);
 
 // Modelled cycles of one 64-sample chunk of a unit: the unpack of its operand
 // rows, with the hand-off of the chunk (measured at 300 to 512 inputs: 1047

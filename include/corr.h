@@ -446,10 +446,9 @@ int corr_batch_dump(corr_batch *b, int inst, int64_t *d_vis, int64_t *d_stokes, 
 int corr_batch_sizes(const corr_batch *b, int inst, size_t *vis_elems, size_t *stokes_elems,
                      long long *samples_integrated);
 
-/* Instance `inst`'s cover (CORR_COVER_*; above 1152 inputs CORR_COVER_PAIRS,
- * which then runs in its CTA-pair form, CORR_COVER_QUADS), its launch group,
- * and the number of launch groups (one CMAC launch each per push).  Any output
- * may be NULL.  Errors: CORR_EINVAL. */
+/* The cover that instance `inst` runs (CORR_COVER_*), its launch group, and
+ * the number of launch groups (one CMAC launch each per push).  Any output may
+ * be NULL.  Errors: CORR_EINVAL. */
 int corr_batch_info(const corr_batch *b, int inst, int *cover, int *group, int *n_groups);
 
 /* As corr_check, for the batch's device status word. */

@@ -74,7 +74,7 @@ int t_bucket(int T) {
 }
 
 std::vector<int> candidate_covers(int n_in) {
-  if (n_in > 256) return {xe::kCoverPairs};
+  if (n_in > 256) return {xe::launch_cover(n_in)};  // nothing to choose from
   return {xe::kCoverWindow, xe::kCoverStrips, xe::kCoverPairs};
 }
 
@@ -365,7 +365,7 @@ int corr_batch_create(int n_inst, const int *n_ant, const int *n_pol, const int 
     in.n_apairs = (long long)in.n_ant * (in.n_ant + 1) / 2;
     in.acc_off = acc_elems;
     acc_elems += (size_t)in.n_chan * in.n_pairs * 2;
-    in.cover = in.n_in <= 256 ? xe::kCoverWindow : xe::kCoverPairs;
+    in.cover = xe::launch_cover(in.n_in);
     if (flags & CORR_BATCH_AUTOTUNE) {
       in.cover = tuned_cover(in.n_in, in.block_len, b->n_sm, optin, &rc);
       if (rc != CORR_OK) {
@@ -394,9 +394,7 @@ int corr_batch_create(int n_inst, const int *n_ant, const int *n_pol, const int 
   std::vector<std::vector<xe::XUnit>> units(n_inst);
   std::map<std::pair<uint32_t, uint32_t>, std::vector<int>> by_layout;
   for (int k = 0; k < n_inst; ++k) {
-    // the pairs cover of the largest arrays runs in its CTA-pair form
-    units[k] = xe::build_schedule(
-        b->inst[k].n_in, b->inst[k].n_in > xe::kPairInputs ? xe::kCoverQuads : b->inst[k].cover);
+    units[k] = xe::build_schedule(b->inst[k].n_in, b->inst[k].cover);
     xe::StageLayout L;
     if (units[k].empty() || !xe::stage_layout({&units[k]}, optin, xe::kMaxZStages, &L)) {
       free_batch(b);

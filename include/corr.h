@@ -187,7 +187,7 @@ int corr_plan(int n_in, uint8_t *cover, int *n_units, long long *issued_cmacs);
  *           (corr_plan_items, corr_plan_launch) are dealt to CTA pairs.
  * WINDOW and STRIPS fall back to PAIRS above 256 inputs, QUADS to PAIRS at
  * 256 and below.  CORR_CMAC_KERNEL=pair in the environment makes contexts of
- * more than 256 inputs use QUADS, =smem PAIRS. */
+ * more than 256 inputs use QUADS, =smem makes contexts and batches use PAIRS. */
 #define CORR_COVER_WINDOW 0
 #define CORR_COVER_STRIPS 1
 #define CORR_COVER_PAIRS 2
@@ -415,6 +415,8 @@ int corr_debug_corrupt_guard(corr_ctx *ctx, int side);
  *     rounded up to a power of two) gets its triangle cover by timing one
  *     launch of every candidate cover on a synthetic problem of that size.
  *     The choice is cached for the process.
+ *   - CORR_CMAC_KERNEL=smem in the environment keeps one-CTA units above 1152
+ *     inputs, as for contexts; its other values have no effect on a batch.
  *   - Results are bit-identical to one context per instance: every sum is
  *     an exact integer.
  */

@@ -160,10 +160,11 @@ int tuned_cover(int n_in, int block_len, int n_sm, int smem_optin, int *rc) {
   *rc = CORR_OK;
   const std::pair<int, int> key(n_in, t_bucket(block_len));
   std::lock_guard<std::mutex> lock(g_tune_mutex);
+  const std::vector<int> cands = candidate_covers(n_in);
+  // nothing to time; the environment may have changed since it was cached
+  if (cands.size() == 1) return g_tune_cache[key] = cands[0];
   auto hit = g_tune_cache.find(key);
   if (hit != g_tune_cache.end()) return hit->second;
-  const std::vector<int> cands = candidate_covers(n_in);
-  if (cands.size() == 1) return g_tune_cache[key] = cands[0];
   const int T = std::min(1 << key.second, 8192);
   const int C = n_sm;
   const long long n_pairs = (long long)n_in * (n_in + 1) / 2;

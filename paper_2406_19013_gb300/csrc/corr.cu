@@ -120,11 +120,10 @@ bool use_tm_kernel(int n_in) {
 }
 
 // The cover of a context of n_in inputs: launch_cover's, unless
-// CORR_CMAC_KERNEL asks for CTA pairs or for one-CTA units (above 256 inputs).
+// CORR_CMAC_KERNEL asks for CTA pairs (above 256 inputs).
 int context_cover(int n_in) {
   const char *e = std::getenv("CORR_CMAC_KERNEL");
   if (n_in > 256 && e && std::strcmp(e, "pair") == 0) return xe::kCoverQuads;
-  if (n_in > 256 && e && std::strcmp(e, "smem") == 0) return xe::kCoverPairs;
   return xe::launch_cover(n_in);
 }
 
@@ -653,7 +652,8 @@ int corr_plan_launch(int n_prob, const int *n_in, const int *n_chan, const int *
   std::vector<std::vector<XUnit>> units(n_prob);
   std::vector<xe::ProbWork> work;
   for (int k = 0; k < n_prob; ++k) {
-    units[k] = xe::build_schedule(n_in[k], xe::launch_cover(n_in[k]));
+    units[k] = xe::build_schedule(
+        n_in[k], n_prob == 1 ? context_cover(n_in[k]) : xe::launch_cover(n_in[k]));
     if (units[k].empty() || units[k][0].pair_rows != units[0][0].pair_rows ||
         units[k][0].gram != units[0][0].gram)
       return CORR_EINVAL;

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cstdlib>
 #include <cstring>
 #include <functional>
 #include <queue>
@@ -253,7 +254,9 @@ int tile_ch_rows(const std::vector<XUnit> &units) {
 
 int launch_cover(int n_in) {
   if (n_in <= 256) return kCoverWindow;
-  return n_in > kPairInputs ? kCoverQuads : kCoverPairs;
+  const char *e = std::getenv("CORR_CMAC_KERNEL");
+  const bool one_cta = e && std::strcmp(e, "smem") == 0;
+  return n_in > kPairInputs && !one_cta ? kCoverQuads : kCoverPairs;
 }
 
 bool stage_layout(const std::vector<const std::vector<XUnit> *> &unit_sets, int smem_optin,

@@ -35,8 +35,9 @@ enum Cover {
 // 3.21.
 constexpr int kPairInputs = 1152;
 
-// The cover that launches of n_in inputs run unless something else is asked
-// for (contexts, batches without the autotuner, the host views).
+// The cover that launches of n_in inputs run (contexts, batches without the
+// autotuner, the host views): CTA pairs above kPairInputs, unless
+// CORR_CMAC_KERNEL=smem in the environment asks for one-CTA units.
 int launch_cover(int n_in);
 
 // Templates of the cover, heaviest first.  kCoverWindow and kCoverStrips

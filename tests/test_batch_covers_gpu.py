@@ -43,3 +43,12 @@ def test_info_reports_the_cover_that_runs(corr, torch_cuda, oracle_mod, synth_mo
         assert [corr.tuned_cover(a * p, t) for a, p, _, t in SHAPES] == got
     else:
         assert got[2] == corr.CORR_COVER_WINDOW
+
+
+@pytest.mark.parametrize("autotune", [False, True])
+def test_one_cta_units_can_be_asked_for(corr, torch_cuda, oracle_mod, synth_mod, monkeypatch,
+                                        autotune):
+    # CTA pairs above 1152 inputs are a default, for batches as for contexts
+    monkeypatch.setenv("CORR_CMAC_KERNEL", "smem")
+    got = _covers(corr, torch_cuda, oracle_mod, synth_mod, autotune)
+    assert got[:2] == [corr.CORR_COVER_PAIRS, corr.CORR_COVER_PAIRS]

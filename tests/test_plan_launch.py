@@ -106,3 +106,19 @@ def test_plan_launch_rejects(corr, shapes, n_blocks, grid):
     with pytest.raises(corr.CorrError) as e:
         corr.plan_launch(shapes, n_blocks, grid)
     assert e.value.code == corr.CORR_EINVAL
+
+
+def test_batch_launches_follow_the_kernel_choice(corr, monkeypatch):
+    # 1280 inputs: 37 one-CTA templates against 15 of CTA pairs
+    shape = [(1280, 2, 256)]
+    pairs = corr.plan_cover(1280, corr.CORR_COVER_PAIRS)[0]
+    quads = corr.plan_cover(1280, corr.CORR_COVER_QUADS)[0]
+    assert corr.plan_launch(shape, 1, 76)[0][:, 1].max() + 1 == quads
+    monkeypatch.setenv("CORR_CMAC_KERNEL", "smem")
+    assert corr.plan_launch(shape, 1, 152)[0][:, 1].max() + 1 == pairs
+    # =pair is for contexts alone
+    monkeypatch.setenv("CORR_CMAC_KERNEL", "pair")
+    assert (corr.plan_launch([(512, 2, 256)], 1, 76)[0][:, 1].max() + 1
+            == corr.plan_cover(512, corr.CORR_COVER_QUADS)[0])
+    assert (corr.plan_launch([(512, 2, 256)] * 2, 1, 76)[0][:, 1].max() + 1
+            == corr.plan_cover(512, corr.CORR_COVER_PAIRS)[0])

@@ -64,10 +64,11 @@ extern "C" {
  * samples; 2^24 - 1 bounds the host-side sample counters of one block). */
 #define CORR_MAX_BLOCK_LEN 16777215
 /* Samples of the blocks that share one launch, at most (a block longer than
- * that is a launch of its own).  The tensor cores accumulate at most 32768
- * samples in fp32, where every partial is an exactly representable integer,
- * before a fold into int64. */
+ * that is a launch of its own). */
 #define CORR_FOLD_SAMPLES 131071
+/* Samples that the tensor cores accumulate in fp32, at most, before a fold
+ * into int64: every partial is then an exactly representable integer. */
+#define CORR_EXACT_SAMPLES 32768
 /* Largest input count N = n_ant * n_pol accepted. */
 #define CORR_MAX_INPUTS 8192
 
@@ -105,7 +106,7 @@ int corr_push_block(corr_ctx *ctx, const uint8_t *d_block, void *stream);
  * Integrates n_blocks blocks (d_blocks: host array of n_blocks device
  * pointers, each as for corr_push_block).  Equivalent to n_blocks calls of
  * corr_push_block, but up to 8 blocks share one launch and its folds into the
- * int64 buffer, one for every 32768 samples or fewer (fewer blocks while
+ * int64 buffer, one for every CORR_EXACT_SAMPLES or fewer (fewer blocks while
  * 8 * block_len exceeds CORR_FOLD_SAMPLES).  The pointer array itself may be
  * reused as soon as the call returns.
  * Errors: CORR_EINVAL (NULL ctx or array, n_blocks < 1, a NULL or misaligned
@@ -209,8 +210,9 @@ int corr_plan_cover(int n_in, int cover, uint8_t *cover_out, int *n_units,
  *     chunks' unpack or matrix products, plus the fold of each item.  Every
  *     CTA runs a contiguous run of items; with CTA pairs or more than 20
  *     templates, the units of a channel (which read the same inputs) go to
- *     the CTAs that are free first.  No item spans more than 256 stages
- *     (32768 samples): each item folds its fp32 partials into int64 once.
+ *     the CTAs that are free first.  No item spans more than
+ *     CORR_EXACT_SAMPLES / 128 = 256 stages: each item folds its fp32 partials
+ *     into int64 once.
  *   - n_blocks: 1..8 (the blocks of one launch).
  *   - items, if not NULL, receives up to `cap` rows of 5 ints:
  *     (problem = 0, template, channel, first stage, stages).  Stage k of the

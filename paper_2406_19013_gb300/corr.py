@@ -30,6 +30,7 @@ CORR_ESTATE = -6
 CORR_EBOUNDS = -7
 CORR_MAX_BLOCK_LEN = 16777215
 CORR_FOLD_SAMPLES = 131071
+CORR_EXACT_SAMPLES = 32768
 CORR_STATIC_MAX_BLOCK_LEN = 131056
 CORR_MAX_INPUTS = 8192
 CORR_COVER_WINDOW = 0

@@ -27,6 +27,8 @@ struct ItemPlan {
   int grid;
 };
 
+static_assert(xe::kMaxFoldStages * xe::kPkSamples == CORR_EXACT_SAMPLES, "the fold window");
+
 struct corr_ctx {
   int n_ant, n_pol, n_chan, block_len, n_in;
   long long n_pairs, n_apairs;

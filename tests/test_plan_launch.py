@@ -34,6 +34,8 @@ def _check(corr, shapes, n_blocks, grid):
         assert np.all(mine[:, 2] % step == 0)
         assert mine[:, 3].min() >= 0 and mine[:, 4].min() >= 1
         assert (mine[:, 3] + mine[:, 4]).max() <= npk
+        # an item folds once, and its fp32 partials are exact over this many samples
+        assert mine[:, 4].max() <= corr.CORR_EXACT_SAMPLES // 128
         seen = np.zeros((n_tpl, -(-n_chan // step), npk), dtype=np.int32)
         for _, tpl, chan, pk0, n in mine:
             seen[tpl, chan // step, pk0:pk0 + n] += 1
@@ -122,3 +124,23 @@ def test_batch_launches_follow_the_kernel_choice(corr, monkeypatch):
             == corr.plan_cover(512, corr.CORR_COVER_QUADS)[0])
     assert (corr.plan_launch([(512, 2, 256)] * 2, 1, 76)[0][:, 1].max() + 1
             == corr.plan_cover(512, corr.CORR_COVER_PAIRS)[0])
+
+
+def test_fold_window_keeps_every_partial_exact(corr):
+    # the operands are v + 8 in [0, 15]: a sample adds up to 2 x 15 x 15 to an
+    # accumulator, and fp32 holds every integer up to 2^24
+    assert 2 * 15 * 15 * corr.CORR_EXACT_SAMPLES < 2**24
+
+
+@pytest.mark.parametrize("cover", [0, 1, 2, 3])
+@pytest.mark.parametrize("n_in,n_chan,block_len,n_blocks,grid", [
+    (16, 3, 300000, 1, 152), (128, 2, 200001, 1, 152), (192, 4, 2000000, 1, 152),
+    (256, 2, 131071, 1, 3), (300, 2, 65536, 2, 152), (512, 1, 32769, 3, 1), (1300, 1, 100000, 1, 76)])
+def test_items_end_within_the_fold_window(corr, n_in, n_chan, block_len, n_blocks, grid, cover):
+    window = corr.CORR_EXACT_SAMPLES // 128
+    items, _ = corr.plan_items(n_in, n_chan, block_len, n_blocks, grid, cover)
+    assert items[:, 4].max() <= window
+    npk = -(-block_len // 128) * n_blocks
+    per_unit = _unit_channels(n_in) if cover == 0 and n_in <= 256 else 1
+    n_tpl = corr.plan_cover(n_in, cover)[0]
+    assert len(items) >= n_tpl * -(-n_chan // per_unit) * -(-npk // window)

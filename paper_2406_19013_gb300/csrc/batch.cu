@@ -60,10 +60,10 @@ struct BGroup {
 
 // ---------------------------------------------------------------- autotuner
 // Cover per (input count, block-length bucket), chosen by timing one launch
-// of each candidate on a synthetic one-wave problem (best of five after a
-// warm-up); a candidate replaces the default only when it is more than 3 %
-// faster.  The kernel's time does
-// not depend on the sample values, so the tuning input is all zeros.
+// of each candidate on a synthetic problem that fills the SMs (tune_channels),
+// split as a batch's launches are (best of five after a warm-up); a candidate
+// replaces the default only when it is more than 3 % faster.  The kernel's time
+// does not depend on the sample values, so the tuning input is all zeros.
 std::mutex g_tune_mutex;
 std::map<std::pair<int, int>, int> g_tune_cache;
 
@@ -87,7 +87,7 @@ float time_cover(const std::vector<xe::XUnit> &units, int n_in, int C, int T, in
   if (!xe::stage_layout({&units}, smem_optin, xe::kMaxZStages, &L)) return -1.0f;
   std::vector<xe::XItem> items;
   std::vector<int> first;
-  const int grid = xe::build_items({{&units, C, T, 1}}, n_sm, items, first);
+  const int grid = xe::build_items_filled({{&units, C, T, 1}}, n_sm, items, first);
   xe::XUnit *d_units = nullptr;
   xe::XProb *d_prob = nullptr;
   xe::XItem *d_items = nullptr;
@@ -166,7 +166,9 @@ int tuned_cover(int n_in, int block_len, int n_sm, int smem_optin, int *rc) {
   auto hit = g_tune_cache.find(key);
   if (hit != g_tune_cache.end()) return hit->second;
   const int T = std::min(1 << key.second, 8192);
-  const int C = n_sm;
+  std::vector<std::vector<xe::XUnit>> units;
+  for (int cv : cands) units.push_back(xe::build_schedule(n_in, cv));
+  const int C = xe::tune_channels(units, n_sm);
   const long long n_pairs = (long long)n_in * (n_in + 1) / 2;
   uint8_t *d_x = nullptr;
   int64_t *d_acc = nullptr;
@@ -183,13 +185,12 @@ int tuned_cover(int n_in, int block_len, int n_sm, int smem_optin, int *rc) {
     goto done;
   // the default cover (the first candidate) is kept unless another one is
   // faster by more than the run-to-run spread of a timing (3 %)
-  for (int cv : cands) {
-    const std::vector<xe::XUnit> units = xe::build_schedule(n_in, cv);
-    if (units.empty()) continue;
-    const float ms = time_cover(units, n_in, C, T, n_sm, smem_optin, d_x, d_acc, d_status, st);
+  for (size_t k = 0; k < cands.size(); ++k) {
+    if (units[k].empty()) continue;
+    const float ms = time_cover(units[k], n_in, C, T, n_sm, smem_optin, d_x, d_acc, d_status, st);
     if (ms >= 0.0f && (best_ms < 0.0f || ms < 0.97f * best_ms)) {
       best_ms = ms;
-      best_cover = cv;
+      best_cover = cands[k];
     }
   }
   {

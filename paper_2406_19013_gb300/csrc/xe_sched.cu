@@ -411,6 +411,13 @@ int build_items_filled(const std::vector<ProbWork> &probs, int grid, std::vector
   return used;
 }
 
+int tune_channels(const std::vector<std::vector<XUnit>> &schedules, int n_sm) {
+  int most = 1;
+  for (const std::vector<XUnit> &units : schedules)
+    for (const XUnit &u : units) most = std::max(most, u.n_chan);
+  return n_sm * most;
+}
+
 int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem> &items,
                 std::vector<int> &cta_first, int min_split_pk, int max_item_pk) {
   items.clear();

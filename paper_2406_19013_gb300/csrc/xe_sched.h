@@ -124,6 +124,11 @@ int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem>
 int build_items_filled(const std::vector<ProbWork> &probs, int grid, std::vector<XItem> &items,
                        std::vector<int> &cta_first);
 
+// Channels of a problem on which schedules are timed against each other: a
+// unit for every SM, whichever schedule's units hold the most channels (with
+// as many channels as SMs, 16 inputs' Gram units ran on 19 of 152).
+int tune_channels(const std::vector<std::vector<XUnit>> &schedules, int n_sm);
+
 // The TMA descriptor of one block, uint8 [n_chan][n_in][row pitch], 3-D
 // (time, input, channel) with boxes of 128 samples x ch_rows inputs x
 // 64 / ch_rows channels (64 rows in all), 128B-swizzled.  ch_rows is 64

@@ -133,9 +133,8 @@ int context_cover(int n_in) {
 // stages of G.z_rows rows (TmGeom), at most as many as the TMEM ring has
 // slots, and packed stages of S = 64 n_rt rows of 128 bytes: three operand
 // stages first, then packed stages up to eight, then operand stages while
-// they fit.  Also returns the one window unit the item split models (its
-// cost: operand rows written per chunk).  False above three row tiles or if
-// two of each stage do not fit.
+// they fit.  Also returns the one unit that the item split models.  False
+// above three row tiles or if two of each stage do not fit.
 bool tm_stage_layout(int n_in, int smem_optin, xe::StageLayout *out, std::vector<XUnit> *units) {
   if (n_in > xe::kTmMaxInputs) return false;
   const xe::TmGeom G = xe::tm_geom(n_in);
@@ -157,12 +156,7 @@ bool tm_stage_layout(int n_in, int smem_optin, xe::StageLayout *out, std::vector
   // one CTA per SM: the kernel holds all 512 TMEM columns
   L.smem_bytes = std::min(std::max(L.smem_bytes, smem_optin / 2 + 1024), smem_optin);
   *out = L;
-  XUnit u;
-  std::memset(&u, 0, sizeof(u));
-  u.n_chan = 1;
-  u.z_rows = 2 * n_st;
-  u.work = G.acc_cols;
-  units->assign(1, u);
+  units->assign(1, xe::tm_unit(n_in));
   return true;
 }
 

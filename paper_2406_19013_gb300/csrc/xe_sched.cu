@@ -252,6 +252,14 @@ int tile_ch_rows(const std::vector<XUnit> &units) {
   return kTileInputs;
 }
 
+XUnit tm_unit(int n_in) {
+  const TmGeom G = tm_geom(n_in);
+  XUnit u = empty_unit();
+  add_reg(u, 0, kTileInputs * G.n_rt, 1);
+  u.work = G.acc_cols;
+  return u;
+}
+
 int launch_cover(int n_in) {
   if (n_in <= 256) return kCoverWindow;
   const char *e = std::getenv("CORR_CMAC_KERNEL");

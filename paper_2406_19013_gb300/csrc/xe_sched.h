@@ -60,6 +60,11 @@ int window_units(int n_in, XUnit *units);
 // 128 inputs does not fit the 512 TMEM columns.
 constexpr int kGramInputs = 128;
 
+// The unit that the item split models for the TMEM-operand kernel (up to
+// kTmMaxInputs inputs): the operand rows that its unpack decodes, two for each
+// staged input, and its accumulator columns.  No launch reads it.
+XUnit tm_unit(int n_in);
+
 // Modelled cycles of one 64-sample chunk of a unit: the unpack of its operand
 // rows, with the hand-off of the chunk (measured at 300 to 512 inputs: 1047
 // cycles for 192 rows written, 1065 for 256, 1260 for 320, 1448 for 384, 1527

@@ -22,6 +22,11 @@ int main(int argc, char **argv) {
         std::printf(" %d", xe::build_items_filled({{&u, C, 256, 1}}, 152, items, first));
       }
       std::printf("\n");
+    } else if (!std::strcmp(argv[k], "tm")) {
+      // the TMEM-operand kernel's unit: operand rows, accumulator columns and
+      // the modelled cycles of a chunk
+      const xe::XUnit u = xe::tm_unit(n_in);
+      std::printf("%d %d %d %d\n", n_in, u.z_rows, u.work, xe::chunk_cost(u));
     }
   }
 }

@@ -35,3 +35,14 @@ def test_tuning_compares_covers_on_a_full_gpu(probe):
         # whole units for every SM, whatever the cover
         assert channels % 152 == 0
         assert ctas == [152, 152, 152], (n_in, channels)
+
+
+def test_tmem_kernel_split_models_its_unpack(probe):
+    # a chunk costs more the more rows it decodes: 2 for each of 64, 128 and 192
+    # staged inputs, at the 2.4 cycles a row that chunk_cost states
+    got = probe("tm", 16, 64, 65, 128, 129, 192)
+    assert [row[1] for row in got] == [128, 128, 256, 256, 384, 384]
+    costs = [row[3] for row in got]
+    assert costs[0] == costs[1] < costs[2] == costs[3] < costs[4] == costs[5]
+    assert abs((costs[2] - costs[0]) - 128 * 2.4) < 1
+    assert abs((costs[4] - costs[2]) - 128 * 2.4) < 1

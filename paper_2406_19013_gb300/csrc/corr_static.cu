@@ -167,7 +167,7 @@ extern "C" int corr_xcorr_static(const uint8_t *d_block, int n_ant, int n_pol, i
   p.cta_first = nullptr;
   p.implicit_n_tpl = n_tpl;
   p.implicit_chan_step = units[0].n_chan;
-  p.implicit_n_chan = (n_chan + units[0].n_chan - 1) / units[0].n_chan;
+  p.implicit_n_chan = xe::channel_units(n_chan, units[0].n_chan);
   p.implicit_npk = prob.pk_per_block;
   // Items per unit: as many as keep every fp32 partial exact, or more where
   // that shortens the modelled run (rounds of items over the SMs, each a piece

@@ -384,7 +384,7 @@ int build_items_filled(const std::vector<ProbWork> &probs, int grid, std::vector
   for (const ProbWork &pr : probs) {
     npk = std::max(npk, (pr.block_len + kPkSamples - 1) / kPkSamples * pr.n_blocks);
     for (const XUnit &u : *pr.units) {
-      n_units += (pr.n_chan + u.n_chan - 1) / std::max(1, u.n_chan);
+      n_units += channel_units(pr.n_chan, u.n_chan);
       fold = std::max(fold, kFold * u.work);
       work = std::max(work, (long long)kChunksPerPk * chunk_cost(u));
     }
@@ -403,10 +403,10 @@ int build_items_filled(const std::vector<ProbWork> &probs, int grid, std::vector
     const int pk = (pr.block_len + kPkSamples - 1) / kPkSamples * pr.n_blocks;
     const int n = std::min(pk, std::max(best_n, (pk + kMaxFoldStages - 1) / kMaxFoldStages));
     for (int t = 0; t < (int)pr.units->size(); ++t)
-      for (int c = 0; c < pr.n_chan; c += std::max(1, (*pr.units)[t].n_chan))
+      for (int w = 0, step = (*pr.units)[t].n_chan; w < channel_units(pr.n_chan, step); ++w)
         for (int k = 0; k < n; ++k) {
           const int lo = (int)((long long)pk * k / n), hi = (int)((long long)pk * (k + 1) / n);
-          it.push_back({(int)p, t, c, lo, hi - lo});
+          it.push_back({(int)p, t, w * step, lo, hi - lo});
         }
   }
   used = std::min(grid, (int)it.size());
@@ -445,7 +445,7 @@ int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem>
     pw[p].npk = pw[p].ppb * pr.n_blocks;
     pw[p].nseg = (pw[p].npk + max_item_pk - 1) / max_item_pk;
     for (const XUnit &u : *pr.units)
-      total += (long long)((pr.n_chan + u.n_chan - 1) / u.n_chan) *
+      total += (long long)channel_units(pr.n_chan, u.n_chan) *
                ((long long)pw[p].cpb * pr.n_blocks * chunk_cost(u) + kFold * u.work * pw[p].nseg);
   }
   if (total == 0 || grid <= 0) {
@@ -505,10 +505,10 @@ int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem>
       const int nseg = pw[p].nseg;
       int step = 1;  // channels of a unit (the same for all templates)
       for (const XUnit &u : us) step = std::max(step, u.n_chan);
-      for (int c = 0; c < probs[p].n_chan; c += step)
+      for (int w = 0; w < channel_units(probs[p].n_chan, step); ++w)
         for (int sg = 0; sg < nseg; ++sg)
           for (int t = 0; t < (int)us.size(); ++t)
-            deal_next(p, t, c, (int)(npk_total * sg / nseg), (int)(npk_total * (sg + 1) / nseg));
+            deal_next(p, t, w * step, (int)(npk_total * sg / nseg), (int)(npk_total * (sg + 1) / nseg));
     }
     cta_first.push_back(0);
     for (const std::vector<XItem> &run : runs) {
@@ -581,10 +581,11 @@ int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem>
     const long long npk_total = pw[p].npk;
     const int nseg = pw[p].nseg;
     for (int t = 0; t < (int)probs[p].units->size(); ++t)
-      for (int c = 0; c < probs[p].n_chan; c += std::max(1, (*probs[p].units)[t].n_chan))
+      for (int w = 0, step = (*probs[p].units)[t].n_chan;
+           w < channel_units(probs[p].n_chan, step); ++w)
         // fold-window segment sg: stages [npk sg / nseg, npk (sg + 1) / nseg)
         for (int sg = 0; sg < nseg; ++sg)
-          deal(p, t, c, (int)(npk_total * sg / nseg), (int)(npk_total * (sg + 1) / nseg));
+          deal(p, t, w * step, (int)(npk_total * sg / nseg), (int)(npk_total * (sg + 1) / nseg));
   }
   if (load > 0 || (int)cta_first.size() == 1) close_cta();
   // drop trailing empty CTAs

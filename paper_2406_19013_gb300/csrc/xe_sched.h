@@ -94,6 +94,10 @@ bool stage_layout(const std::vector<const std::vector<XUnit> *> &unit_sets, int 
 bool stage_layout(int max_zr, int max_pk, int max_sum, int smem_optin, int max_z,
                   StageLayout *out);
 
+// Units of per_unit channels that n_chan channels take (no int on the way
+// exceeds n_chan: unit w starts at channel w per_unit < n_chan).
+constexpr int channel_units(int n_chan, int per_unit) { return (n_chan - 1) / per_unit + 1; }
+
 // One problem as the item builder sees it.
 struct ProbWork {
   const std::vector<XUnit> *units;

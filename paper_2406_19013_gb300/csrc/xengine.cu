@@ -396,7 +396,8 @@ __global__ void __launch_bounds__(kThreads, 1)
           for (int r = 0; r < n_reg; ++r) {
             const int in_lo = rank ? u->reg[r].in_lo1 : u->reg[r].in_lo, n_in = u->reg[r].n_in;
             const int off = u->reg[r].pk_off;
-            const int ch = item.chan + u->reg[r].chan_off;  // past the last: zero fill
+            // past the last channel: zero fill (also where the sum wraps around)
+            const int ch = (int)((uint32_t)item.chan + (uint32_t)u->reg[r].chan_off);
             for (int bx = 0; bx < n_in; bx += kTileInputs) {
               if (TCN)  // (input, channel, time): a [128 samples][64 inputs] box
                 tma_load_3d(dst0 + off + bx * kPackedRowBytes, tmap, full, in_lo + bx, ch,
@@ -734,8 +735,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int i_tile = (rank ? sgm.row_in1 : sgm.row_in0) + 8 * g;
         // a tile of several channels: the 8 rows belong to channel block ci
         const int ci = rpc ? i_tile / rpc : 0;
+        // a multi-channel unit's missing last channels (item.chan < n_chan, so
+        // no sum overflows, however many channels there are)
+        if (sgm.chan_off + ci >= pb.n_chan - item.chan) continue;
         const int c = item.chan + sgm.chan_off + ci;
-        if (c >= pb.n_chan) continue;  // a multi-channel unit's missing last channels
         const int i0 = i_tile - ci * rpc;
         if (i0 >= pb.n_in) continue;
         int64_t *cacc = pb.acc + (long long)c * pb.n_pairs * 2;

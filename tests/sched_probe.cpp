@@ -27,6 +27,10 @@ int main(int argc, char **argv) {
       // the modelled cycles of a chunk
       const xe::XUnit u = xe::tm_unit(n_in);
       std::printf("%d %d %d %d\n", n_in, u.z_rows, u.work, xe::chunk_cost(u));
+    } else if (!std::strcmp(argv[k], "channels")) {
+      // units of 8 channels, and the first channel of the last one
+      const int n = xe::channel_units(n_in, 8);
+      std::printf("%d %d %d\n", n_in, n, (n - 1) * 8);
     }
   }
 }

@@ -46,3 +46,11 @@ def test_tmem_kernel_split_models_its_unpack(probe):
     assert costs[0] == costs[1] < costs[2] == costs[3] < costs[4] == costs[5]
     assert abs((costs[2] - costs[0]) - 128 * 2.4) < 1
     assert abs((costs[4] - costs[2]) - 128 * 2.4) < 1
+
+
+def test_unit_counts_do_not_overflow(probe):
+    # the allocation-free call takes any channel count, with units of 8 channels
+    sizes = (1, 7, 8, 9, 1000, 2**31 - 9, 2**31 - 8, 2**31 - 7, 2**31 - 1)
+    for n_chan, n_units, last in probe("channels", *sizes):
+        assert n_units == -(-n_chan // 8)
+        assert 0 <= last < n_chan <= last + 8

@@ -504,16 +504,27 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
           store32(out_codes + ((long long)c * n_in + in) * n_spec + k0,
                   reinterpret_cast<const uint32_t *>(&stage[c * kStagePitch]));
       } else {
-        // rows of any alignment or length: a warp per row, a lane per code
-        // (a thread per row, code by code, touched 32 rows an instruction: 17
-        // inputs x 1003 spectra took 220 us against 87)
-        const int b = tid & 31;
-        if (b < ns) {
-          uint8_t *dst = out_codes + (long long)in * n_spec + k0 + b;
-          const long long pitch = (long long)n_in * n_spec;
+        // rows of any alignment or length: a lane per code, a warp for as many
+        // rows as it holds (a thread per row, code by code, touched 32 rows an
+        // instruction: 17 inputs x 1003 spectra took 209 us against 71)
+        const long long pitch = (long long)n_in * n_spec;
+        uint8_t *dst = out_codes + (long long)in * n_spec + k0;
+        if (ns > 16) {
+          const int b = tid & 31;
+          if (b < ns) {
 #pragma unroll 8
-          for (int c = tid >> 5; c < kHalf; c += kThreads / 32)
-            dst[c * pitch] = stage[c * kStagePitch + b];
+            for (int c = tid >> 5; c < kHalf; c += kThreads / 32)
+              dst[c * pitch + b] = stage[c * kStagePitch + b];
+          }
+        } else {
+          // 2^lg lanes a row (a whole warp for a row of one spectrum cost 2 of a
+          // run's 6.5 us)
+          const int lg = 32 - __clz(ns - 1), b = tid & ((1 << lg) - 1);
+          if (b < ns) {
+#pragma unroll 2
+            for (int c = tid >> lg; c < kHalf; c += kThreads >> lg)
+              dst[c * pitch + b] = stage[c * kStagePitch + b];
+          }
         }
       }
       __syncthreads();

@@ -239,3 +239,23 @@ def test_fengine_output_alignments(corr, torch_cuda, synth_mod, n_in, n_spectra)
         fe.run(adc, out=store[16:16 + n])
     assert torch.equal(store[16:16 + n], want.view(-1))
     assert (store[:16] == 0xAB).all() and (store[16 + n:] == 0xAB).all()
+
+
+@pytest.mark.parametrize("n_in", [1, 3])
+@pytest.mark.parametrize("n_spectra", [1, 2, 3, 4, 5, 8, 9, 15, 16, 17, 31, 33, 36, 47, 63])
+def test_fengine_rows_of_any_length(corr, torch_cuda, synth_mod, n_in, n_spectra):
+    # a spectrum's codes depend on its own samples alone: the first columns of
+    # a run of whole tiles, with nothing written around them
+    torch = torch_cuda
+    whole = 64
+    x = synth_mod.adc_streams(n_in, (whole + 3) * 2048, seed=43)
+    eq = synth_mod.eq_for_noise(n_in, 20.0)
+    with corr.FEngine(n_in, whole, eq) as fe:
+        want = fe.run(torch.from_numpy(x).cuda())[:, :, :n_spectra]
+    n = 1024 * n_in * n_spectra
+    store = torch.full((n + 64,), 0xAB, dtype=torch.uint8, device="cuda")
+    with corr.FEngine(n_in, n_spectra, eq) as fe:
+        head = np.ascontiguousarray(x[:, : (n_spectra + 3) * 2048])
+        fe.run(torch.from_numpy(head).cuda(), out=store[16:16 + n])
+    assert torch.equal(store[16:16 + n].view(1024, n_in, n_spectra), want)
+    assert (store[:16] == 0xAB).all() and (store[16 + n:] == 0xAB).all()

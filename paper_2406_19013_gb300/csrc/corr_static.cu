@@ -116,7 +116,15 @@ extern "C" int corr_xcorr_static(const uint8_t *d_block, int n_ant, int n_pol, i
   StaticPlan plan;
   std::memset(&plan, 0, sizeof(plan));
   xe::XUnit *units = plan.units;
-  const int n_tpl = xe::window_units((int)N, units);
+  int n_tpl = xe::window_units((int)N, units);
+  // Where even every stage of every unit on an SM of its own leaves more than
+  // half of them idle, units of one tile: a unit's tiles are folded one after
+  // the other (64 inputs, 8 channels: 64 samples 13.1 -> 10.6 us a call, 1024
+  // 13.2 -> 10.6; 5 inputs, 256 channels, 16 samples 9.4 -> 8.5; the one-channel
+  // A/Q units of before took 10.1, 17.3 and 8.7).
+  const long long stages = (block_len + xe::kPkSamples - 1) / xe::kPkSamples;
+  if (2 * stages * xe::channel_units(n_chan, units[0].n_chan) <= g_n_sm[dev])
+    n_tpl = xe::window_units((int)N, units, 1);
   if (n_tpl > kMaxStaticUnits) return CORR_EINVAL;
   plan.n_units = n_tpl;
   int max_z = 0, max_pk = 0, max_sum = 0;

@@ -77,19 +77,19 @@ static void set_sums(XUnit &u) {
   }
 }
 
-static int gram_units(int N, XUnit *units) {
+static int gram_units(int N, XUnit *units, int tiles) {
   const int n16 = round_up(N, 16);
   XUnit &u = units[0] = empty_unit();
   u.gram = 1;
   if (N <= kTileInputs) {
-    // two tiles: of one channel each, or of 64 / n16 channels (ch_rows)
+    // tiles of one channel each, or of 64 / n16 channels (ch_rows)
     const int cpt = N <= 32 ? kTileInputs / n16 : 1;
-    u.n_chan = 2 * cpt;
-    for (int r = 0; r < 2; ++r) {
+    u.n_chan = tiles * cpt;
+    for (int r = 0; r < tiles; ++r) {
       add_reg(u, 0, kTileInputs, 1);
       u.reg[r].chan_off = r * cpt;
     }
-    for (int r = 0; r < 2; ++r) {
+    for (int r = 0; r < tiles; ++r) {
       add_seg(u, u.reg[r].z_row, u.reg[r].z_row, 1024, N <= 32 ? 2 * kTileInputs : 2 * n16, 0, 0);
       u.seg[r].chan_off = r * cpt;
       u.seg[r].ch_rows = N <= 32 ? n16 : 0;
@@ -107,8 +107,8 @@ static int gram_units(int N, XUnit *units) {
 // Tiles of 64 inputs (rows) cover the lower triangle strip by strip: row tile
 // t needs columns [0, min(64 (t + 1), N)).  Within a unit, columns are staged
 // once per chunk and shared by all its row tiles.
-int window_units(int N, XUnit *units) {
-  if (N <= kGramInputs) return gram_units(N, units);
+int window_units(int N, XUnit *units, int tiles) {
+  if (N <= kGramInputs) return gram_units(N, units, tiles);
   const int n16 = round_up(N, 16);
   const int n_rt = (N + kTileInputs - 1) / kTileInputs;
   int n_units = 0;

@@ -48,7 +48,9 @@ std::vector<XUnit> build_schedule(int n_in, int cover);
 // (n_in <= 256; allocates nothing).  Returns their number; all of them cover
 // the same number of channels.
 constexpr int kMaxWindowUnits = 4;
-int window_units(int n_in, XUnit *units);
+// tiles: 64-row tiles of a unit of at most 64 inputs (1 or 2), each with its
+// own channels.
+int window_units(int n_in, XUnit *units, int tiles = 2);
 
 // Up to kGramInputs inputs the window cover's units are of the Gram form: the
 // same triangle with half of the operand bytes.  A tile's 128 rows are the real

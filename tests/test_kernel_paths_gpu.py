@@ -259,3 +259,19 @@ def test_fengine_rows_of_any_length(corr, torch_cuda, synth_mod, n_in, n_spectra
         fe.run(torch.from_numpy(head).cuda(), out=store[16:16 + n])
     assert torch.equal(store[16:16 + n].view(1024, n_in, n_spectra), want)
     assert (store[:16] == 0xAB).all() and (store[16 + n:] == 0xAB).all()
+
+
+@pytest.mark.parametrize("N,C,T", [
+    (1, 1, 16), (5, 9, 16), (16, 5, 128), (17, 3, 144), (32, 76, 128),   # tiles of several channels
+    (33, 2, 16), (48, 7, 1024), (64, 1, 16), (64, 9, 256),               # one channel a tile
+    (64, 76, 256), (64, 77, 256), (16, 608, 128), (16, 616, 128),        # both sides of the rule at 152 SMs
+    (65, 1, 16), (128, 1, 128),                                          # two row tiles
+])
+def test_static_entry_on_few_units(corr, torch_cuda, oracle_mod, synth_mod, N, C, T):
+    torch = torch_cuda
+    x = synth_mod.make_block(N, C, T, seed=1010 + N)
+    vis = torch.full((C + 1, N * (N + 1) // 2, 2), -1, dtype=torch.int64, device="cuda")
+    corr.xcorr_static(torch.from_numpy(x).cuda(), N, 1, vis=vis)
+    got = vis.cpu().numpy()
+    assert np.array_equal(got[:C], oracle_mod.xcorr(x, n_threads=N_THREADS))
+    assert (got[C] == -1).all()

@@ -735,10 +735,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int i_tile = (rank ? sgm.row_in1 : sgm.row_in0) + 8 * g;
         // a tile of several channels: the 8 rows belong to channel block ci
         const int ci = rpc ? i_tile / rpc : 0;
-        // a multi-channel unit's missing last channels (item.chan < n_chan, so
-        // no sum overflows, however many channels there are)
-        if (sgm.chan_off + ci >= pb.n_chan - item.chan) continue;
-        const int c = item.chan + sgm.chan_off + ci;
+        // a multi-channel unit's missing last channels (as unsigned, so that a
+        // sum past 2^31 - 1 is past the last as well)
+        const uint32_t c = (uint32_t)item.chan + (uint32_t)sgm.chan_off + (uint32_t)ci;
+        if (c >= (uint32_t)pb.n_chan) continue;
         const int i0 = i_tile - ci * rpc;
         if (i0 >= pb.n_in) continue;
         int64_t *cacc = pb.acc + (long long)c * pb.n_pairs * 2;

@@ -726,7 +726,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int n_seg = u->n_seg;
       for (int sg = 0; sg < n_seg; ++sg) {
         const XSeg sgm = u->seg[sg];
-        const int rpc = sgm.ch_rows;
+        const int rpc = GRAM ? sgm.ch_rows : 0;  // no other units hold several channels a tile
         // 8 inputs: group g of the tile.  In F-engine-order launches group
         // position l holds input (l - g) % 8 of the group, and column 8 G +
         // e the one at (e - G) % 8 (a row tile or column range starts at a

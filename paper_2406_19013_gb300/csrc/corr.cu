@@ -112,9 +112,9 @@ int free_ctx(corr_ctx *ctx) {
 
 // Whether the TMEM-operand kernel (xengine_tm.cu) runs a context of n_in
 // inputs: only when CORR_CMAC_KERNEL=tm asks for it (up to three row tiles).
-// The all-shared-memory kernel (xengine.cu) with two-channel units measured
-// 1.25x faster at 80..128 inputs and the TMEM-operand kernel 9 % slower at
-// 192 inputs.
+// It was the slower one at every size before the all-shared-memory kernel
+// (xengine.cu) had biased operands and the Gram form (by 1.25x at 80..128
+// inputs, 9 % at 192), which it has not.
 bool use_tm_kernel(int n_in) {
   (void)n_in;
   const char *e = std::getenv("CORR_CMAC_KERNEL");
@@ -257,8 +257,8 @@ int corr_create(int n_ant, int n_pol, int n_chan, int block_len, corr_ctx **out)
   ctx->pk_stage_bytes = L.pk_stage_bytes;
   ctx->sum_rows = L.sum_rows;
   ctx->smem_bytes = L.smem_bytes;
-  // the TMEM-operand kernel where it is the faster one (up to three row
-  // tiles); the item split then models its one window unit
+  // the TMEM-operand kernel where it was asked for (up to three row tiles);
+  // the item split then models its one window unit
   std::vector<XUnit> tm_units;
   xe::StageLayout TL;
   if (use_tm_kernel(ctx->n_in) && tm_stage_layout(ctx->n_in, smem_optin, &TL, &tm_units)) {
@@ -271,9 +271,10 @@ int corr_create(int n_ant, int n_pol, int n_chan, int block_len, corr_ctx **out)
   }
   const std::vector<XUnit> &plan_units = ctx->tm ? tm_units : units;
   ctx->ch_rows = ctx->tm ? xe::kTileInputs : xe::tile_ch_rows(units);
-  // a fold must come before 2^24 / 128 samples have been accumulated in
-  // fp32: launches of several blocks stay within that window, and the item
-  // split cuts a longer block into pieces that each fold on their own
+  // blocks that share a launch: as many as CORR_FOLD_SAMPLES holds.  Exactness
+  // does not need the limit (the item split cuts any launch at the fold
+  // window); it bounds a launch's length, which the device-side time limit of a
+  // wait and the latency of a dump behind it see
   ctx->per_launch = std::max(1, std::min(xe::kMaxBlocksPerLaunch, CORR_FOLD_SAMPLES / block_len));
   if (ctx->pitch != block_len) ctx->per_launch = 1;  // one pitched staging buffer
 

@@ -72,7 +72,13 @@ XUnit tm_unit(int n_in);
 // cycles for 192 rows written, 1065 for 256, 1260 for 320, 1448 for 384, 1527
 // for 448), or its MMAs if they take longer (four K slices of each segment, on
 // shared-memory operands 57 cycles at N = 64, 122 at 192, 155 at 256, and 182
-// for a CTA pair's M = 256, N = 256).
+// for a CTA pair's M = 256, N = 256).  Fitted where two operand stages fit and
+// the unpack binds; with three or more the two overlap better (192 inputs: 1371
+// modelled, 1100 to 1130 measured, folds included, bound by the MMAs), and the
+// TMA stream that binds Gram units is not modelled (532 modelled; 666 measured
+// at 128 inputs, 693 at 64, 755 at 16).  The splits use the costs of a launch's
+// units against each other and against kFold, which weighs a third too little
+// where the model is a third too high.
 int chunk_cost(const XUnit &u);
 // Modelled cycles of a unit's fold per accumulator column (measured: 384
 // columns in about 20 000 cycles).
@@ -85,9 +91,10 @@ struct StageLayout {
   int sum_rows;  // entries of a table of operand sums
   int smem_bytes;
 };
-// Largest z_stages (<= max_z, >= 2) and pk_stages (3 if it leaves >= 2
-// operand stages, else 2) that fit `smem_optin`.  Returns false if not even
-// 2 + 2 stages fit.
+// The stages that fit `smem_optin`: three operand stages beside three or two
+// packed ones, or else two beside three or two; then a fourth operand stage,
+// packed stages up to kMaxPkStages and operand stages up to max_z, while they
+// fit.  Returns false if not even 2 + 2 stages fit.
 bool stage_layout(const std::vector<const std::vector<XUnit> *> &unit_sets, int smem_optin,
                   int max_z, StageLayout *out);
 
@@ -117,12 +124,12 @@ static_assert(2LL * 15 * 15 * kMaxFoldStages * kPkSamples < (1LL << 24), "exact 
 
 // Cuts every unit (problem, template, channel) into items and deals them to at
 // most `grid` CTAs, in contiguous runs, or, where many templates or CTA pairs
-// share a channel's inputs, channel by channel to the CTA that is free first.  Each CTA receives about
-// the same modelled cost: the unpack work (operand rows x chunks) of its
-// items plus a fixed fold cost per item.  A unit is split only at 128-sample
-// stage boundaries and only into pieces of at least min_split_pk stages;
-// first it is cut into equal segments of at most max_item_pk stages (the
-// fold window), which every item stays inside.
+// share a channel's inputs, channel by channel to the CTA that is free first.
+// Each CTA receives about the same modelled cost: chunk_cost for every chunk of
+// its items, plus kFold per accumulator column for the fold of each.  A unit is
+// split only at 128-sample stage boundaries and only into pieces of at least
+// min_split_pk stages; first it is cut into equal segments of at most
+// max_item_pk stages (the fold window), which every item stays inside.
 // Fills items and cta_first (size used_grid + 1) and returns used_grid.
 int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem> &items,
                 std::vector<int> &cta_first, int min_split_pk = 16,

@@ -22,9 +22,10 @@
 //
 // What bounds it at 192 inputs: the MMAs on shared-memory operands.  One of N
 // columns takes about 24 + N / 2 cycles per 32-byte K slice (57 at N = 64, 155
-// at 256), so the three strips take about 955 of a 64-sample chunk's 1035
-// cycles (256 channels, 8 blocks of 8192 samples: 940 us a launch, 868 without
-// the decode).  Other sizes: see chunk_cost in xe_sched.h.
+// at 256), so the three strips take about 1056 of a 64-sample chunk's 1100 to
+// 1130 cycles (256 channels, 8 blocks of 8192 samples: 943 to 978 us a launch
+// at 1.99 GHz; without the decode 8 % less).  Other sizes: see chunk_cost in
+// xe_sched.h.
 //
 // Kernel structure (persistent, one CTA per SM, 28 warps):
 //   warp 24     TMA producer: packed bytes [channel][input][time] -> smem ring
@@ -55,6 +56,9 @@
 // hand-off per 128 samples, twice the accumulator columns.  (128 inputs, 512
 // channels, 4 blocks of 8192 samples: 741 -> 567 us a launch; 64 inputs, 8
 // blocks: 824 -> 612; 16 inputs: 237 -> 179.)
+// At 72 registers a thread every instance spills a little (bytes stored /
+// loaded: one CTA 12 / 12, pair 20 / 28, Gram 44 / 116, F-engine order 48 / 56,
+// Gram in F-engine order 68 / 144, pair in F-engine order 84 / 140).
 // The CTA-pair instance (PAIR) runs clusters of two CTAs on two SMs: each
 // stages and unpacks two row tiles and half of a B operand of up to 256
 // columns, the even CTA's two issuers run M = 256 MMAs (cta_group::2) over
@@ -538,13 +542,13 @@ __global__ void __launch_bounds__(kThreads, 1)
     // stage, and has all its loads of a chunk in flight together.  Taking turns
     // strictly, also past a block's odd last chunk, keeps a group at most two
     // chunks from its last wait on an operand stage: a parity wait then never
-    // mistakes a stage's phase for the one two uses before.  (All warps on every chunk spent half of
-    // their instructions on that hand-off: 3200 warp instructions per chunk
-    // of 192 inputs.)  A region's inputs are a multiple of kTileInputs, so
-    // every warp has the same number of 8-row groups: rows 8 w + 64 k + 0..7
-    // of the region, a lane one 16-sample group (lane / 8) of one row (lane %
-    // 8); the 8 lanes of a quarter-warp take 8 consecutive rows, so their
-    // swizzled 16-byte accesses fall on 8 different bank groups.
+    // mistakes a stage's phase for the one two uses before.  (All warps on
+    // every chunk spent half of their instructions on that hand-off: 3200 warp
+    // instructions per chunk of 192 inputs.)  A region's inputs are a multiple
+    // of kTileInputs, so every warp has the same number of 8-row groups: rows
+    // 8 w + 64 k + 0..7 of the region, a lane one 16-sample group (lane / 8) of
+    // one row (lane % 8); the 8 lanes of a quarter-warp take 8 consecutive
+    // rows, so their swizzled 16-byte accesses fall on 8 different bank groups.
     const int grp = warp / kUnpackGroup, w8 = warp % kUnpackGroup;
     const int g = lane >> 3, sw = lane & 7;
     const int t_grp = 32 * w8 + lane;  // thread of the group
@@ -691,10 +695,11 @@ __global__ void __launch_bounds__(kThreads, 1)
     // lanes on, an imaginary one; each of the quarter's two warps folds 8 of
     // them.  A 16-lane load brings 16 columns of the 8 inputs, a thread
     // getting both parts of two column pairs of one input: the bias comes off
-    // there, and the 8 x 16 complex values go through a 1 KB buffer so that each atomic instruction adds 256 contiguous bytes
-    // of one row of the integration buffer.  (Lane-per-row adds, 32 rows an
-    // instruction, made four times the memory requests: the fold of a
-    // 192-input channel took 31 us.)
+    // there, and the 8 x 16 complex values go through a 1 KB buffer so that
+    // each atomic instruction adds 256 contiguous bytes of one row of the
+    // integration buffer.  (Lane-per-row adds, 32 rows an instruction, made
+    // four times the memory requests: the fold of a 192-input channel took 31
+    // us.)
     const int q = warp & 3, h = (warp - kWarpEpi0) >> 2;
     const uint32_t ebuf = smem_u32(epi_mem) + (uint32_t)(warp - kWarpEpi0) * kEpiBufBytes;
     const int er = lane >> 2, ec = lane & 3;  // the thread's row and column pair as loaded

@@ -240,7 +240,8 @@ int corr_plan_items(int n_in, int n_chan, int block_len, int n_blocks, int cover
  *   - grid (CTAs, or CTA pairs) and the outputs as for corr_plan_items; an
  *     item's first int is its problem.
  * Errors: CORR_EINVAL (NULL array, sizes out of range, problems of different
- * forms, or cap < *n_items with items given; *n_items is still set).
+ * forms, or cap < *n_items with items given; *n_items is still set),
+ * CORR_ENOMEM.
  */
 int corr_plan_launch(int n_prob, const int *n_in, const int *n_chan, const int *block_len,
                      int n_blocks, int grid, int *items, int cap, int *n_items, int *cta_first,

@@ -646,20 +646,24 @@ int corr_plan_launch(int n_prob, const int *n_in, const int *n_chan, const int *
     if (n_in[k] <= 0 || n_in[k] > CORR_MAX_INPUTS || n_chan[k] <= 0 || block_len[k] <= 0 ||
         block_len[k] > CORR_MAX_BLOCK_LEN)
       return CORR_EINVAL;
-  std::vector<std::vector<XUnit>> units(n_prob);
-  std::vector<xe::ProbWork> work;
-  for (int k = 0; k < n_prob; ++k) {
-    units[k] = xe::build_schedule(
-        n_in[k], n_prob == 1 ? context_cover(n_in[k]) : xe::launch_cover(n_in[k]));
-    if (units[k].empty() || units[k][0].pair_rows != units[0][0].pair_rows ||
-        units[k][0].gram != units[0][0].gram)
-      return CORR_EINVAL;
-    work.push_back({&units[k], n_chan[k], block_len[k], n_blocks});
+  try {
+    std::vector<std::vector<XUnit>> units(n_prob);
+    std::vector<xe::ProbWork> work;
+    for (int k = 0; k < n_prob; ++k) {
+      units[k] = xe::build_schedule(
+          n_in[k], n_prob == 1 ? context_cover(n_in[k]) : xe::launch_cover(n_in[k]));
+      if (units[k].empty() || units[k][0].pair_rows != units[0][0].pair_rows ||
+          units[k][0].gram != units[0][0].gram)
+        return CORR_EINVAL;
+      work.push_back({&units[k], n_chan[k], block_len[k], n_blocks});
+    }
+    std::vector<xe::XItem> it;
+    std::vector<int> first;
+    xe::build_items_filled(work, grid, it, first);
+    return copy_split(it, first, items, cap, n_items, cta_first, used_grid);
+  } catch (const std::bad_alloc &) {
+    return CORR_ENOMEM;
   }
-  std::vector<xe::XItem> it;
-  std::vector<int> first;
-  xe::build_items_filled(work, grid, it, first);
-  return copy_split(it, first, items, cap, n_items, cta_first, used_grid);
 }
 
 int corr_plan_cover(int n_in, int cover_kind, uint8_t *cover, int *n_units,

@@ -9,8 +9,6 @@
 #include <atomic>
 #include <cstdlib>
 #include <cstring>
-#include <functional>
-#include <queue>
 #include <utility>
 
 namespace xe {
@@ -482,25 +480,42 @@ int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem>
   if (shared_inputs) {
     std::vector<std::vector<XItem>> runs(grid);
     typedef std::pair<long long, int> Load;  // modelled cost so far, CTA
-    std::priority_queue<Load, std::vector<Load>, std::greater<Load>> free_first;
-    for (int k = 0; k < grid; ++k) free_first.push({0, k});
-    auto deal_next = [&](size_t p, int t, int c, int pk, int npk) {
-      const XUnit &u = (*probs[p].units)[t];
-      const long long fold = kFold * u.work, per = (long long)kChunksPerPk * chunk_cost(u);
+    // a heap whose top is the CTA that is free first; a deal raises the top's
+    // cost and lets it sink (a priority queue's pop and push, and the costs
+    // worked out anew for each unit, made up most of a large context's creation)
+    std::vector<Load> heap;
+    for (int k = 0; k < grid; ++k) heap.push_back({0, k});
+    auto before = [](const Load &a, const Load &b) {  // without a branch
+      return (a.first < b.first) | ((a.first == b.first) & (a.second < b.second));
+    };
+    auto sink_top = [&]() {
+      const Load x = heap[0];
+      size_t at = 0;
+      for (size_t c = 1; c < heap.size(); c = 2 * at + 1) {
+        c += (c + 1 < heap.size()) && before(heap[c + 1], heap[c]);
+        if (before(x, heap[c])) break;
+        heap[at] = heap[c];
+        at = c;
+      }
+      heap[at] = x;
+    };
+    long long mean = (total + grid - 1) / grid;
+    auto deal_next = [&](size_t p, int t, int c, int pk, int npk, long long per, long long fold) {
       while (pk < npk) {
-        const Load l = free_first.top();
-        free_first.pop();
-        const long long room = (total + grid - 1) / grid - l.first - fold;
+        Load &l = heap[0];
+        const long long room = mean - l.first - fold;
         int n = npk - pk;
         if (per * n > room) {
           const int fit = (int)std::max<long long>(0, room / per);
           if (fit >= min_split_pk && n - fit >= min_split_pk) {
             n = fit;
             total += fold;  // the rest of the unit is folded once more
+            mean = (total + grid - 1) / grid;
           }
         }
         runs[l.second].push_back({(int)p, t, c, pk, n});
-        free_first.push({l.first + per * n + fold, l.second});
+        l.first += per * n + fold;
+        sink_top();
         pk += n;
       }
     };
@@ -509,11 +524,17 @@ int build_items(const std::vector<ProbWork> &probs, int grid, std::vector<XItem>
       const long long npk_total = pw[p].npk;
       const int nseg = pw[p].nseg;
       int step = 1;  // channels of a unit (the same for all templates)
-      for (const XUnit &u : us) step = std::max(step, u.n_chan);
+      std::vector<long long> per, fold;  // cost of a template's stage and of its fold
+      for (const XUnit &u : us) {
+        step = std::max(step, u.n_chan);
+        per.push_back((long long)kChunksPerPk * chunk_cost(u));
+        fold.push_back(kFold * u.work);
+      }
       for (int w = 0; w < channel_units(probs[p].n_chan, step); ++w)
         for (int sg = 0; sg < nseg; ++sg)
           for (int t = 0; t < (int)us.size(); ++t)
-            deal_next(p, t, w * step, (int)(npk_total * sg / nseg), (int)(npk_total * (sg + 1) / nseg));
+            deal_next(p, t, w * step, (int)(npk_total * sg / nseg),
+                      (int)(npk_total * (sg + 1) / nseg), per[t], fold[t]);
     }
     cta_first.push_back(0);
     for (const std::vector<XItem> &run : runs) {

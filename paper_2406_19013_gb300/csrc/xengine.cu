@@ -742,8 +742,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int ci = rpc ? i_tile / rpc : 0;
         // a multi-channel unit's missing last channels (as unsigned, so that a
         // sum past 2^31 - 1 is past the last as well)
-        const uint32_t c = (uint32_t)item.chan + (uint32_t)sgm.chan_off + (uint32_t)ci;
-        if (c >= (uint32_t)pb.n_chan) continue;
+        const int c = (int)((uint32_t)item.chan + (uint32_t)sgm.chan_off + (uint32_t)ci);
+        if ((uint32_t)c >= (uint32_t)pb.n_chan) continue;
         const int i0 = i_tile - ci * rpc;
         if (i0 >= pb.n_in) continue;
         int64_t *cacc = pb.acc + (long long)c * pb.n_pairs * 2;
